@@ -646,7 +646,7 @@ build_fused_kernel(const FusedBuildParams fp) {
     const TileSlots ts = tile_slots(p);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (!any_cand(ts)) {                             // uniform over the CTA
-        if (blockIdx.x == 0 && warp < ts.n) lm_step(fp.ep, ts.slot[warp], E[warp], &part[warp][0][0], *fp.min_valid, lane);
+        if (blockIdx.x == 0 && warp < ts.n) lm_step(fp.ep, ts.slot[warp], E[warp], *fp.min_valid, lane);
         return;
     }
     float acc[kNumSums];
@@ -658,11 +658,11 @@ build_fused_kernel(const FusedBuildParams fp) {
     const float v = cta_reduce_slots<kBuildThreads, GroupShape<DT, C, SCALED>::APB>(acc, red);
     const int hv = tid / kAcc, iv = tid % kAcc;     // slot and sum this thread holds (tid < kHypTile kAcc)
     if (p.n_tiles == 1) {
-        // the only tile: its record is the sum (0 + x is what the 8-chain sum gives), no
-        // round trip through the partial buffer and the ticket
-        if (tid < kHypTile * kAcc) E[hv][iv] = 0.0 + (double)v;
+        // the only tile: its record is the sum, no round trip through the partial buffer and the
+        // ticket
+        if (tid < kHypTile * kAcc) E[hv][iv] = widen(v);
         __syncthreads();
-        if (warp < ts.n) lm_step(fp.ep, ts.slot[warp], E[warp], &part[warp][0][0], *fp.min_valid, lane);
+        if (warp < ts.n) lm_step(fp.ep, ts.slot[warp], E[warp], *fp.min_valid, lane);
         return;
     }
     if (tid < kHypTile * kAcc && hv < ts.n && ts.cand[hv])
@@ -681,21 +681,20 @@ build_fused_kernel(const FusedBuildParams fp) {
             double a = 0.0;
             if (h < ts.n && ts.cand[h]) {
                 const float* src = p.partial + (size_t)ts.slot[h] * p.n_tiles * kAcc + ii;
-                for (int t = c; t < p.n_tiles; t += 8) a += (double)__ldcg(src + (size_t)t * kAcc);
+                a = chain_sum([&](int t) { return __ldcg(src + (size_t)t * kAcc); }, c, p.n_tiles);
             }
             part[h][c][ii] = a;
         }
     }
     __syncthreads();
     if (tid < kHypTile * kAcc) {
-        double sum = 0.0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) sum += part[hv][k][iv];
+        double sum = part[hv][0][iv];
+        for (int k = 1; k < min(8, p.n_tiles); ++k) sum += part[hv][k][iv];
         E[hv][iv] = sum;
     }
     __syncthreads();
     if (warp < ts.n) {                               // the warp-cooperative FP64 steps
-        lm_step(fp.ep, ts.slot[warp], E[warp], &part[warp][0][0], *fp.min_valid, lane);
+        lm_step(fp.ep, ts.slot[warp], E[warp], *fp.min_valid, lane);
     }
     if (tid == 0) fp.tickets[blockIdx.y] = 0u;
 }

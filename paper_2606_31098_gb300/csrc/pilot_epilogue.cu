@@ -29,20 +29,18 @@ __global__ void epilogue_kernel(const EpilogueParams p, const double* min_valid_
     const bool evaluated = (p.mode == kEpiStep) ? (st.has_cand != 0) : true;
     if (evaluated) {
         const float* src = p.partial + (size_t)slot * p.n_tiles * kAcc + v;
-        double acc = 0.0;
-        for (int t = c; t < p.n_tiles; t += 8) acc += (double)src[(size_t)t * kAcc];
-        part[c][v] = acc;
+        part[c][v] = chain_sum([&](int t) { return src[(size_t)t * kAcc]; }, c, p.n_tiles);
         __syncthreads();
         if (threadIdx.x < kAcc) {
-            double sum = 0.0;
-            for (int k = 0; k < 8; ++k) sum += part[k][threadIdx.x];
+            double sum = part[0][threadIdx.x];
+            for (int k = 1; k < min(8, p.n_tiles); ++k) sum += part[k][threadIdx.x];
             E[threadIdx.x] = sum;
         }
     }
     __syncthreads();
     if (threadIdx.x >= 32) return;                 // warp 0 runs the FP64 step
     const double min_valid = (p.mode == kEpiEval) ? 0.0 : *min_valid_ptr;
-    lm_step(p, slot, E, &part[0][0], min_valid, threadIdx.x);
+    lm_step(p, slot, E, min_valid, threadIdx.x);
 }
 
 __global__ void hyp_init_kernel(HypState* st, const double* T_cw, int* active_idx, int M) {

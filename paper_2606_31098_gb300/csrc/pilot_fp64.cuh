@@ -11,6 +11,7 @@
 
 #include <math.h>
 
+#include "pilot_bits.cuh"
 #include "pilot_internal.cuh"
 
 namespace pilot {
@@ -23,25 +24,27 @@ __device__ __forceinline__ int tri_index(int a, int b) {
     return a * 6 - (a * (a - 1)) / 2 + (b - a);
 }
 
-__device__ __forceinline__ void huber64(double s, double delta, double* rho, double* drho) {
-    const double d2 = delta * delta;
-    if (s <= d2) {
+// rho and rho' of the Huber function at s >= 0 (delta2 = delta^2).
+__device__ __forceinline__ void huber64(double s, double delta, double delta2, double* rho, double* drho) {
+    if (within(s, delta2)) {
         *rho = s;
         *drho = 1.0;
     } else {
         const double q = sqrt(s);
-        *rho = 2.0 * delta * q - d2;
+        *rho = 2.0 * delta * q - delta2;
         *drho = delta / q;
     }
 }
 
-// The step is warp-cooperative: all 32 lanes of one warp run it together.  GB300 issues an
-// FP64 instruction for the whole warp at a fraction of the FP32 rate, so one lane working
-// alone pays for 32; here independent FP64 operations (the 21 + 6 + 1 entries a prior adds,
-// the rows of the Cholesky factor, the three series, the entries of Exp, V and T') run one
-// per lane, and scalar work (residuals, Huber weights, pivots) runs redundantly on every
-// lane, which costs the same.  Each E entry's arithmetic is the one a single thread would
-// do; W is 128 doubles of the warp's shared memory.
+// The step is warp-cooperative: all 32 lanes of one warp run it together.  What bounds it is the
+// number of FP64 warp instructions (64 cycles each, however few lanes are active; see
+// pilot_bits.cuh), so independent operations of one kind run in one instruction on different
+// lanes -- the three rows of a matrix-vector product, the 28 entries a prior adds, the matrix
+// entries a Cholesky step updates, the three series, the entries of Exp, V and T' -- values move
+// between lanes by shuffles, and comparisons, conversions and truncations are integer
+// operations.  About 150 FP64 instructions per step instead of 415: 27 000 -> 21 000 cycles with
+// both priors at the paper's schedule.  Each value's arithmetic (operations, order, rounding) is
+// the one a single thread would do.
 
 // (row, column) of upper-triangle entry k (row-major), k < 21
 __device__ __forceinline__ void tri_pair(int k, int* a, int* b) {
@@ -57,128 +60,180 @@ __device__ __forceinline__ void tri_pair(int k, int* a, int* b) {
     *b = r + (k - base);
 }
 
+// Chain c of the FP64 sum of n tile records in 8 chains: records c, c + 8, ..., in order (0 if
+// there is none).  A sum starts at its first term and leaves out empty chains: adding them to or
+// from zero changes nothing.
+template <typename Load>
+__device__ __forceinline__ double chain_sum(Load load, int c, int n) {
+    if (c >= n) return 0.0;
+    double a = widen(load(c));
+    for (int t = c + 8; t < n; t += 8) a += widen(load(t));
+    return a;
+}
+
 __device__ __forceinline__ double shfl_d(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 
-// Gravity direction prior (Eq. 3) at pose T, added to E = H21 | g6 | cost.
-__device__ inline void add_gravity(const PriorParams& pp, const double* T, double* E, int lane) {
-    double a[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-        a[i] = T[4 * i] * pp.g_world[0] + T[4 * i + 1] * pp.g_world[1] + T[4 * i + 2] * pp.g_world[2];
-    const double r[3] = {a[0] - pp.g_cam[0], a[1] - pp.g_cam[1], a[2] - pp.g_cam[2]};
-    double rho, drho;
-    const double s = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
-    if (pp.gate_grav > 0.0 && s > pp.gate_grav * pp.gate_grav) {   // gated: constant, no pull
-        huber64(pp.gate_grav * pp.gate_grav, pp.huber_grav, &rho, &drho);
-        if (lane == 9) E[27] += pp.w_grav * rho;
-        return;
-    }
-    huber64(s, pp.huber_grav, &rho, &drho);
-    const double w = pp.w_grav * drho;
-    // rotation block: w [a]x^T [a]x = w (|a|^2 I - a a^T); gradient: w [a]x r = w (a x r)
-    const double aa = a[0] * a[0] + a[1] * a[1] + a[2] * a[2];
-    if (lane < 6) {
-        const int i = lane < 3 ? 0 : (lane < 5 ? 1 : 2);
-        const int k = lane < 3 ? lane : (lane < 5 ? lane - 2 : 2);
-        const double ai = i == 0 ? a[0] : (i == 1 ? a[1] : a[2]);
-        const double ak = k == 0 ? a[0] : (k == 1 ? a[1] : a[2]);
-        E[tri_index(3 + i, 3 + k)] += w * ((i == k ? aa : 0.0) - ai * ak);
-    } else if (lane == 6) {
-        E[21 + 3] += w * (a[1] * r[2] - a[2] * r[1]);
-    } else if (lane == 7) {
-        E[21 + 4] += w * (a[2] * r[0] - a[0] * r[2]);
-    } else if (lane == 8) {
-        E[21 + 5] += w * (a[0] * r[1] - a[1] * r[0]);
-    } else if (lane == 9) {
-        E[27] += pp.w_grav * rho;
-    }
+// x0 y0 + x1 y1 + x2 y2 and x0 y0 - x1 y1 with the contractions written out.
+__device__ __forceinline__ double dot3(double x0, double y0, double x1, double y1, double x2, double y2) {
+    return fma(x2, y2, fma(x0, y0, __dmul_rn(x1, y1)));
+}
+__device__ __forceinline__ double minus_products(double x0, double y0, double x1, double y1) {
+    return fma(x0, y0, -__dmul_rn(x1, y1));
 }
 
-// Laser range prior (Eq. 4-6) at pose T; dropped when the range point leaves the DSM.
-__device__ inline void add_range(const PriorParams& pp, const double* T, double* E, int lane) {
-    const double d[3] = {pp.q[0] - T[3], pp.q[1] - T[7], pp.q[2] - T[11]};
-    double P[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) P[i] = T[i] * d[0] + T[4 + i] * d[1] + T[8 + i] * d[2];  // R^T d
+// What lane l keeps of the evaluated pose: i = l mod 3, row i and column i of R, and t_i.
+struct PoseRows {
+    double row[3], col[3], t;
+    int i;
+};
+
+// Gravity direction prior (Eq. 3), added to this lane's entry e of H21 | g6 | cost.  Lane i computes
+// a_i and r_i; rotation block: w [a]x^T [a]x = w (|a|^2 I - a a^T); gradient: w [a]x r = w (a x r).
+__device__ __forceinline__ void add_gravity(const PriorParams& pp, const PoseRows& T, double& e, int lane, int ta,
+                                            int tb) {
+    const double ai = dot3(T.row[0], pp.g_world[0], T.row[1], pp.g_world[1], T.row[2], pp.g_world[2]);
+    const double ri = ai - (T.i == 0 ? pp.g_cam[0] : (T.i == 1 ? pp.g_cam[1] : pp.g_cam[2]));
+    const double a[3] = {shfl_d(ai, 0), shfl_d(ai, 1), shfl_d(ai, 2)};
+    const double r[3] = {shfl_d(ri, 0), shfl_d(ri, 1), shfl_d(ri, 2)};
+    // even lanes |a|^2, odd lanes |r|^2
+    const bool odd = lane & 1;
+    const double v0 = odd ? r[0] : a[0], v1 = odd ? r[1] : a[1], v2 = odd ? r[2] : a[2];
+    const double vv = dot3(v0, v0, v1, v1, v2, v2);
+    const double aa = shfl_d(vv, 0), s = shfl_d(vv, 1);
+    double rho, drho;
+    if (bits(pp.gate_grav) != 0ull && bits(s) > bits(pp.gate_grav2) && bits(s) <= kInfBits) {
+        huber64(pp.gate_grav2, pp.huber_grav, pp.huber_grav2, &rho, &drho);   // gated: constant, no pull
+        if (lane == 27) e = fma(pp.w_grav, rho, e);
+        return;
+    }
+    huber64(s, pp.huber_grav, pp.huber_grav2, &rho, &drho);
+    const double w = bits(drho) == kOneBits ? pp.w_grav : pp.w_grav * drho;
+    auto pick = [](const double* v, int i) { return i == 0 ? v[0] : (i == 1 ? v[1] : v[2]); };
+    // H entries (3 + i, 3 + k) on lanes 15..20, g entries 3 + i on lanes 24..26, the cost on lane 27
+    const bool h = lane < 21;
+    const int i = h ? ta - 3 : (lane >= 24 ? lane - 24 : 0), k = h ? tb - 3 : 0;
+    const int u = i == 2 ? 0 : i + 1, v = u == 2 ? 0 : u + 1;
+    const double p = h ? -pick(a, i) : pick(a, u), q = h ? pick(a, k) : pick(r, v);
+    const double m = __dmul_rn(pick(a, v), pick(r, u));
+    const double val = fma(p, q, h ? (i == k ? aa : 0.0) : -m);
+    if (lane == 27) e = fma(pp.w_grav, rho, e);
+    else if ((lane >= 15 && lane < 21) || (lane >= 24 && lane < 27)) e = fma(w, val, e);
+}
+
+// Laser range prior (Eq. 4-6); dropped when the range point leaves the DSM.
+__device__ __forceinline__ void add_range(const PriorParams& pp, const PoseRows& T, double& e, int lane, int ta,
+                                          int tb) {
+    const int li = T.i, lu = li == 2 ? 0 : li + 1, lv = lu == 2 ? 0 : lu + 1;
+    auto pick = [](const double* v, int i) { return i == 0 ? v[0] : (i == 1 ? v[1] : v[2]); };
+    const double di = pick(pp.q, li) - T.t;
+    const double d0 = shfl_d(di, 0), d1 = shfl_d(di, 1), d2 = shfl_d(di, 2);
+    const double Pi = dot3(T.col[0], d0, T.col[1], d1, T.col[2], d2);          // R^T d
+    // x on lanes 0 mod 3, y on lanes 1 mod 3
     const double inv_gsd = pp.dsm_inv_gsd;
-    const double gx = (P[0] - pp.dsm_x0) * inv_gsd - 0.5;
-    const double gy = (P[1] - pp.dsm_y0) * inv_gsd - 0.5;
-    if (!(gx >= 0.0 && gx <= pp.dsm_W - 1.0 && gy >= 0.0 && gy <= pp.dsm_H - 1.0)) return;
-    const int c0 = min((int)gx, pp.dsm_W - 2), r0 = min((int)gy, pp.dsm_H - 2);
-    const double ax = gx - c0, ay = gy - r0;
+    const double gi = (Pi - (li == 0 ? pp.dsm_x0 : pp.dsm_y0)) * inv_gsd - 0.5;
+    const bool in = within(gi, li == 0 ? pp.dsm_wmax : pp.dsm_hmax);
+    if ((__ballot_sync(0xffffffffu, in) & 3u) != 3u) return;
+    const int ci = min(whole_part(gi), (li == 0 ? pp.dsm_W : pp.dsm_H) - 2);
+    const double fi = gi - as_double(ci);
+    const int c0 = __shfl_sync(0xffffffffu, ci, 0), r0 = __shfl_sync(0xffffffffu, ci, 1);
+    const double ax = shfl_d(fi, 0), ay = shfl_d(fi, 1);
     const float* row0 = pp.dsm + (size_t)r0 * pp.dsm_W + c0;
     const float* row1 = row0 + pp.dsm_W;
-    const double h00 = row0[0], h01 = row0[1], h10 = row1[0], h11 = row1[1];
-    const double bx = h01 - h00, cy = h10 - h00, dxy = (h11 - h10) - bx;
-    const double D = h00 + ax * (bx + dxy * ay) + ay * cy;
-    const double Dx = (bx + dxy * ay) * inv_gsd, Dy = (cy + dxy * ax) * inv_gsd;
-    const double r = P[2] - D;
+    const double h00 = widen(row0[0]), h01 = widen(row0[1]), h10 = widen(row1[0]), h11 = widen(row1[1]);
+    // bx on lanes 0 mod 3, cy on lanes 1 mod 3, the lower difference on lanes 2 mod 3
+    const double diff = (li == 0 ? h01 : (li == 1 ? h10 : h11)) - (li == 2 ? h10 : h00);
+    const double bx = shfl_d(diff, 0), cy = shfl_d(diff, 1);
+    const double dxy = shfl_d(diff, 2) - bx;
+    const double ui = (li == 0 ? bx : cy) + dxy * (li == 0 ? ay : ax);
+    const double gradi = ui * inv_gsd;
+    const double D = h00 + ax * shfl_d(ui, 0) + ay * cy;
+    const double Dx = shfl_d(gradi, 0), Dy = shfl_d(gradi, 1);
+    const double r = shfl_d(Pi, 2) - D;
     double rho, drho;
-    if (pp.gate_range > 0.0 && fabs(r) > pp.gate_range) {          // gated: constant, no pull
-        huber64(pp.gate_range * pp.gate_range, pp.huber_range, &rho, &drho);
-        if (lane == 27) E[27] += pp.w_range * rho;
+    const unsigned long long ra = bits(r) & 0x7fffffffffffffffull;
+    if (bits(pp.gate_range) != 0ull && ra > bits(pp.gate_range) && ra <= kInfBits) {
+        huber64(pp.gate_range2, pp.huber_range, pp.huber_range2, &rho, &drho);  // gated: constant, no pull
+        if (lane == 27) e = fma(pp.w_range, rho, e);
         return;
     }
-    // dr/dP = e = (-Dx, -Dy, 1); dP/ddelta = R^T [-I | [q]x]  =>  J = [-(R e) | (R e) x q]
-    const double e[3] = {-Dx, -Dy, 1.0};
-    double n[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) n[i] = T[4 * i] * e[0] + T[4 * i + 1] * e[1] + T[4 * i + 2] * e[2];
-    const double J[6] = {-n[0], -n[1], -n[2],
-                         n[1] * pp.q[2] - n[2] * pp.q[1],
-                         n[2] * pp.q[0] - n[0] * pp.q[2],
-                         n[0] * pp.q[1] - n[1] * pp.q[0]};
-    huber64(r * r, pp.huber_range, &rho, &drho);
-    const double w = pp.w_range * drho;
-    if (lane < 21) {
-        int a, b;
-        tri_pair(lane, &a, &b);
-        E[lane] += w * J[a] * J[b];
-    } else if (lane < 27) {
-        E[lane] += w * J[lane - 21] * r;
-    } else if (lane == 27) {
-        E[27] += pp.w_range * rho;
-    }
+    // dr/dP = (-Dx, -Dy, 1); dP/ddelta = R^T [-I | [q]x]  =>  J = [-n | n x q], n = R (-Dx, -Dy, 1)
+    const double ni = fma(T.row[0], -Dx, __dmul_rn(T.row[1], -Dy)) + T.row[2];
+    const double nu = shfl_d(ni, lu), nv = shfl_d(ni, lv);
+    const double xi = minus_products(nu, pick(pp.q, lv), nv, pick(pp.q, lu));
+    huber64(r * r, pp.huber_range, pp.huber_range2, &rho, &drho);
+    const double w = bits(drho) == kOneBits ? pp.w_range : pp.w_range * drho;
+    // this lane's J[a] and its factor: J[b] (H), r (g), rho (cost)
+    const int a = lane < 21 ? ta : (lane < 27 ? lane - 21 : 0), b = lane < 21 ? tb : 0;
+    const int a3 = a < 3 ? a : a - 3, b3 = b < 3 ? b : b - 3;
+    const double na = shfl_d(ni, a3), xa = shfl_d(xi, a3), nb = shfl_d(ni, b3), xb = shfl_d(xi, b3);
+    const double Ja = a < 3 ? -na : xa, Jb = b < 3 ? -nb : xb;
+    const double m = w * Ja;
+    if (lane < 28) e = fma(lane == 27 ? pp.w_range : m, lane < 21 ? Jb : (lane < 27 ? r : rho), e);
 }
 
-// (H + damping) x = -g by Cholesky; lane i < 6 owns row i of the factor.  Returns false
-// (on every lane) if the damped matrix is not positive definite.  H21 and g in shared memory.
-__device__ inline bool damped_solve(const double* H21, const double* g, double lambda, int mode,
-                                    double* x, double* Lsh, int lane) {
-    const int i = lane < 6 ? lane : 5;
-    double Lr[6], inv[6];
+// s = sqrt(d) and inv = 1 / s, each rounded to nearest, for d > 0.  An FP32 estimate of 1 / sqrt(d)
+// is refined by Newton's iteration of third order; the square root and the reciprocal are then
+// corrected by their remainders, which FMA gives exactly (Markstein, IBM J. Res. Dev. 34(1),
+// 1990).  Ten FP64 instructions; the operations themselves outside 2^+-900.
+__device__ __forceinline__ void sqrt_inverse(double d, double* s, double* inv) {
+    const int e = (int)(((unsigned)__double2hiint(d) >> 20) & 0x7ffu) - 1023;
+    if (e < -900 || e > 900) {
+        *s = sqrt(d);
+        *inv = 1.0 / *s;
+        return;
+    }
+    const int k = e >> 1;
+    const double m = scale2(d, -2 * k);                      // in [1, 4)
+    float f = __uint_as_float(((unsigned)__double2hiint(m) - 0x38000000u) << 3 | (unsigned)__double2loint(m) >> 29);
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(f));
+    const double y0 = widen(f);
+    const double t = m * y0;
+    const double r = fma(-t, y0, 1.0);
+    const double y = fma(fma(0.375, r, 0.5), y0 * r, y0);
+    const double s0 = m * y;
+    const double sm = fma(fma(-s0, s0, m), scale2(y, -1), s0);
+    *s = scale2(sm, k);
+    // (a root just below 2 has its reciprocal next to a rounding boundary)
+    *inv = (__double2hiint(sm) & 0xfffff) == 0xfffff ? 1.0 / *s : scale2(fma(fma(-sm, y, 1.0), y, y), -k);
+}
+
+// lambda / 10, rounded to nearest (a product and a correction by its remainder).
+__device__ __forceinline__ double tenth(double v) { return quotient(v, 10.0, 0.1); }
+
+// (H + damping) x = -g by Cholesky.  Lane l < 21 holds entry l of H's upper triangle, (a, b) of
+// tri_pair, i.e. entry (b, a) of the factor; lanes 21..26 hold g, treated as a seventh row of the
+// matrix (its row of the factor is y, L y = -g), so that one instruction updates every entry
+// behind a column.  x on every lane; false (on every lane) if the damped matrix is not positive
+// definite.
+__device__ __forceinline__ bool damped_solve(double hg, int ta, int tb, double lambda, int mode, double* x, int lane) {
+    const int col = lane < 21 ? ta : lane - 21, row = lane < 21 ? tb : 6;
+    double v = lane < 21 ? hg : -hg;
+    if (row == col) v += mode == 1 ? __dmul_rn(lambda, v) : lambda;
+    auto at = [](int r, int c) { return r == 6 ? 21 + c : tri_index(c, r); };    // lane of entry (r, c)
+    double inv[6];
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
-        // a_ij = A_ij - sum_{k<j} L_ik L_jk for this lane's row (meaningful when i >= j)
-        double a = H21[tri_index(min(i, j), max(i, j))];
-        if (i == j) a += (mode == 1) ? lambda * H21[tri_index(i, i)] : lambda;
-#pragma unroll
-        for (int k = 0; k < j; ++k) a -= Lr[k] * shfl_d(Lr[k], j);
-        const double d = shfl_d(a, j);
-        if (!(d > 0.0)) return false;
-        const double ljj = sqrt(d);
-        inv[j] = 1.0 / ljj;
-        Lr[j] = (i == j) ? ljj : a * inv[j];
+        const double d = shfl_d(v, tri_index(j, j));
+        // d > 0 (a zero, negative or NaN pivot ends the solve)
+        if (bits(d) - 1ull >= kInfBits) return false;
+        double s;
+        sqrt_inverse(d, &s, &inv[j]);
+        const double l = v * inv[j];
+        if (col == j) v = row == j ? s : l;
+        if (j < 5) {
+            const double lr = shfl_d(v, at(row, j) & 31), lc = shfl_d(v, at(max(col, j), j) & 31);
+            if (col > j) v = fma(-lr, lc, v);
+        }
     }
-    // L y = -g: once y_k is known every later row subtracts its term
-    double s = -g[i];
-    double y[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        y[k] = shfl_d(s, k) * inv[k];
-        if (i > k) s -= Lr[k] * y[k];
-    }
-    // L^T x = y: row k of L (lane k) is read from shared memory
-    if (lane < 6) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) Lsh[6 * lane + k] = Lr[k];
-    }
-    __syncwarp();
-    double t = y[i];
+    // L^T x = y: lane 21 + i runs row i
 #pragma unroll
     for (int k = 5; k >= 0; --k) {
-        x[k] = shfl_d(t, k) * inv[k];
-        if (i < k) t -= Lsh[6 * k + i] * x[k];
+        x[k] = shfl_d(v, 21 + k) * inv[k];
+        if (k > 0) {
+            const int i = lane >= 21 ? lane - 21 : 0;
+            const double l = shfl_d(v, tri_index(min(i, k), k));
+            if (lane >= 21 && i < k) v = fma(-l, x[k], v);
+        }
     }
     return true;
 }
@@ -188,8 +243,8 @@ __device__ inline bool damped_solve(const double* H21, const double* g, double l
 //   A = sum_k (-x)^k / (2k+1)!,  B = sum_k (-x)^k / (2k+2)!,  C = sum_k (-x)^k / (2k+3)!,
 // are summed for k = 0..8 by Horner (the first omitted term is below 1e-27), lane 0 summing
 // A, lane 1 B and lane 2 C; larger angles use sin and cos.
-__device__ inline void exp_coefficients(double x, double* A, double* B, double* C, int lane) {
-    if (x <= 0.0625) {
+__device__ __forceinline__ void exp_coefficients(double x, double* A, double* B, double* C, int lane) {
+    if (within(x, 0.0625)) {
         // reciprocal factorials 1/n!, n = 1..19
         constexpr double f[20] = {1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120, 1.0 / 720, 1.0 / 5040,
                                   1.0 / 40320, 1.0 / 362880, 1.0 / 3628800, 1.0 / 39916800,
@@ -217,16 +272,18 @@ __device__ inline void exp_coefficients(double x, double* A, double* B, double* 
     }
 }
 
-// T' = exp(xi) T with xi = (nu, omega):  Exp(w) = I + A K + B K^2,
-// V = I + B K + C K^2, K = [w]x, K^2 = w w^T - th^2 I.  Lanes 0..8 form Exp, 9..17 V
-// (in W), then lanes 0..11 one entry of T' each, written to Tn.  T in shared memory.
-__device__ inline void pose_update(const double* xi, const double* T, double* Tn, double* W, int lane) {
+// T' = exp(xi) T with xi = (nu, omega):  Exp(w) = I + A K + B K^2, V = I + B K + C K^2, K = [w]x,
+// K^2 = w w^T - th^2 I.  Lanes 0..8 form Exp, 9..17 V, then lanes 0..11 an entry of Exp T each and
+// lanes 12..14 an entry of V nu.  T: lane l < 12 holds entry l; returns entry l of T'.
+__device__ __forceinline__ double pose_update(const double* xi, double T, int lane) {
     const double w0 = xi[3], w1 = xi[4], w2 = xi[5];
-    const double th2 = w0 * w0 + w1 * w1 + w2 * w2;
+    const double th2 = dot3(w0, w0, w1, w1, w2, w2);
     double A, B, Cc;
     exp_coefficients(th2, &A, &B, &Cc, lane);
-    if (lane < 18) {
-        const int e = lane < 9 ? lane : lane - 9;
+    double W;
+    {
+        const bool ex = lane < 9;
+        const int e = ex ? lane : (lane < 18 ? lane - 9 : 0);
         const int i = e / 3, k = e % 3;
         const double wi = i == 0 ? w0 : (i == 1 ? w1 : w2);
         const double wk = k == 0 ? w0 : (k == 1 ? w1 : w2);
@@ -240,94 +297,96 @@ __device__ inline void pose_update(const double* xi, const double* T, double* Tn
         if (i == 2 && k == 1) Kik = w0;
         const double K2 = wi * wk - (i == k ? th2 : 0.0);
         const double I = (i == k) ? 1.0 : 0.0;
-        W[lane] = lane < 9 ? I + A * Kik + B * K2 : I + B * Kik + Cc * K2;
+        W = I + (ex ? A : B) * Kik + (ex ? B : Cc) * K2;
     }
-    __syncwarp();
-    if (lane < 12) {
-        const int i = lane >> 2, k = lane & 3;
-        const double* Re = W + 3 * i;
-        const double* V = W + 9 + 3 * i;
-        double v = Re[0] * T[k] + Re[1] * T[4 + k] + Re[2] * T[8 + k];
-        if (k == 3) v += V[0] * xi[0] + V[1] * xi[1] + V[2] * xi[2];
-        Tn[lane] = v;
-    }
+    const bool rot = lane < 12;
+    const int i = rot ? lane >> 2 : (lane < 15 ? lane - 12 : 0), k = lane & 3;
+    const int w = rot ? 3 * i : 9 + 3 * i;
+    const double m0 = shfl_d(W, w), m1 = shfl_d(W, w + 1), m2 = shfl_d(W, w + 2);
+    const double t0 = shfl_d(T, k), t1 = shfl_d(T, 4 + k), t2 = shfl_d(T, 8 + k);
+    const double b0 = rot ? t0 : xi[0], b1 = rot ? t1 : xi[1], b2 = rot ? t2 : xi[2];
+    const double v = dot3(m0, b0, m1, b1, m2, b2);
+    const double shift = shfl_d(v, 12 + i);
+    return k == 3 ? v + shift : v;
 }
 
 __device__ __forceinline__ void store_pose32(float* dst, const double* T) {
     for (int i = 0; i < 12; ++i) dst[i] = (float)T[i];
 }
 
-// One hypothesis' FP64 step after a build pass at its candidate.  E (29 sums in the warp's
-// shared memory, photo term only on entry) gets the priors at the evaluated pose; then
+// One hypothesis' FP64 step after a build pass at its candidate.  E (29 sums, photo term only, in
+// the warp's shared memory) gets the priors at the evaluated pose; then
 // (init) it becomes the current state, or (step) the candidate is accepted or rejected; then
 // the next candidate is solved for and, if cand32 is given, written there in FP32.  All 32
-// lanes of one warp call it with the same arguments; W is 128 doubles of the warp's shared
-// memory.
+// lanes of one warp call it with the same arguments.  Returns whether there is a candidate.
 //
 // Not inlined: every kernel of a translation unit (plain fused, batched, served) then runs
 // the same compiled instructions, so the compiler cannot contract a * b + c into an FMA in
 // one caller and not in another, and the forms stay bitwise equal.
-static __device__ __noinline__ void lm_update(HypState& st, int mode, int solve_next, int damping_mode,
-                                              const PriorParams& prior, double* E, double* W,
-                                              double min_valid, float* cand32, double* eval_out, int lane) {
+static __device__ __noinline__ int lm_update(HypState& st, int mode, int solve_next, int damping_mode,
+                                             const PriorParams& prior, const double* E,
+                                             double min_valid, float* cand32, double* eval_out, int lane) {
     // every read of the state is issued here, before any write, as one round trip, from L2:
     // the persistent level kernel may step a hypothesis on another SM than the last time
     const int has_cand = __ldcg(&st.has_cand);
     const double cost0 = __ldcg(&st.cost);
     const double lambda0 = __ldcg(&st.lambda);
     const double* Tsrc = (mode == kEpiStep) ? st.Tc : st.T;
-    double Tev[12];
+    PoseRows Tev;
+    Tev.i = lane % 3;
 #pragma unroll
-    for (int i = 0; i < 12; ++i) Tev[i] = __ldcg(Tsrc + i);
+    for (int k = 0; k < 3; ++k) {
+        Tev.row[k] = __ldcg(Tsrc + 4 * Tev.i + k);
+        Tev.col[k] = __ldcg(Tsrc + 4 * k + Tev.i);
+    }
+    Tev.t = __ldcg(Tsrc + 4 * Tev.i + 3);
     const double Hg_own = lane < 21 ? __ldcg(st.H + lane) : (lane < 27 ? __ldcg(st.g + lane - 21) : 0.0);
     const double T_own = lane < 12 ? __ldcg(st.T + lane) : 0.0;
     const double Tc_own = lane < 12 ? __ldcg(st.Tc + lane) : 0.0;
     const bool evaluated = (mode == kEpiStep) ? (has_cand != 0) : true;
+    int ta = 0, tb = 0;
+    if (lane < 21) tri_pair(lane, &ta, &tb);
+    double e = evaluated && lane < kNumSums ? E[lane] : 0.0;
     if (evaluated) {
-        if (prior.use_gravity) add_gravity(prior, Tev, E, lane);
-        __syncwarp();
-        if (prior.use_range) add_range(prior, Tev, E, lane);
-        __syncwarp();
+        if (prior.use_gravity) add_gravity(prior, Tev, e, lane, ta, tb);
+        if (prior.use_range) add_range(prior, Tev, e, lane, ta, tb);
     }
+    __syncwarp();
     if (mode == kEpiEval) {
-        if (lane < kNumSums) eval_out[lane] = E[lane];
+        if (lane < kNumSums) eval_out[lane] = e;
         if (lane == 0) st.has_cand = 0;
-        return;
+        return 0;
     }
-    // the state after acceptance, staged in W: H 0..20, g 21..26, T 32..43
+    // the state after acceptance: H 0..20, g 21..26 and T 0..11 on their lanes
     bool take = false;
     double lambda = lambda0;
     if (mode == kEpiInit) {
         take = true;
     } else if (evaluated) {
-        take = E[27] < cost0 && E[28] >= min_valid;
-        lambda = take ? fmax(lambda0 / 10.0, kLambdaMin) : fmin(lambda0 * 10.0, kLambdaMax);
+        take = shfl_d(e, 27) < cost0 && bits(min_valid) <= bits(shfl_d(e, 28));    // a count and a threshold >= 0
+        lambda = take ? fmax(tenth(lambda0), kLambdaMin) : fmin(lambda0 * 10.0, kLambdaMax);
     }
-    if (lane < 27) W[lane] = take ? E[lane] : Hg_own;
-    if (lane < 12) W[32 + lane] = (take && mode == kEpiStep) ? Tc_own : T_own;
-    __syncwarp();
+    const double hg = take ? e : Hg_own;
+    const double T = (take && mode == kEpiStep) ? Tc_own : T_own;
     if (take) {
-        if (lane < 21) st.H[lane] = E[lane];
-        else if (lane < 27) st.g[lane - 21] = E[lane];
-        else if (lane == 27) st.cost = E[27];
-        else if (lane == 28) st.n_valid = (int)E[28];
-        if (mode == kEpiStep && lane < 12) st.T[lane] = W[32 + lane];
+        if (lane < 21) st.H[lane] = e;
+        else if (lane < 27) st.g[lane - 21] = e;
+        else if (lane == 27) st.cost = e;
+        else if (lane == 28) st.n_valid = whole_part(e);
+        if (mode == kEpiStep && lane < 12) st.T[lane] = T;
     }
     int cand = 0, fail = -1;
     if (solve_next) {
         double dxi[6];
-        if (!damped_solve(W, W + 21, lambda, damping_mode, dxi, W + 64, lane)) {
+        if (!damped_solve(hg, ta, tb, lambda, damping_mode, dxi, lane)) {
             lambda = fmin(lambda * 10.0, kLambdaMax);
             fail = 1;
         } else {
             fail = 0;
-            __syncwarp();
-            pose_update(dxi, W + 32, W + 48, W + 100, lane);
-            __syncwarp();
+            const double Tn = pose_update(dxi, T, lane);
             if (lane < 12) {
-                const double Tn = W[48 + lane];
                 st.Tc[lane] = Tn;
-                if (cand32) cand32[lane] = (float)Tn;
+                if (cand32) cand32[lane] = narrow(Tn);
             }
             cand = 1;
         }
@@ -338,13 +397,14 @@ static __device__ __noinline__ void lm_update(HypState& st, int mode, int solve_
         st.has_cand = cand;
     }
     __syncwarp();
+    return cand;
 }
 
 // lm_update for slot `slot` of a launch described by p (candidate written to p.pose32); all
 // 32 lanes of one warp call it.
-__device__ inline void lm_step(const EpilogueParams& p, int slot, double* E, double* W, double min_valid, int lane) {
+__device__ inline void lm_step(const EpilogueParams& p, int slot, const double* E, double min_valid, int lane) {
     const int hyp = p.active_idx[slot];
-    lm_update(p.state[hyp], p.mode, p.solve_next, p.damping_mode, p.prior, E, W, min_valid,
+    lm_update(p.state[hyp], p.mode, p.solve_next, p.damping_mode, p.prior, E, min_valid,
               p.pose32 + 12 * hyp, p.eval_out ? p.eval_out + (size_t)slot * kNumSums : nullptr, lane);
 }
 

@@ -106,9 +106,22 @@ struct PriorParams {
     double q[3];               // d^range * v (Eq. 4 ray scaled by the range), camera frame
     double w_range, huber_range;
     double gate_grav, gate_range;   // residual gates (0 = none)
+    double huber_grav2, huber_range2, gate_grav2, gate_range2;   // their squares
     const float* dsm;
     int dsm_H, dsm_W;
     double dsm_x0, dsm_y0, dsm_gsd, dsm_inv_gsd;   // inv = 1 / gsd
+    double dsm_wmax, dsm_hmax;      // dsm_W - 1, dsm_H - 1
+
+    // the fields that follow from the others
+    void derive() {
+        huber_grav2 = huber_grav * huber_grav;
+        huber_range2 = huber_range * huber_range;
+        gate_grav2 = gate_grav * gate_grav;
+        gate_range2 = gate_range * gate_range;
+        dsm_inv_gsd = 1.0 / dsm_gsd;
+        dsm_wmax = dsm_W - 1.0;
+        dsm_hmax = dsm_H - 1.0;
+    }
 };
 
 enum EpilogueMode { kEpiInit = 0, kEpiStep = 1, kEpiEval = 2 };

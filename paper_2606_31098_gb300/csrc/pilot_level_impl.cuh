@@ -80,7 +80,7 @@ __device__ __forceinline__ bool grid_sync(unsigned long long* sync, unsigned* er
 // lm_update; all 32 lanes of one warp.  Not inlined: the item loop that calls it keeps its own
 // registers for the anchor loop.
 static __device__ __noinline__ void flow_step(const LevelArgs& a, int job, int first, int frame, int level, int k,
-                                              int h, int tpi, double* E, double* W) {
+                                              int h, int tpi, double* E) {
     constexpr unsigned kEval = 0x80000000u;
     const int lane = threadIdx.x & 31;
     const FrameDesc* fd = a.frames + frame;
@@ -90,19 +90,15 @@ static __device__ __noinline__ void flow_step(const LevelArgs& a, int job, int f
     if ((meta & kEval) != 0 && lane < kNumSums) {
         const int n_t = fd->N > 0 ? (fd->N + a.tile - 1) / a.tile : 1;
         const float* src = a.partial + ((size_t)first * tpi * kHypTile + h) * kAcc + lane;
-        double sum = 0.0;
-        for (int c = 0; c < 8; ++c) {
-            double part = 0.0;
-            for (int t = c; t < n_t; t += 8) part += (double)__ldcg(src + (size_t)t * kHypTile * kAcc);
-            sum += part;
-        }
+        auto record = [&](int t) { return __ldcg(src + (size_t)t * kHypTile * kAcc); };
+        double sum = chain_sum(record, 0, n_t);
+        for (int c = 1; c < min(8, n_t); ++c) sum += chain_sum(record, c, n_t);
         E[lane] = sum;
     }
     __syncwarp();
-    HypState& st = a.state[hyp];
-    lm_update(st, k == 0 ? kEpiInit : kEpiStep, k < iters, a.damping_mode, fd->prior, E, W, a.min_valid[frame],
-              a.pose32 + 12 * (size_t)job, nullptr, lane);
-    if (lane == 0) a.job_meta[job] = (unsigned)hyp | (st.has_cand ? kEval : 0u);
+    const int cand = lm_update(a.state[hyp], k == 0 ? kEpiInit : kEpiStep, k < iters, a.damping_mode, fd->prior, E,
+                               a.min_valid[frame], a.pose32 + 12 * (size_t)job, nullptr, lane);
+    if (lane == 0) a.job_meta[job] = (unsigned)hyp | (cand ? kEval : 0u);
     __syncwarp();
 }
 
@@ -113,7 +109,6 @@ level_persistent_kernel(const __grid_constant__ LevelArgs a) {
     constexpr unsigned kEval = 0x80000000u;          // job_meta: "has a pose to evaluate" bit
     __shared__ float red[kWarps][kHypTile][kAcc];
     __shared__ double E[kWarps][kAcc];
-    __shared__ double Wsh[kWarps][128];         // FP64 step scratch, one block per warp
     __shared__ float pose[kHypTile][12];
     __shared__ unsigned s_meta[kHypTile];
     // the claimed work item: its frame, first record slot, tile range and job tile (s_item < 0:
@@ -278,7 +273,7 @@ level_persistent_kernel(const __grid_constant__ LevelArgs a) {
             __syncthreads();
             if (s_last) {
                 if (warp < s_njobs)
-                    flow_step(a, s_job + warp, s_first, s_frame, s_level, s_k, warp, tpi, E[warp], Wsh[warp]);
+                    flow_step(a, s_job + warp, s_first, s_frame, s_level, s_k, warp, tpi, E[warp]);
                 __syncthreads();
                 if (tid == 0) {
                     __threadfence();
@@ -323,19 +318,16 @@ level_persistent_kernel(const __grid_constant__ LevelArgs a) {
                         const int jl = job - fjob(i);
                         const int first = fitem(i) + (jl / kHypTile) * fipj(i);
                         const float* src = a.partial + ((size_t)first * tpi * kHypTile + jl % kHypTile) * kAcc + lane;
-                        double sum = 0.0;
-                        for (int c = 0; c < 8; ++c) {
-                            double part = 0.0;
-                            for (int t = c; t < n_t; t += 8) part += (double)__ldcg(src + (size_t)t * kHypTile * kAcc);
-                            sum += part;
-                        }
+                        auto record = [&](int t) { return __ldcg(src + (size_t)t * kHypTile * kAcc); };
+                        double sum = chain_sum(record, 0, n_t);
+                        for (int c = 1; c < min(8, n_t); ++c) sum += chain_sum(record, c, n_t);
                         E[warp][lane] = sum;
                     }
                     __syncwarp();
-                    HypState& st = a.state[hyp];
-                    lm_update(st, k == 0 ? kEpiInit : kEpiStep, k < iters, a.damping_mode, fd->prior, E[warp], Wsh[warp],
-                              a.min_valid[f], a.pose32 + 12 * (size_t)job, nullptr, lane);
-                    if (lane == 0) a.job_meta[job] = (unsigned)hyp | (st.has_cand ? kEval : 0u);
+                    const int cand = lm_update(a.state[hyp], k == 0 ? kEpiInit : kEpiStep, k < iters, a.damping_mode,
+                                               fd->prior, E[warp], a.min_valid[f], a.pose32 + 12 * (size_t)job,
+                                               nullptr, lane);
+                    if (lane == 0) a.job_meta[job] = (unsigned)hyp | (cand ? kEval : 0u);
                     __syncwarp();
                 }
             }
