@@ -33,6 +33,7 @@
 // deterministic and independent of the grid shape and of how hypotheses are grouped.
 #pragma once
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
@@ -48,70 +49,65 @@ template <> struct Storage<PILOT_BF16> { using T = uint16_t; static constexpr in
 template <> struct Storage<PILOT_F16> { using T = uint16_t; static constexpr int VEC = 16; };
 template <> struct Storage<PILOT_FP8E4M3> { using T = uint8_t; static constexpr int VEC = 16; };
 
-// Load W (4, 8 or 16) consecutive channels at p and widen them to FP32 (one load of W
-// elements: 4 to 16 bytes for the narrow types, 16 or 32 bytes for FP32).
+// W (4, 8 or 16) consecutive channels at p as they are stored (one load of W elements: 4 to 32
+// bytes).
+template <pilot_dtype DT, int W> struct RawVec {
+    static constexpr int NW = W * (int)sizeof(typename Storage<DT>::T) / 4;
+    uint32_t w[NW];
+};
+
+template <pilot_dtype DT, int W>
+__device__ __forceinline__ void load_raw(const typename Storage<DT>::T* p, RawVec<DT, W>& o) {
+    constexpr int NW = RawVec<DT, W>::NW;
+    static_assert(NW == 1 || NW == 2 || NW == 4 || NW == 8, "vector width");
+    if constexpr (NW == 8) {
+        // one 256-bit load (32-byte aligned: device feature pointers are validated for it)
+        asm("ld.global.nc.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=r"(o.w[0]), "=r"(o.w[1]), "=r"(o.w[2]), "=r"(o.w[3]), "=r"(o.w[4]), "=r"(o.w[5]), "=r"(o.w[6]),
+              "=r"(o.w[7])
+            : "l"(p));
+    } else if constexpr (NW == 4) {
+        asm("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];"
+            : "=r"(o.w[0]), "=r"(o.w[1]), "=r"(o.w[2]), "=r"(o.w[3]) : "l"(p));
+    } else if constexpr (NW == 2) {
+        asm("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(o.w[0]), "=r"(o.w[1]) : "l"(p));
+    } else {
+        asm("ld.global.nc.u32 %0, [%1];" : "=r"(o.w[0]) : "l"(p));
+    }
+}
+
+// Channels e and e + 1 (e even) widened to FP32.
+template <pilot_dtype DT, int W>
+__device__ __forceinline__ void raw_pair(const RawVec<DT, W>& v, int e, float& lo, float& hi) {
+    if constexpr (DT == PILOT_F32) {
+        lo = __uint_as_float(v.w[e]);
+        hi = __uint_as_float(v.w[e + 1]);
+    } else if constexpr (DT == PILOT_BF16) {
+        // bfloat16 is the upper half of an IEEE binary32: widening is a 16-bit shift
+        lo = __uint_as_float(v.w[e / 2] << 16);
+        hi = __uint_as_float(v.w[e / 2] & 0xffff0000u);
+    } else if constexpr (DT == PILOT_F16) {
+        __half2 h;
+        memcpy(&h, &v.w[e / 2], 4);
+        const float2 f = __half22float2(h);
+        lo = f.x;
+        hi = f.y;
+    } else {
+        const __half2_raw h =
+            __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)((v.w[e / 4] >> (8 * (e & 2))) & 0xffffu), __NV_E4M3);
+        const float2 f = __half22float2(__half2(h));
+        lo = f.x;
+        hi = f.y;
+    }
+}
+
+// Loaded and widened to FP32.
 template <pilot_dtype DT, int W>
 __device__ __forceinline__ void load_vec(const typename Storage<DT>::T* p, float* out) {
-    static_assert(W == 4 || W == 8 || W == 16, "vector width");
-    if constexpr (DT == PILOT_F32) {
-        static_assert(W <= 8, "FP32 vectors are at most 8 wide");
-        if constexpr (W == 8) {
-            // one 256-bit load (32-byte aligned: device feature pointers are validated for it)
-            asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                : "=f"(out[0]), "=f"(out[1]), "=f"(out[2]), "=f"(out[3]), "=f"(out[4]), "=f"(out[5]),
-                  "=f"(out[6]), "=f"(out[7])
-                : "l"(p));
-        } else {
-            const float4 v = __ldg(reinterpret_cast<const float4*>(p));
-            out[0] = v.x; out[1] = v.y; out[2] = v.z; out[3] = v.w;
-        }
-    } else if constexpr (DT == PILOT_BF16 || DT == PILOT_F16) {
-        uint32_t w[W / 2];
-        if constexpr (W == 16) {
-            // one 256-bit load (32-byte aligned: device feature pointers are validated for it)
-            asm("ld.global.nc.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
-                : "l"(p));
-        } else if constexpr (W == 8) {
-            const uint4 r = __ldg(reinterpret_cast<const uint4*>(p));
-            w[0] = r.x; w[1] = r.y; w[2] = r.z; w[3] = r.w;
-        } else {
-            const uint2 r = __ldg(reinterpret_cast<const uint2*>(p));
-            w[0] = r.x; w[1] = r.y;
-        }
+    RawVec<DT, W> v;
+    load_raw<DT, W>(p, v);
 #pragma unroll
-        for (int k = 0; k < W / 2; ++k) {
-            if constexpr (DT == PILOT_BF16) {
-                // bfloat16 is the upper half of an IEEE binary32: widening is a 16-bit shift
-                out[2 * k] = __uint_as_float(w[k] << 16);
-                out[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
-            } else {
-                __half2 h;
-                memcpy(&h, &w[k], 4);
-                const float2 f = __half22float2(h);
-                out[2 * k] = f.x;
-                out[2 * k + 1] = f.y;
-            }
-        }
-    } else {
-        uint32_t w[W / 4];
-        if constexpr (W == 16) {
-            const uint4 r = __ldg(reinterpret_cast<const uint4*>(p));
-            w[0] = r.x; w[1] = r.y; w[2] = r.z; w[3] = r.w;
-        } else if constexpr (W == 8) {
-            const uint2 r = __ldg(reinterpret_cast<const uint2*>(p));
-            w[0] = r.x; w[1] = r.y;
-        } else {
-            w[0] = __ldg(reinterpret_cast<const uint32_t*>(p));
-        }
-#pragma unroll
-        for (int k = 0; k < W / 4; ++k) {
-            const __half2_raw lo = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)(w[k] & 0xffffu), __NV_E4M3);
-            const __half2_raw hi = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)(w[k] >> 16), __NV_E4M3);
-            const float2 a = __half22float2(__half2(lo)), b = __half22float2(__half2(hi));
-            out[4 * k] = a.x; out[4 * k + 1] = a.y; out[4 * k + 2] = b.x; out[4 * k + 3] = b.y;
-        }
-    }
+    for (int e = 0; e < W; e += 2) raw_pair<DT, W>(v, e, out[e], out[e + 1]);
 }
 
 struct ChanSums {
@@ -550,6 +546,347 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
     }
 }
 
+// The 4 taps of one record in this lane's channels (vector k covers VW (q + k LP) .. + VW).
+template <pilot_dtype DT, int C, bool SCALED> struct TapBuf {
+    using G = GroupShape<DT, C, SCALED>;
+    RawVec<DT, G::VW> t[G::NV][4];
+
+    __device__ __forceinline__ void load(const typename Storage<DT>::T* t00, int WC, int q) {
+#pragma unroll
+        for (int k = 0; k < G::NV; ++k) {
+            const typename Storage<DT>::T* p = t00 + G::VW * (q + k * G::LP);
+            load_raw<DT, G::VW>(p, t[k][0]);
+            load_raw<DT, G::VW>(p + C, t[k][1]);
+            load_raw<DT, G::VW>(p + WC, t[k][2]);
+            load_raw<DT, G::VW>(p + WC + C, t[k][3]);
+        }
+    }
+};
+
+// This lane's channels of one anchor's reference row.
+template <pilot_dtype DT, int C, bool SCALED> struct RefBuf {
+    using G = GroupShape<DT, C, SCALED>;
+    RawVec<DT, G::VW> r[G::NV];
+
+    __device__ __forceinline__ void load(const typename Storage<DT>::T* row, int q) {
+#pragma unroll
+        for (int k = 0; k < G::NV; ++k) load_raw<DT, G::VW>(row + G::VW * (q + k * G::LP), r[k]);
+    }
+};
+
+// record_partials on taps and a reference row already loaded: the 4 taps against the anchor's
+// reference values: bilinear value and in-cell gradient, residual, and the six partial sums.
+template <pilot_dtype DT, int C, bool SCALED>
+__device__ __forceinline__ void raw_partials(const TapBuf<DT, C, SCALED>& b, const RefBuf<DT, C, SCALED>& rr,
+                                                float ax, float ay, const float* qs, const float* rs, float* p) {
+    using G = GroupShape<DT, C, SCALED>;
+    constexpr int VW = G::VW;
+    const f2 ax2 = pk(ax, ax), ay2 = pk(ay, ay), z2 = pk(0.f, 0.f);
+    ChanSums2 cs{z2, z2, z2, z2, z2, z2};
+#pragma unroll
+    for (int k = 0; k < G::NV; ++k) {
+#pragma unroll
+        for (int e = 0; e < VW; e += 2) {
+            float a[4][2], r[2];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) raw_pair<DT, VW>(b.t[k][i], e, a[i][0], a[i][1]);
+            raw_pair<DT, VW>(rr.r[k], e, r[0], r[1]);
+            channel_pair<SCALED>(cs, pk(a[0][0], a[0][1]), pk(a[1][0], a[1][1]), pk(a[2][0], a[2][1]),
+                                 pk(a[3][0], a[3][1]), pk(r[0], r[1]), ax2, ay2,
+                                 pk(qs[k * VW + e], qs[k * VW + e + 1]), pk(rs[k * VW + e], rs[k * VW + e + 1]));
+        }
+    }
+    p[0] = hsum(cs.s);
+    p[1] = hsum(cs.m00);
+    p[2] = hsum(cs.m01);
+    p[3] = hsum(cs.m11);
+    p[4] = hsum(cs.b0);
+    p[5] = hsum(cs.b1);
+}
+
+// ---- one hypothesis per CTA ----
+// A record's factors as the chains below read them: W0[6], W1[6] (W = om A), B0[6], B1[6], b0, b1,
+// rho, 1; a record that is not visible is all zeros (adding zero products changes nothing).
+// Rows of 29 words: the lanes' own rows fall into different banks.
+constexpr int kRowWords = 29;
+enum RowCell { kRowW0 = 0, kRowW1 = 6, kRowB0 = 12, kRowB1 = 18, kRowb0 = 24, kRowb1 = 25, kRowRho = 26, kRowOne = 27,
+               kRowZero = 1 /* W0[1] */ };
+
+// The 29 sums over four lanes (the slots of a quad), eight each: four of the form
+// acc = fma(x, y, acc) (the first two rows of H, their g, the cost, the count) and four of the form
+// acc = fma(x, y, fma(z, w, acc)).  Entry: the sum's index, then its cells.
+struct RoleTable {
+    unsigned char sum[4][8], cell[4][24];
+};
+constexpr RoleTable make_roles() {
+    RoleTable t{};
+    int n1 = 0, n2 = 0;
+    for (int i = 0; i < 32; ++i) {
+        t.sum[i / 8][i % 8] = kNumSums;                      // none
+    }
+    for (int i = 0; i < 96; ++i) t.cell[i / 24][i % 24] = kRowZero;
+    int e = 0;
+    for (int a = 0; a < 6; ++a)
+        for (int b = a; b < 6; ++b, ++e) {
+            if (a < 2) {
+                t.sum[n1 / 4][n1 % 4] = e;
+                t.cell[n1 / 4][2 * (n1 % 4)] = (a == 0 ? kRowW0 : kRowW1) + a;
+                t.cell[n1 / 4][2 * (n1 % 4) + 1] = (a == 0 ? kRowB0 : kRowB1) + b;
+                ++n1;
+            } else {
+                unsigned char* c = t.cell[n2 / 4] + 8 + 4 * (n2 % 4);
+                t.sum[n2 / 4][4 + n2 % 4] = e;
+                c[0] = kRowW0 + a, c[1] = kRowB0 + b, c[2] = kRowW1 + a, c[3] = kRowB1 + b;
+                ++n2;
+            }
+        }
+    for (int a = 0; a < 6; ++a) {
+        if (a < 2) {
+            t.sum[n1 / 4][n1 % 4] = 21 + a;
+            t.cell[n1 / 4][2 * (n1 % 4)] = (a == 0 ? kRowW0 : kRowW1) + a;
+            t.cell[n1 / 4][2 * (n1 % 4) + 1] = a == 0 ? kRowb0 : kRowb1;
+            ++n1;
+        } else {
+            unsigned char* c = t.cell[n2 / 4] + 8 + 4 * (n2 % 4);
+            t.sum[n2 / 4][4 + n2 % 4] = 21 + a;
+            c[0] = kRowW0 + a, c[1] = kRowb0, c[2] = kRowW1 + a, c[3] = kRowb1;
+            ++n2;
+        }
+    }
+    for (int i = 0; i < 2; ++i) {                            // cost, count
+        t.sum[n1 / 4][n1 % 4] = 27 + i;
+        t.cell[n1 / 4][2 * (n1 % 4)] = i == 0 ? kRowRho : kRowOne;
+        t.cell[n1 / 4][2 * (n1 % 4) + 1] = kRowOne;
+        ++n1;
+    }
+    return t;
+}
+static __constant__ RoleTable kRoles = make_roles();
+
+// Accumulate anchors [j_begin, j_end) under one hypothesis: the layout of accumulate_anchors with
+// a lane's slot standing for the batch of anchors it takes (slot h: every fourth batch from the
+// h-th), so that a step covers four batches, all of their taps in flight at once.  The records'
+// factors pass through shared memory (rows, one per thread) and a quad's lanes add them in the
+// order of their anchors, eight sums each: the same sums in the same order as with four
+// hypotheses per CTA.  acc: this lane's eight (kRoles.sum[slot]).
+template <pilot_dtype DT, int C, bool SCALED, bool CONF>
+__device__ __forceinline__ void accumulate_spread(const LevelView& v, const float* pose, int j_begin, int j_end,
+                                                  float (*rows)[kRowWords], float* acc) {
+    using Elem = typename Storage<DT>::T;
+    using G = GroupShape<DT, C, SCALED>;
+    constexpr int VW = G::VW, LP = G::LP, NS = G::NS, APB = G::APB, NV = G::NV, CPL = C / LP;
+    constexpr int BATCH = kBuildThreads / (LP * NS) * APB, STEP = kHypTile * BATCH;
+    constexpr int CHUNK = LP < 4 ? LP : 4, HALF = LP / 2;   // records whose taps are in flight
+    const int tid = threadIdx.x, lane = tid & 31, q = lane & (LP - 1), src0 = lane & ~(LP - 1);
+    const int slot = (lane / APB) % kHypTile;
+    const int mine = q % APB + slot * BATCH;                // this lane's anchor in the step
+    const float R00 = pose[0], R01 = pose[1], R02 = pose[2], T0 = pose[3];
+    const float R10 = pose[4], R11 = pose[5], R12 = pose[6], T1 = pose[7];
+    const float R20 = pose[8], R21 = pose[9], R22 = pose[10], T2 = pose[11];
+    float qs[CPL], rs[CPL];
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+#pragma unroll
+        for (int e = 0; e < VW; ++e) {
+            const int ch = VW * (q + k * LP) + e;
+            qs[k * VW + e] = SCALED ? __ldg(v.qscale + ch) : 1.0f;
+            rs[k * VW + e] = SCALED ? __ldg(v.rscale + ch) : 1.0f;
+        }
+    const Elem* qry = static_cast<const Elem*>(v.qry);
+    const Elem* ref = static_cast<const Elem*>(v.ref);
+    const int WC = v.W * C;
+    const float xmax = (float)(v.W - 1), ymax = (float)(v.H - 1), d2 = v.huber * v.huber;
+    int cell[24];
+#pragma unroll
+    for (int i = 0; i < 24; ++i) cell[i] = kRoles.cell[slot][i];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+    float* row = rows[tid];
+
+    float nX = 0.f, nY = 0.f, nZ = 0.f;
+    bool nok = false;
+    const int jfirst = j_begin + (tid / (LP * NS)) * APB;
+    auto fetch = [&](int j) {
+        nok = false;
+        if (j < j_end) {
+            nok = !v.valid || v.valid[j];
+            nX = __ldg(v.px + j), nY = __ldg(v.py + j), nZ = __ldg(v.pz + j);
+        }
+    };
+    fetch(jfirst + mine);
+    const int steps = (j_end - j_begin + STEP - 1) / STEP;  // the same for every thread
+    for (int b = 0, jb = jfirst; b < steps; ++b, jb += STEP) {
+        const float X = nX, Y = nY, Z = nZ;
+        const bool ok = nok;
+        fetch(jb + STEP + mine);
+        bool vis = false;
+        int off = 0;
+        float ax = 0.f, ay = 0.f, x = 0.f, y = 0.f, z = 1.f, iz = 1.f, wq = 1.f;
+        if (ok) {
+            // p = R P + t  (world -> camera)
+            x = fmaf(R00, X, fmaf(R01, Y, fmaf(R02, Z, T0)));
+            y = fmaf(R10, X, fmaf(R11, Y, fmaf(R12, Z, T1)));
+            z = fmaf(R20, X, fmaf(R21, Y, fmaf(R22, Z, T2)));
+            if (z > kZNear) {
+                iz = 1.0f / z;
+                // pixel i covers [i, i+1): array coordinate = pixel - 1/2
+                const float xs = fmaf(v.fx * x, iz, v.cx) - 0.5f;
+                const float ys = fmaf(v.fy * y, iz, v.cy) - 0.5f;
+                if (xs >= 0.f && xs <= xmax && ys >= 0.f && ys <= ymax) {
+                    const int c0 = min((int)xs, v.W - 2);
+                    const int r0 = min((int)ys, v.H - 2);
+                    ax = xs - (float)c0;
+                    ay = ys - (float)r0;
+                    off = (r0 * v.W + c0) * C;
+                    vis = true;
+                    if constexpr (CONF) {  // query confidence, bilinear in the same cell
+                        const float* cp = v.conf + r0 * v.W + c0;
+                        const float c00 = __ldg(cp), c01 = __ldg(cp + 1);
+                        const float c10 = __ldg(cp + v.W), c11 = __ldg(cp + v.W + 1);
+                        const float bq = c01 - c00, cq2 = c10 - c00, dq = (c11 - c10) - bq;
+                        wq = fmaf(ax, fmaf(dq, ay, bq), fmaf(ay, cq2, c00));
+                    }
+                }
+            }
+        }
+        auto combine = [&](float* lo, const float* hi, int half) {
+            const bool upper = (q & half) != 0;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const float send = upper ? lo[k] : hi[k];
+                const float keep = upper ? hi[k] : lo[k];
+                lo[k] = keep + __shfl_xor_sync(0xffffffffu, send, half);
+            }
+        };
+        // the order accumulate_anchors combines its records in: pairs (t, t + LP / 2), the pairs
+        // bit-reversed, as a tree
+        float S[6], B[3][6];
+#pragma unroll
+        for (int c = 0; c < LP; c += CHUNK) {
+            TapBuf<DT, C, SCALED> taps[CHUNK];
+            RefBuf<DT, C, SCALED> rr[CHUNK];
+#pragma unroll
+            for (int m = 0; m < CHUNK; ++m) {
+                const int k = c + m;
+                const int i = LP == 8 ? (k & 1) * 4 + ((k >> 1) & 1) * 2 + (k >> 2) : (LP == 4 ? (k & 1) * 2 + (k >> 1) : k);
+                const int o = LP > 1 ? __shfl_sync(0xffffffffu, off, src0 + i) : off;
+                taps[m].load(qry + o, WC, q);
+                const int ja = jb + i % APB + BATCH * (((src0 + i) / APB) % kHypTile);
+                rr[m].load(ref + (ja < j_end ? ja : j_begin) * C, q);
+            }
+#pragma unroll
+            for (int m = 0; m < CHUNK; ++m) {
+                const int k = c + m;
+                const int i = LP == 8 ? (k & 1) * 4 + ((k >> 1) & 1) * 2 + (k >> 2) : (LP == 4 ? (k & 1) * 2 + (k >> 1) : k);
+                const float axi = LP > 1 ? __shfl_sync(0xffffffffu, ax, src0 + i) : ax;
+                const float ayi = LP > 1 ? __shfl_sync(0xffffffffu, ay, src0 + i) : ay;
+                float* P = LP == 1 || k == 6 ? S : (k & 1) ? B[2] : (k == 0 ? B[0] : B[1]);
+                raw_partials<DT, C, SCALED>(taps[m], rr[m], axi, ayi, qs, rs, P);
+                if (k == 1) combine(B[0], B[2], HALF);
+                if (k == 3) {
+                    combine(B[1], B[2], HALF);
+                    combine(B[0], B[1], HALF / 2);
+                }
+                if (k == 5) combine(B[1], B[2], HALF);
+                if (k == 7) {
+                    combine(S, B[2], HALF);
+                    combine(B[1], S, HALF / 2);
+                    combine(B[0], B[1], 1);
+                }
+            }
+        }
+        if constexpr (LP > 1) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) S[k] = B[0][k];
+        }
+        // the lane's own record: Huber weight, A = d(u,v)/dp [I | -[p]x], the factors of
+        // H += w A^T M A, g += w A^T b
+        float f[28];
+#pragma unroll
+        for (int k = 0; k < 28; ++k) f[k] = 0.f;
+        if (vis) {
+            const float s = S[0], m00 = S[1], m01 = S[2], m11 = S[3];
+            const float w = (v.weight ? __ldg(v.weight + jb + mine) : 1.0f) * wq;
+            const float sw = w * s;
+            float rho, drho;
+            if (sw <= d2) {
+                rho = sw;
+                drho = 1.0f;
+            } else {
+                const float rt = sqrtf(sw);
+                rho = 2.0f * v.huber * rt - d2;
+                drho = v.huber / rt;
+            }
+            const float om = w * drho;
+            const float du_dx = v.fx * iz, du_dz = -v.fx * x * iz * iz;
+            const float dv_dy = v.fy * iz, dv_dz = -v.fy * y * iz * iz;
+            const float A0[6] = {du_dx, 0.f, du_dz, y * du_dz, z * du_dx - x * du_dz, -y * du_dx};
+            const float A1[6] = {0.f, dv_dy, dv_dz, y * dv_dz - z * dv_dy, -x * dv_dz, x * dv_dy};
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                if (k == 0) {
+                    f[kRowB0 + k] = m00 * A0[k];
+                    f[kRowB1 + k] = m01 * A0[k];
+                } else if (k == 1) {
+                    f[kRowB0 + k] = m01 * A1[k];
+                    f[kRowB1 + k] = m11 * A1[k];
+                } else {
+                    f[kRowB0 + k] = fmaf(m00, A0[k], m01 * A1[k]);
+                    f[kRowB1 + k] = fmaf(m01, A0[k], m11 * A1[k]);
+                }
+                if (k != 1) f[kRowW0 + k] = om * A0[k];
+                if (k != 0) f[kRowW1 + k] = om * A1[k];
+            }
+            f[kRowb0] = S[4];
+            f[kRowb1] = S[5];
+            f[kRowRho] = rho;
+            f[kRowOne] = 1.0f;
+        }
+#pragma unroll
+        for (int k = 0; k < 28; ++k) row[k] = f[k];
+        __syncwarp();
+        const float* quad = rows[(tid & ~31) + (lane & ~((kHypTile - 1) * APB))];
+#pragma unroll
+        for (int h = 0; h < kHypTile; ++h) {
+            const float* r = quad + h * APB * kRowWords;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                acc[m] = fmaf(r[cell[2 * m]], r[cell[2 * m + 1]], acc[m]);
+                acc[4 + m] = fmaf(r[cell[8 + 4 * m]], r[cell[9 + 4 * m]],
+                                  fmaf(r[cell[10 + 4 * m]], r[cell[11 + 4 * m]], acc[4 + m]));
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// The CTA's sums of accumulate_spread, in cta_reduce_slots' order: thread t < 32 returns sum t (0
+// pads).  Called by the accumulating warps only (barrier 1).
+template <int APB>
+__device__ __forceinline__ float cta_reduce_spread(float* acc, float (*red)[kAcc]) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        if (off >= APB && off < APB * kHypTile) continue;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
+    }
+    if (lane % APB == 0 && lane < APB * kHypTile) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int s = kRoles.sum[lane / APB][i];
+            if (s < kNumSums) red[warp][s] = acc[i];
+        }
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(kBuildThreads) : "memory");
+    float v = 0.f;
+    if (tid < kNumSums) {
+#pragma unroll
+        for (int w = 0; w < kBuildThreads / 32; ++w) v += red[w][tid];
+    }
+    return v;
+}
+
 // Fixed-order CTA reduction of the lanes' 29 sums, per hypothesis slot: the lanes of a slot
 // are reduced by a butterfly over every lane bit but the slot bits (APB .. APB kHypTile / 2),
 // then the warps in order.  Thread t < kHypTile kAcc returns sum t mod kAcc of slot t / kAcc
@@ -699,6 +1036,186 @@ build_fused_kernel(const FusedBuildParams fp) {
     if (tid == 0) fp.tickets[blockIdx.y] = 0u;
 }
 
+// ---- a whole level of a small frame in one launch ----
+// The CTAs of a hypothesis tile (one per anchor tile, at most kMaxCluster: a thread-block cluster)
+// stay on their SMs through all of a level's LM iterations.  An iteration's tile records and next
+// poses pass through (distributed) shared memory between cluster barriers; the cluster's first
+// CTA sums the records (FP64, the order of the 8-chain sum: at most one record per chain) and runs
+// the FP64 steps.
+//
+// Why: with few anchors an iteration is a chain of latencies -- the launch, eight or more
+// dependent batches of gathers, the FP64 step.  One launch per level drops the launches, and
+// level_spread_kernel shortens the rest while SMs would be idle.  solve_small (4096 anchors, 1
+// hypothesis, 20 iterations): 752 -> 381 us; paper's schedule (500 anchors, 1210 -> 128
+// hypotheses, 12 evaluations): 552 -> 343 us (with the FP64 step's own gain).
+
+// kHypTile hypotheses per CTA.
+template <pilot_dtype DT, int C, bool SCALED, bool CONF>
+__global__ void __launch_bounds__(kBuildThreads, 2)
+level_resident_kernel(const __grid_constant__ ResidentParams rp) {
+    namespace cg = cooperative_groups;
+    const BuildParams& p = rp.b;
+    __shared__ float red[kBuildThreads / 32][kHypTile][kAcc];
+    __shared__ double E[kHypTile][kAcc];
+    __shared__ float rec[kHypTile][kAcc];
+    __shared__ float pose[kHypTile][12];
+    __shared__ int s_cand[kHypTile];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = blockIdx.x, slot0 = kHypTile * (int)blockIdx.y, n = min(kHypTile, p.n_active - slot0);
+    const int iters = rp.iters;
+    auto hyp_of = [&](int h) { return p.active_idx ? p.active_idx[slot0 + h] : slot0 + h; };
+    auto all_ctas = [&]() {
+        if (p.n_tiles > 1) cluster.sync();
+        else __syncthreads();
+    };
+    // level start: damping and flags by the stepping warps, the FP32 poses by every CTA
+    if (rank == 0 && warp < n) {
+        HypState& st = rp.ep.state[hyp_of(warp)];
+        if (rp.T_cw && lane < 12) st.T[lane] = rp.T_cw[12 * (size_t)hyp_of(warp) + lane];
+        if (lane == 0) {
+            st.lambda = rp.ep.lambda0;
+            st.last_fail = 0;
+            st.has_cand = 1;
+        }
+        __syncwarp();
+    }
+    if (tid < 12 * kHypTile) {
+        const int h = tid / 12, hyp = hyp_of(h < n ? h : 0);
+        pose[h][tid % 12] = narrow(rp.T_cw ? rp.T_cw[12 * (size_t)hyp + tid % 12] : __ldcg(rp.ep.state[hyp].T + tid % 12));
+    }
+    if (tid < kHypTile) s_cand[tid] = tid < n;
+    __syncthreads();
+    for (int k = 0; k <= iters; ++k) {
+        SlotPoses sp;
+        bool any = false;
+#pragma unroll
+        for (int h = 0; h < kHypTile; ++h) {
+            sp.p[h] = pose[h];
+            sp.act[h] = s_cand[h] != 0;
+            any = any || sp.act[h];
+        }
+        if (any) {                                       // the same in every CTA of the cluster
+            float acc[kNumSums];
+#pragma unroll
+            for (int i = 0; i < kNumSums; ++i) acc[i] = 0.f;
+            const int j0 = rank * p.tile;
+            accumulate_anchors<DT, C, SCALED, CONF, kBuildThreads>(level_view(p), sp, j0, min(j0 + p.tile, p.N), acc);
+            const float v = cta_reduce_slots<kBuildThreads, GroupShape<DT, C, SCALED>::APB>(acc, red);
+            if (tid < kHypTile * kAcc) rec[tid / kAcc][tid % kAcc] = v;
+        }
+        all_ctas();
+        if (rank == 0) {
+            if (tid < kHypTile * kAcc) {
+                double sum = widen((&rec[0][0])[tid]);
+                for (int t = 1; t < p.n_tiles; ++t) sum += widen(cluster.map_shared_rank(&rec[0][0], t)[tid]);
+                (&E[0][0])[tid] = sum;
+            }
+            __syncthreads();
+            if (warp < n) {
+                const int mode = rp.T_cw ? kEpiEval : (k == 0 ? kEpiInit : kEpiStep);
+                const int cand = lm_update(rp.ep.state[hyp_of(warp)], mode, k < iters, rp.ep.damping_mode, rp.ep.prior,
+                                           E[warp], rp.T_cw ? 0.0 : *rp.min_valid, pose[warp],
+                                           rp.T_cw ? rp.ep.eval_out + (size_t)(slot0 + warp) * kNumSums : nullptr, lane);
+                if (lane == 0) s_cand[warp] = cand;
+            }
+        }
+        all_ctas();
+        if (k < iters && rank != 0) {
+            if (tid < 12 * kHypTile) (&pose[0][0])[tid] = cluster.map_shared_rank(&pose[0][0], 0)[tid];
+            if (tid < kHypTile) s_cand[tid] = cluster.map_shared_rank(s_cand, 0)[tid];
+            __syncthreads();
+        }
+    }
+}
+
+// One hypothesis per CTA, and a ninth warp for its FP64 work: the warp keeps the LM state on its
+// lanes through the level, works out the priors at the candidate while the others gather (they
+// depend on the pose only) and then steps on the records.  One CTA per SM: the registers hold the
+// taps of four batches at once (accumulate_spread).
+constexpr int kSpreadThreads = kBuildThreads + 32;
+
+template <pilot_dtype DT, int C, bool SCALED, bool CONF>
+__global__ void __launch_bounds__(kSpreadThreads, 1)
+level_spread_kernel(const __grid_constant__ ResidentParams rp) {
+    namespace cg = cooperative_groups;
+    const BuildParams& p = rp.b;
+    __shared__ float rows[kBuildThreads][kRowWords];
+    __shared__ float red[kBuildThreads / 32][kAcc];
+    __shared__ float rec[kAcc];
+    __shared__ float pose[12];
+    __shared__ int s_cand;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rank = blockIdx.x, iters = rp.iters;
+    const bool steps = warp == kBuildThreads / 32 && rank == 0;
+    const int slot = blockIdx.y, hyp = p.active_idx ? p.active_idx[slot] : slot;
+    HypState& st = rp.ep.state[hyp];
+    auto all_ctas = [&]() {
+        if (p.n_tiles > 1) cluster.sync();
+        else __syncthreads();
+    };
+    LmLanes s{};
+    int ta = 0, tb = 0;
+    if (warp == kBuildThreads / 32) {
+        s.T = lane < 12 ? (rp.T_cw ? rp.T_cw[12 * (size_t)hyp + lane] : __ldcg(st.T + lane)) : 0.0;
+        s.lambda = rp.ep.lambda0;
+        s.has_cand = 1;
+        if (lane < 12) pose[lane] = narrow(s.T);
+        if (lane == 0) s_cand = 1;
+        if (lane < 21) tri_pair(lane, &ta, &tb);
+    }
+    __syncthreads();
+    for (int k = 0; k <= iters; ++k) {
+        const bool cand = s_cand != 0;                   // the same in every CTA of the cluster
+        PriorTerms terms{};
+        if (warp < kBuildThreads / 32) {
+            if (cand) {
+                float acc[8];
+                const int j0 = rank * p.tile;
+                accumulate_spread<DT, C, SCALED, CONF>(level_view(p), pose, j0, min(j0 + p.tile, p.N), rows, acc);
+                const float v = cta_reduce_spread<GroupShape<DT, C, SCALED>::APB>(acc, red);
+                if (tid < kAcc) rec[tid] = v;
+            }
+        } else if (steps && cand) {
+            terms = prior_terms(rp.ep.prior, k == 0 ? s.T : s.Tc, lane, ta, tb);
+        }
+        all_ctas();
+        if (steps) {
+            double e = 0.0;
+            if (cand && lane < kNumSums) {
+                e = widen(rec[lane]);
+                for (int t = 1; t < p.n_tiles; ++t) e += widen(cluster.map_shared_rank(rec, t)[lane]);
+            }
+            if (cand) e = with_priors(e, terms);
+            if (rp.T_cw) {
+                if (lane < kNumSums) rp.ep.eval_out[(size_t)slot * kNumSums + lane] = e;
+            } else {
+                bool take;
+                lm_lanes_step(s, k == 0 ? kEpiInit : kEpiStep, cand, k < iters, rp.ep.damping_mode, e, *rp.min_valid, lane,
+                              ta, tb, &take);
+                if (s.has_cand && lane < 12) pose[lane] = narrow(s.Tc);
+                if (lane == 0) s_cand = s.has_cand;
+            }
+        }
+        all_ctas();
+        if (k < iters && rank != 0) {
+            if (tid < 12) pose[tid] = cluster.map_shared_rank(pose, 0)[tid];
+            if (tid == 0) s_cand = *cluster.map_shared_rank(&s_cand, 0);
+            __syncthreads();
+        }
+    }
+    if (steps && !rp.T_cw) {                             // what the next level and the selection read
+        if (lane < 12) st.T[lane] = s.T;
+        if (lane == 0) {
+            st.cost = s.cost;
+            st.lambda = s.lambda;
+            st.n_valid = s.n_valid;
+            st.has_cand = s.has_cand;
+            st.last_fail = s.last_fail;
+        }
+    }
+}
+
 template <pilot_dtype DT, int C>
 cudaError_t launch_build_typed(const BuildParams& p, cudaStream_t s) {
     dim3 grid(p.n_tiles, (p.n_active + kHypTile - 1) / kHypTile);
@@ -725,6 +1242,42 @@ cudaError_t launch_build_fused_typed(const FusedBuildParams& p, cudaStream_t s) 
     else
         build_fused_kernel<DT, C, false, false><<<grid, kBuildThreads, 0, s>>>(p);
     return cudaGetLastError();
+}
+
+template <pilot_dtype DT, int C, bool SCALED, bool CONF>
+cudaError_t launch_resident_kernel(const ResidentParams& p, bool spread, cudaStream_t s) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = p.b.n_tiles;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(p.b.n_tiles, spread ? p.b.n_active : (p.b.n_active + kHypTile - 1) / kHypTile);
+    cfg.blockDim = dim3(spread ? kSpreadThreads : kBuildThreads);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return spread ? cudaLaunchKernelEx(&cfg, level_spread_kernel<DT, C, SCALED, CONF>, p)
+                  : cudaLaunchKernelEx(&cfg, level_resident_kernel<DT, C, SCALED, CONF>, p);
+}
+
+template <pilot_dtype DT, int C>
+cudaError_t launch_resident_typed(const ResidentParams& p, bool spread, cudaStream_t s) {
+    if (p.b.qscale && p.b.conf) return launch_resident_kernel<DT, C, true, true>(p, spread, s);
+    if (p.b.qscale) return launch_resident_kernel<DT, C, true, false>(p, spread, s);
+    if (p.b.conf) return launch_resident_kernel<DT, C, false, true>(p, spread, s);
+    return launch_resident_kernel<DT, C, false, false>(p, spread, s);
+}
+
+template <pilot_dtype DT>
+cudaError_t launch_resident_dtype(const ResidentParams& p, bool spread, cudaStream_t s) {
+    switch (p.b.C) {
+        case 4: return launch_resident_typed<DT, 4>(p, spread, s);
+        case 8: return launch_resident_typed<DT, 8>(p, spread, s);
+        case 16: return launch_resident_typed<DT, 16>(p, spread, s);
+        case 32: return launch_resident_typed<DT, 32>(p, spread, s);
+        case 64: return launch_resident_typed<DT, 64>(p, spread, s);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 template <pilot_dtype DT>

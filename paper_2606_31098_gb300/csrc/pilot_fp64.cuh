@@ -31,7 +31,7 @@ __device__ __forceinline__ void huber64(double s, double delta, double delta2, d
         *drho = 1.0;
     } else {
         const double q = sqrt(s);
-        *rho = 2.0 * delta * q - delta2;
+        *rho = fma(2.0 * delta, q, -delta2);
         *drho = delta / q;
     }
 }
@@ -42,22 +42,17 @@ __device__ __forceinline__ void huber64(double s, double delta, double delta2, d
 // lanes -- the three rows of a matrix-vector product, the 28 entries a prior adds, the matrix
 // entries a Cholesky step updates, the three series, the entries of Exp, V and T' -- values move
 // between lanes by shuffles, and comparisons, conversions and truncations are integer
-// operations.  About 150 FP64 instructions per step instead of 415: 27 000 -> 21 000 cycles with
+// operations.  About 150 FP64 instructions per step instead of 415: 27 000 -> 17 000 cycles with
 // both priors at the paper's schedule.  Each value's arithmetic (operations, order, rounding) is
 // the one a single thread would do.
 
-// (row, column) of upper-triangle entry k (row-major), k < 21
-__device__ __forceinline__ void tri_pair(int k, int* a, int* b) {
-    int r = 0, base = 0;           // row r starts at entry base; rows hold 6, 5, ..., 1 entries
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        if (r == i && k >= base + (6 - i)) {
-            base += 6 - i;
-            r = i + 1;
-        }
-    }
-    *a = r;
-    *b = r + (k - base);
+// tri_pair's table: the smaller (or larger) index of upper-triangle entry k (row-major)
+__host__ __device__ constexpr unsigned long long pack_tri(bool second) {
+    unsigned long long v = 0;
+    int k = 0;
+    for (int a = 0; a < 6; ++a)
+        for (int b = a; b < 6; ++b, ++k) v |= (unsigned long long)(second ? b : a) << (3 * k);
+    return v;
 }
 
 // Chain c of the FP64 sum of n tile records in 8 chains: records c, c + 8, ..., in order (0 if
@@ -81,94 +76,97 @@ __device__ __forceinline__ double minus_products(double x0, double y0, double x1
     return fma(x0, y0, -__dmul_rn(x1, y1));
 }
 
-// What lane l keeps of the evaluated pose: i = l mod 3, row i and column i of R, and t_i.
-struct PoseRows {
-    double row[3], col[3], t;
-    int i;
-};
-
-// Gravity direction prior (Eq. 3), added to this lane's entry e of H21 | g6 | cost.  Lane i computes
-// a_i and r_i; rotation block: w [a]x^T [a]x = w (|a|^2 I - a a^T); gradient: w [a]x r = w (a x r).
-__device__ __forceinline__ void add_gravity(const PriorParams& pp, const PoseRows& T, double& e, int lane, int ta,
-                                            int tb) {
-    const double ai = dot3(T.row[0], pp.g_world[0], T.row[1], pp.g_world[1], T.row[2], pp.g_world[2]);
-    const double ri = ai - (T.i == 0 ? pp.g_cam[0] : (T.i == 1 ? pp.g_cam[1] : pp.g_cam[2]));
-    const double a[3] = {shfl_d(ai, 0), shfl_d(ai, 1), shfl_d(ai, 2)};
-    const double r[3] = {shfl_d(ri, 0), shfl_d(ri, 1), shfl_d(ri, 2)};
-    // even lanes |a|^2, odd lanes |r|^2
-    const bool odd = lane & 1;
-    const double v0 = odd ? r[0] : a[0], v1 = odd ? r[1] : a[1], v2 = odd ? r[2] : a[2];
-    const double vv = dot3(v0, v0, v1, v1, v2, v2);
-    const double aa = shfl_d(vv, 0), s = shfl_d(vv, 1);
-    double rho, drho;
-    if (bits(pp.gate_grav) != 0ull && bits(s) > bits(pp.gate_grav2) && bits(s) <= kInfBits) {
-        huber64(pp.gate_grav2, pp.huber_grav, pp.huber_grav2, &rho, &drho);   // gated: constant, no pull
-        if (lane == 27) e = fma(pp.w_grav, rho, e);
-        return;
-    }
-    huber64(s, pp.huber_grav, pp.huber_grav2, &rho, &drho);
-    const double w = bits(drho) == kOneBits ? pp.w_grav : pp.w_grav * drho;
-    auto pick = [](const double* v, int i) { return i == 0 ? v[0] : (i == 1 ? v[1] : v[2]); };
-    // H entries (3 + i, 3 + k) on lanes 15..20, g entries 3 + i on lanes 24..26, the cost on lane 27
-    const bool h = lane < 21;
-    const int i = h ? ta - 3 : (lane >= 24 ? lane - 24 : 0), k = h ? tb - 3 : 0;
-    const int u = i == 2 ? 0 : i + 1, v = u == 2 ? 0 : u + 1;
-    const double p = h ? -pick(a, i) : pick(a, u), q = h ? pick(a, k) : pick(r, v);
-    const double m = __dmul_rn(pick(a, v), pick(r, u));
-    const double val = fma(p, q, h ? (i == k ? aa : 0.0) : -m);
-    if (lane == 27) e = fma(pp.w_grav, rho, e);
-    else if ((lane >= 15 && lane < 21) || (lane >= 24 && lane < 27)) e = fma(w, val, e);
+// (column, row) of the upper triangle for lane l < 21, three bits per lane
+__device__ __forceinline__ void tri_pair(int l, int* a, int* b) {
+    // lanes 0-5: a = 0; 6-10: 1; 11-14: 2; 15-17: 3; 18-19: 4; 20: 5
+    constexpr unsigned long long ka = pack_tri(false), kb = pack_tri(true);
+    *a = (int)(ka >> (3 * l)) & 7;
+    *b = (int)(kb >> (3 * l)) & 7;
 }
 
-// Laser range prior (Eq. 4-6); dropped when the range point leaves the DSM.
-__device__ __forceinline__ void add_range(const PriorParams& pp, const PoseRows& T, double& e, int lane, int ta,
-                                          int tb) {
-    const int li = T.i, lu = li == 2 ? 0 : li + 1, lv = lu == 2 ? 0 : lu + 1;
-    auto pick = [](const double* v, int i) { return i == 0 ? v[0] : (i == 1 ? v[1] : v[2]); };
-    const double di = pick(pp.q, li) - T.t;
-    const double d0 = shfl_d(di, 0), d1 = shfl_d(di, 1), d2 = shfl_d(di, 2);
-    const double Pi = dot3(T.col[0], d0, T.col[1], d1, T.col[2], d2);          // R^T d
-    // x on lanes 0 mod 3, y on lanes 1 mod 3
-    const double inv_gsd = pp.dsm_inv_gsd;
-    const double gi = (Pi - (li == 0 ? pp.dsm_x0 : pp.dsm_y0)) * inv_gsd - 0.5;
-    const bool in = within(gi, li == 0 ? pp.dsm_wmax : pp.dsm_hmax);
-    if ((__ballot_sync(0xffffffffu, in) & 3u) != 3u) return;
-    const int ci = min(whole_part(gi), (li == 0 ? pp.dsm_W : pp.dsm_H) - 2);
-    const double fi = gi - as_double(ci);
-    const int c0 = __shfl_sync(0xffffffffu, ci, 0), r0 = __shfl_sync(0xffffffffu, ci, 1);
-    const double ax = shfl_d(fi, 0), ay = shfl_d(fi, 1);
-    const float* row0 = pp.dsm + (size_t)r0 * pp.dsm_W + c0;
-    const float* row1 = row0 + pp.dsm_W;
-    const double h00 = widen(row0[0]), h01 = widen(row0[1]), h10 = widen(row1[0]), h11 = widen(row1[1]);
-    // bx on lanes 0 mod 3, cy on lanes 1 mod 3, the lower difference on lanes 2 mod 3
-    const double diff = (li == 0 ? h01 : (li == 1 ? h10 : h11)) - (li == 2 ? h10 : h00);
-    const double bx = shfl_d(diff, 0), cy = shfl_d(diff, 1);
-    const double dxy = shfl_d(diff, 2) - bx;
-    const double ui = (li == 0 ? bx : cy) + dxy * (li == 0 ? ay : ax);
-    const double gradi = ui * inv_gsd;
-    const double D = h00 + ax * shfl_d(ui, 0) + ay * cy;
-    const double Dx = shfl_d(gradi, 0), Dy = shfl_d(gradi, 1);
-    const double r = shfl_d(Pi, 2) - D;
-    double rho, drho;
-    const unsigned long long ra = bits(r) & 0x7fffffffffffffffull;
-    if (bits(pp.gate_range) != 0ull && ra > bits(pp.gate_range) && ra <= kInfBits) {
-        huber64(pp.gate_range2, pp.huber_range, pp.huber_range2, &rho, &drho);  // gated: constant, no pull
-        if (lane == 27) e = fma(pp.w_range, rho, e);
-        return;
+// What the priors add to this lane's entry of H21 | g6 | cost: entry + gw gx (gravity), then + rw rx
+// (range), each fused.  They depend on the pose only, so they can be had before the photo sums.
+struct PriorTerms {
+    double gw, gx, rw, rx;
+};
+
+__device__ __forceinline__ double with_priors(double e, const PriorTerms& t) { return fma(t.rw, t.rx, fma(t.gw, t.gx, e)); }
+
+// Gravity direction prior (Eq. 3) and laser range prior (Eq. 4-6; dropped when the range point
+// leaves the DSM) at the pose of which lane l < 12 holds entry l.  Gravity: lane i computes a_i and
+// r_i; rotation block w [a]x^T [a]x = w (|a|^2 I - a a^T), gradient w [a]x r = w (a x r).
+__device__ __forceinline__ PriorTerms prior_terms(const PriorParams& pp, double T, int lane, int ta, int tb) {
+    PriorTerms out{0.0, 0.0, 0.0, 0.0};
+    const int li = lane % 3, lu = li == 2 ? 0 : li + 1, lv = lu == 2 ? 0 : lu + 1;
+    const double R0 = shfl_d(T, 4 * li), R1 = shfl_d(T, 4 * li + 1), R2 = shfl_d(T, 4 * li + 2);
+    if (pp.use_gravity) {
+        const double ai = dot3(R0, pp.g_world[0], R1, pp.g_world[1], R2, pp.g_world[2]);
+        const double ri = ai - pp.g_cam[li];
+        // even lanes |a|^2, odd lanes |r|^2: a on lanes 0..2, r on lanes 3..5
+        const double y = lane < 3 ? ai : ri;
+        const int o = (lane & 1) ? 3 : 0;
+        const double v0 = shfl_d(y, o), v1 = shfl_d(y, o + 1), v2 = shfl_d(y, o + 2);
+        const double vv = dot3(v0, v0, v1, v1, v2, v2);
+        const double aa = shfl_d(vv, 0), s = shfl_d(vv, 1);
+        // H entries (3 + i, 3 + k) on lanes 15..20, g entries 3 + i on lanes 24..26, the cost on lane 27
+        const bool h = lane < 21;
+        const int i = h ? max(ta - 3, 0) : (lane >= 24 && lane < 27 ? lane - 24 : 0), k = h ? max(tb - 3, 0) : 0;
+        const int u = i == 2 ? 0 : i + 1, v = u == 2 ? 0 : u + 1;
+        // p q - m with p q = -a_i a_k (H) or a_u r_v (g)
+        const double p = shfl_d(y, h ? i : u), q = shfl_d(y, h ? k : 3 + v);
+        const double m = __dmul_rn(shfl_d(y, v), shfl_d(y, 3 + u));
+        const double val = fma(h ? -p : p, q, h ? (i == k ? aa : 0.0) : -m);
+        double rho, drho;
+        const bool gated = bits(pp.gate_grav) != 0ull && bits(s) > bits(pp.gate_grav2) && bits(s) <= kInfBits;
+        huber64(gated ? pp.gate_grav2 : s, pp.huber_grav, pp.huber_grav2, &rho, &drho);
+        const double w = bits(drho) == kOneBits ? pp.w_grav : pp.w_grav * drho;
+        if (lane == 27) out.gw = pp.w_grav, out.gx = rho;
+        else if (!gated && ((lane >= 15 && lane < 21) || (lane >= 24 && lane < 27))) out.gw = w, out.gx = val;
     }
-    // dr/dP = (-Dx, -Dy, 1); dP/ddelta = R^T [-I | [q]x]  =>  J = [-n | n x q], n = R (-Dx, -Dy, 1)
-    const double ni = fma(T.row[0], -Dx, __dmul_rn(T.row[1], -Dy)) + T.row[2];
-    const double nu = shfl_d(ni, lu), nv = shfl_d(ni, lv);
-    const double xi = minus_products(nu, pick(pp.q, lv), nv, pick(pp.q, lu));
-    huber64(r * r, pp.huber_range, pp.huber_range2, &rho, &drho);
-    const double w = bits(drho) == kOneBits ? pp.w_range : pp.w_range * drho;
-    // this lane's J[a] and its factor: J[b] (H), r (g), rho (cost)
-    const int a = lane < 21 ? ta : (lane < 27 ? lane - 21 : 0), b = lane < 21 ? tb : 0;
-    const int a3 = a < 3 ? a : a - 3, b3 = b < 3 ? b : b - 3;
-    const double na = shfl_d(ni, a3), xa = shfl_d(xi, a3), nb = shfl_d(ni, b3), xb = shfl_d(xi, b3);
-    const double Ja = a < 3 ? -na : xa, Jb = b < 3 ? -nb : xb;
-    const double m = w * Ja;
-    if (lane < 28) e = fma(lane == 27 ? pp.w_range : m, lane < 21 ? Jb : (lane < 27 ? r : rho), e);
+    if (pp.use_range) {
+        const double C0 = shfl_d(T, li), C1 = shfl_d(T, 4 + li), C2 = shfl_d(T, 8 + li);
+        const double di = pp.q[li] - shfl_d(T, 4 * li + 3);
+        const double d0 = shfl_d(di, 0), d1 = shfl_d(di, 1), d2 = shfl_d(di, 2);
+        const double Pi = dot3(C0, d0, C1, d1, C2, d2);                           // R^T d
+        // x on lanes 0 mod 3, y on lanes 1 mod 3
+        const double inv_gsd = pp.dsm_inv_gsd;
+        const double gi = fma(Pi - (li == 0 ? pp.dsm_x0 : pp.dsm_y0), inv_gsd, -0.5);
+        const bool in = within(gi, li == 0 ? pp.dsm_wmax : pp.dsm_hmax);
+        if ((__ballot_sync(0xffffffffu, in) & 3u) != 3u) return out;
+        const int ci = min(whole_part(gi), (li == 0 ? pp.dsm_W : pp.dsm_H) - 2);
+        const double fi = gi - as_double(ci);
+        const int c0 = __shfl_sync(0xffffffffu, ci, 0), r0 = __shfl_sync(0xffffffffu, ci, 1);
+        const float* row0 = pp.dsm + (size_t)r0 * pp.dsm_W + c0;
+        const float* row1 = row0 + pp.dsm_W;
+        const float f00 = row0[0], f01 = row0[1], f10 = row1[0], f11 = row1[1];
+        const double ax = shfl_d(fi, 0), ay = shfl_d(fi, 1);
+        const double h00 = widen(f00), h10 = widen(f10);
+        // bx on lanes 0 mod 3, cy on lanes 1 mod 3, the lower difference on lanes 2 mod 3
+        const double diff = (li == 0 ? widen(f01) : (li == 1 ? h10 : widen(f11))) - (li == 2 ? h10 : h00);
+        const double bx = shfl_d(diff, 0), cy = shfl_d(diff, 1);
+        const double dxy = shfl_d(diff, 2) - bx;
+        const double ui = fma(dxy, li == 0 ? ay : ax, li == 0 ? bx : cy);
+        const double gradi = ui * inv_gsd;
+        const double D = fma(ay, cy, fma(ax, shfl_d(ui, 0), h00));
+        const double Dx = shfl_d(gradi, 0), Dy = shfl_d(gradi, 1);
+        const double r = shfl_d(Pi, 2) - D;
+        const unsigned long long ra = bits(r) & 0x7fffffffffffffffull;
+        const bool gated = bits(pp.gate_range) != 0ull && ra > bits(pp.gate_range) && ra <= kInfBits;
+        // dr/dP = (-Dx, -Dy, 1); dP/ddelta = R^T [-I | [q]x]  =>  J = [-n | n x q], n = R (-Dx, -Dy, 1)
+        const double ni = fma(R0, -Dx, __dmul_rn(R1, -Dy)) + R2;
+        const double xi = minus_products(shfl_d(ni, lu), pp.q[lv], shfl_d(ni, lv), pp.q[lu]);
+        double rho, drho;
+        huber64(gated ? pp.gate_range2 : r * r, pp.huber_range, pp.huber_range2, &rho, &drho);
+        const double w = bits(drho) == kOneBits ? pp.w_range : pp.w_range * drho;
+        // this lane's J[a] and its factor: J[b] (H), r (g), rho (cost)
+        const int a = lane < 21 ? ta : (lane < 27 ? lane - 21 : 0), b = lane < 21 ? tb : 0;
+        const double y = lane < 3 ? -ni : xi;                                     // J on lanes 0..5
+        const double Ja = shfl_d(y, a), Jb = shfl_d(y, b);
+        const double m = w * Ja;
+        if (lane == 27) out.rw = pp.w_range, out.rx = rho;
+        else if (!gated && lane < 27) out.rw = m, out.rx = lane < 21 ? Jb : r;
+    }
+    return out;
 }
 
 // s = sqrt(d) and inv = 1 / s, each rounded to nearest, for d > 0.  An FP32 estimate of 1 / sqrt(d)
@@ -257,7 +255,7 @@ __device__ __forceinline__ void exp_coefficients(double x, double* A, double* B,
 #pragma unroll
         for (int k = 7; k >= 0; --k) {
             const double c = o == 0 ? f[2 * k + 1] : (o == 1 ? f[2 * k + 2] : f[2 * k + 3]);
-            v = c - x * v;
+            v = fma(-x, v, c);
         }
         *A = shfl_d(v, 0);
         *B = shfl_d(v, 1);
@@ -295,9 +293,9 @@ __device__ __forceinline__ double pose_update(const double* xi, double T, int la
         if (i == 1 && k == 2) Kik = -w0;
         if (i == 2 && k == 0) Kik = -w1;
         if (i == 2 && k == 1) Kik = w0;
-        const double K2 = wi * wk - (i == k ? th2 : 0.0);
+        const double K2 = fma(wi, wk, -(i == k ? th2 : 0.0));
         const double I = (i == k) ? 1.0 : 0.0;
-        W = I + (ex ? A : B) * Kik + (ex ? B : Cc) * K2;
+        W = fma(ex ? B : Cc, K2, fma(ex ? A : B, Kik, I));
     }
     const bool rot = lane < 12;
     const int i = rot ? lane >> 2 : (lane < 15 ? lane - 12 : 0), k = lane & 3;
@@ -314,90 +312,97 @@ __device__ __forceinline__ void store_pose32(float* dst, const double* T) {
     for (int i = 0; i < 12; ++i) dst[i] = (float)T[i];
 }
 
-// One hypothesis' FP64 step after a build pass at its candidate.  E (29 sums, photo term only, in
-// the warp's shared memory) gets the priors at the evaluated pose; then
+// LM state of one hypothesis on a warp: entry l of T and of the candidate Tc on lane l < 12, of H
+// and g on lanes l < 27; the rest on every lane.
+struct LmLanes {
+    double T, Tc, hg, cost, lambda;
+    int n_valid, has_cand, last_fail;
+};
+
+// The LM step (kEpiInit or kEpiStep) after a build pass at the candidate: e is this lane's entry of
+// the sums, priors included (lane 27: cost, lane 28: visible anchors), read only when evaluated.
+// Accepts or rejects, then solves for the next candidate (solve_next).  All 32 lanes.
+__device__ __forceinline__ void lm_lanes_step(LmLanes& s, int mode, bool evaluated, int solve_next, int damping_mode,
+                                              double e, double min_valid, int lane, int ta, int tb, bool* take) {
+    *take = false;
+    if (mode == kEpiInit) {
+        *take = true;
+    } else if (evaluated) {
+        *take = shfl_d(e, 27) < s.cost && bits(min_valid) <= bits(shfl_d(e, 28));  // a count and a threshold >= 0
+        s.lambda = *take ? fmax(tenth(s.lambda), kLambdaMin) : fmin(s.lambda * 10.0, kLambdaMax);
+    }
+    if (*take) {
+        s.hg = e;
+        s.cost = shfl_d(e, 27);
+        s.n_valid = whole_part(shfl_d(e, 28));
+        if (mode == kEpiStep) s.T = s.Tc;
+    }
+    s.has_cand = 0;
+    if (solve_next) {
+        double dxi[6];
+        if (!damped_solve(s.hg, ta, tb, s.lambda, damping_mode, dxi, lane)) {
+            s.lambda = fmin(s.lambda * 10.0, kLambdaMax);
+            s.last_fail = 1;
+        } else {
+            s.last_fail = 0;
+            s.Tc = pose_update(dxi, s.T, lane);
+            s.has_cand = 1;
+        }
+    }
+}
+
+// One hypothesis' FP64 step after a build pass at its candidate, its state in memory.  E (29 sums,
+// photo term only, in the warp's shared memory) gets the priors at the evaluated pose; then
 // (init) it becomes the current state, or (step) the candidate is accepted or rejected; then
-// the next candidate is solved for and, if cand32 is given, written there in FP32.  All 32
-// lanes of one warp call it with the same arguments.  Returns whether there is a candidate.
-//
-// Not inlined: every kernel of a translation unit (plain fused, batched, served) then runs
-// the same compiled instructions, so the compiler cannot contract a * b + c into an FMA in
-// one caller and not in another, and the forms stay bitwise equal.
+// the next candidate is solved for and, if cand32 is given, written there in FP32; or (eval) the
+// sums go to eval_out.  All 32 lanes of one warp call it with the same arguments.  Returns whether
+// there is a candidate.  The contractions of its products are written out, so that every kernel
+// computes the same bits; not inlined, to keep the callers' registers.
 static __device__ __noinline__ int lm_update(HypState& st, int mode, int solve_next, int damping_mode,
                                              const PriorParams& prior, const double* E,
                                              double min_valid, float* cand32, double* eval_out, int lane) {
     // every read of the state is issued here, before any write, as one round trip, from L2:
     // the persistent level kernel may step a hypothesis on another SM than the last time
+    LmLanes s;
     const int has_cand = __ldcg(&st.has_cand);
-    const double cost0 = __ldcg(&st.cost);
-    const double lambda0 = __ldcg(&st.lambda);
-    const double* Tsrc = (mode == kEpiStep) ? st.Tc : st.T;
-    PoseRows Tev;
-    Tev.i = lane % 3;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        Tev.row[k] = __ldcg(Tsrc + 4 * Tev.i + k);
-        Tev.col[k] = __ldcg(Tsrc + 4 * k + Tev.i);
-    }
-    Tev.t = __ldcg(Tsrc + 4 * Tev.i + 3);
-    const double Hg_own = lane < 21 ? __ldcg(st.H + lane) : (lane < 27 ? __ldcg(st.g + lane - 21) : 0.0);
-    const double T_own = lane < 12 ? __ldcg(st.T + lane) : 0.0;
-    const double Tc_own = lane < 12 ? __ldcg(st.Tc + lane) : 0.0;
+    s.cost = __ldcg(&st.cost);
+    s.lambda = __ldcg(&st.lambda);
+    s.hg = lane < 21 ? __ldcg(st.H + lane) : (lane < 27 ? __ldcg(st.g + lane - 21) : 0.0);
+    s.T = lane < 12 ? __ldcg(st.T + lane) : 0.0;
+    s.Tc = lane < 12 ? __ldcg(st.Tc + lane) : 0.0;
+    s.last_fail = -1;
     const bool evaluated = (mode == kEpiStep) ? (has_cand != 0) : true;
     int ta = 0, tb = 0;
     if (lane < 21) tri_pair(lane, &ta, &tb);
     double e = evaluated && lane < kNumSums ? E[lane] : 0.0;
-    if (evaluated) {
-        if (prior.use_gravity) add_gravity(prior, Tev, e, lane, ta, tb);
-        if (prior.use_range) add_range(prior, Tev, e, lane, ta, tb);
-    }
-    __syncwarp();
+    if (evaluated) e = with_priors(e, prior_terms(prior, mode == kEpiStep ? s.Tc : s.T, lane, ta, tb));
     if (mode == kEpiEval) {
         if (lane < kNumSums) eval_out[lane] = e;
         if (lane == 0) st.has_cand = 0;
         return 0;
     }
-    // the state after acceptance: H 0..20, g 21..26 and T 0..11 on their lanes
-    bool take = false;
-    double lambda = lambda0;
-    if (mode == kEpiInit) {
-        take = true;
-    } else if (evaluated) {
-        take = shfl_d(e, 27) < cost0 && bits(min_valid) <= bits(shfl_d(e, 28));    // a count and a threshold >= 0
-        lambda = take ? fmax(tenth(lambda0), kLambdaMin) : fmin(lambda0 * 10.0, kLambdaMax);
-    }
-    const double hg = take ? e : Hg_own;
-    const double T = (take && mode == kEpiStep) ? Tc_own : T_own;
+    bool take;
+    lm_lanes_step(s, mode, evaluated, solve_next, damping_mode, e, min_valid, lane, ta, tb, &take);
     if (take) {
-        if (lane < 21) st.H[lane] = e;
-        else if (lane < 27) st.g[lane - 21] = e;
-        else if (lane == 27) st.cost = e;
-        else if (lane == 28) st.n_valid = whole_part(e);
-        if (mode == kEpiStep && lane < 12) st.T[lane] = T;
+        if (lane < 21) st.H[lane] = s.hg;
+        else if (lane < 27) st.g[lane - 21] = s.hg;
+        if (mode == kEpiStep && lane < 12) st.T[lane] = s.T;
     }
-    int cand = 0, fail = -1;
-    if (solve_next) {
-        double dxi[6];
-        if (!damped_solve(hg, ta, tb, lambda, damping_mode, dxi, lane)) {
-            lambda = fmin(lambda * 10.0, kLambdaMax);
-            fail = 1;
-        } else {
-            fail = 0;
-            const double Tn = pose_update(dxi, T, lane);
-            if (lane < 12) {
-                st.Tc[lane] = Tn;
-                if (cand32) cand32[lane] = narrow(Tn);
-            }
-            cand = 1;
-        }
+    if (s.has_cand && lane < 12) {
+        st.Tc[lane] = s.Tc;
+        if (cand32) cand32[lane] = narrow(s.Tc);
     }
     if (lane == 0) {
-        st.lambda = lambda;
-        if (fail >= 0) st.last_fail = fail;
-        st.has_cand = cand;
+        if (take) {
+            st.cost = s.cost;
+            st.n_valid = s.n_valid;
+        }
+        st.lambda = s.lambda;
+        if (s.last_fail >= 0) st.last_fail = s.last_fail;
+        st.has_cand = s.has_cand;
     }
     __syncwarp();
-    return cand;
+    return s.has_cand;
 }
 
 // lm_update for slot `slot` of a launch described by p (candidate written to p.pose32); all

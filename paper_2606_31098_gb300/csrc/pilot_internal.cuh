@@ -150,6 +150,34 @@ struct FusedBuildParams {
     const double* min_valid;
 };
 
+// A whole level in one launch (level_resident_kernel): ep's state, prior, damping_mode, lambda0;
+// ep.mode and ep.solve_next follow from the iteration.  T_cw given: instead, one evaluation at
+// these poses (M x 12, device), the sums to ep.eval_out, slot s being hypothesis s when
+// b.active_idx is NULL.
+struct ResidentParams {
+    BuildParams b;
+    EpilogueParams ep;
+    const double* min_valid;
+    const double* T_cw;
+    int iters;
+};
+
+constexpr int kMaxCluster = 8;     // anchor tiles of a level run that way (portable cluster size)
+
+// Whether a level of n_active hypotheses over n_tiles anchor tiles runs in one launch, and with one
+// hypothesis per CTA (2, level_spread_kernel) or kHypTile (1, level_resident_kernel); 0: a launch
+// per iteration.  One hypothesis per CTA while every CTA has an SM of its own.  Else kHypTile: with
+// one tile always (no CTA waits for another), with more while all CTAs are resident at once (two
+// per SM), since the other CTAs of a cluster idle during its FP64 steps and larger levels use
+// those SMs for the next launch.
+inline int resident_kind(int n_active, int n_tiles) {
+    constexpr int kSms = 152;
+    if (n_tiles > kMaxCluster) return 0;
+    if ((long long)n_active * n_tiles <= kSms) return 2;
+    const long long ctas = (long long)((n_active + kHypTile - 1) / kHypTile) * n_tiles;
+    return n_tiles == 1 || ctas <= 2 * kSms ? 1 : 0;
+}
+
 // ---- batched form: many frames, one persistent launch per pyramid level ----
 
 // One frame of a batch, as the device kernels see it.
@@ -255,6 +283,10 @@ template <pilot_dtype DT>
 cudaError_t launch_build_dtype(const BuildParams& p, cudaStream_t s);
 template <pilot_dtype DT>
 cudaError_t launch_build_fused_dtype(const FusedBuildParams& p, cudaStream_t s);
+
+template <pilot_dtype DT>
+cudaError_t launch_resident_dtype(const ResidentParams& p, bool spread, cudaStream_t s);
+cudaError_t launch_resident(pilot_dtype dt, const ResidentParams& p, bool spread, cudaStream_t s);
 
 template <pilot_dtype DT>
 cudaError_t launch_level_persistent_dtype(int C, int variant, const LevelArgs& a, int grid,

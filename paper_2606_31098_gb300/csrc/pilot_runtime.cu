@@ -392,9 +392,9 @@ cudaError_t dispatch_build_fused(pilot_dtype dt, const FusedBuildParams& b, cuda
     return cudaErrorInvalidValue;
 }
 
-// One build launch, plain (ep == nullptr) or with the FP64 step fused in.
-pilot_status run_build(pilot_align_handle* h, pilot_dtype dt, const BuildParams& b, cudaStream_t s,
-                       const EpilogueParams* ep = nullptr, int slot_offset = 0) {
+// One build launch (with profiling, between two events).
+template <typename Launch>
+pilot_status timed_build(pilot_align_handle* h, cudaStream_t s, Launch launch) {
     const bool prof = h->cfg.profile != 0;
     size_t k = 2 * (size_t)h->build_launches;
     if (prof) {
@@ -405,16 +405,20 @@ pilot_status run_build(pilot_align_handle* h, pilot_dtype dt, const BuildParams&
         }
         PILOT_CUDA(cudaEventRecord(h->events[k], s), "event record");
     }
-    if (ep) {
-        FusedBuildParams fb{b, *ep, h->tickets + slot_offset, h->min_valid};
-        PILOT_CUDA(dispatch_build_fused(dt, fb, s), "fused build-pass launch");
-    } else {
-        PILOT_CUDA(dispatch_build(dt, b, s), "build-pass launch");
-    }
+    PILOT_CUDA(launch(), "build-pass launch");
     if (prof) PILOT_CUDA(cudaEventRecord(h->events[k + 1], s), "event record");
     ++h->build_launches;
     ++h->total_launches;
     return PILOT_OK;
+}
+
+// One build launch, plain (ep == nullptr) or with the FP64 step fused in.
+pilot_status run_build(pilot_align_handle* h, pilot_dtype dt, const BuildParams& b, cudaStream_t s,
+                       const EpilogueParams* ep = nullptr, int slot_offset = 0) {
+    return timed_build(h, s, [&]() {
+        return ep ? dispatch_build_fused(dt, FusedBuildParams{b, *ep, h->tickets + slot_offset, h->min_valid}, s)
+                  : dispatch_build(dt, b, s);
+    });
 }
 
 long long schedule_key(int batched, pilot_dtype dt, int C, double mean_n, double mean_m) {
@@ -587,6 +591,15 @@ cudaError_t level_occupancy(pilot_dtype dt, int C, int variant, int* n) {
 }  // namespace
 
 namespace pilot {
+cudaError_t launch_resident(pilot_dtype dt, const ResidentParams& p, bool spread, cudaStream_t s) {
+    switch (dt) {
+        case PILOT_F32: return launch_resident_dtype<PILOT_F32>(p, spread, s);
+        case PILOT_BF16: return launch_resident_dtype<PILOT_BF16>(p, spread, s);
+        case PILOT_F16: return launch_resident_dtype<PILOT_F16>(p, spread, s);
+        case PILOT_FP8E4M3: return launch_resident_dtype<PILOT_FP8E4M3>(p, spread, s);
+    }
+    return cudaErrorInvalidValue;
+}
 cudaError_t level_launch(pilot_dtype dt, int C, int variant, const LevelArgs& a, int grid, cudaStream_t s) {
     return launch_level(dt, C, variant, a, grid, s);
 }
@@ -828,39 +841,46 @@ pilot_status pilot_align_solve(pilot_align_handle* h, const pilot_frame* f, pilo
         ep.damping_mode = c.damping_mode;
         ep.prior = prior;
         if (overlap && level < f->L - 1) PILOT_CUDA(cudaStreamWaitEvent(s, h->level_ready[level], 0), "level copy wait");
-        PILOT_CUDA(launch_level_init(h->state, h->pose32, h->active[cur], n_active, c.lambda0, s), "level_init launch");
-        ++h->total_launches;
-        // parts of the active list, part p = slots [off[p], off[p + 1]) on stream p (s for
-        // p = 0), each with its own slice of the partial records and tickets
-        const int parts = n_streams < n_active ? n_streams : n_active;
-        int off[kMaxStreams + 1];
-        BuildParams bp[kMaxStreams];
-        EpilogueParams epp[kMaxStreams];
-        cudaStream_t sp[kMaxStreams];
-        for (int p = 0; p <= parts; ++p) off[p] = (int)(((long long)n_active * p) / parts);
-        for (int p = 0; p < parts; ++p) {
-            bp[p] = b;
-            epp[p] = ep;
-            bp[p].n_active = epp[p].n_active = off[p + 1] - off[p];
-            bp[p].active_idx = epp[p].active_idx = b.active_idx + off[p];
-            bp[p].partial = b.partial + (size_t)off[p] * b.n_tiles * kAcc;
-            epp[p].partial = bp[p].partial;
-            sp[p] = p ? h->pstream[p - 1] : s;
-        }
-        if (parts > 1) {
-            PILOT_CUDA(cudaEventRecord(h->pfork, s), "fork record");
-            for (int p = 1; p < parts; ++p) PILOT_CUDA(cudaStreamWaitEvent(sp[p], h->pfork, 0), "fork wait");
-        }
-        for (int k = 0; k <= iters; ++k) {
+        const int kind = resident_kind(n_active, b.n_tiles);
+        if (kind != 0) {
+            const ResidentParams rp{b, ep, h->min_valid, nullptr, iters};
+            if ((st = timed_build(h, s, [&]() { return launch_resident(f->feat_dtype, rp, kind == 2, s); })) != PILOT_OK)
+                return st;
+        } else {
+            PILOT_CUDA(launch_level_init(h->state, h->pose32, h->active[cur], n_active, c.lambda0, s), "level_init launch");
+            ++h->total_launches;
+            // parts of the active list, part p = slots [off[p], off[p + 1]) on stream p (s for
+            // p = 0), each with its own slice of the partial records and tickets
+            const int parts = n_streams < n_active ? n_streams : n_active;
+            int off[kMaxStreams + 1];
+            BuildParams bp[kMaxStreams];
+            EpilogueParams epp[kMaxStreams];
+            cudaStream_t sp[kMaxStreams];
+            for (int p = 0; p <= parts; ++p) off[p] = (int)(((long long)n_active * p) / parts);
             for (int p = 0; p < parts; ++p) {
-                epp[p].mode = (k == 0) ? kEpiInit : kEpiStep;
-                epp[p].solve_next = k < iters;
-                if ((st = run_build(h, f->feat_dtype, bp[p], sp[p], &epp[p], off[p])) != PILOT_OK) return st;
+                bp[p] = b;
+                epp[p] = ep;
+                bp[p].n_active = epp[p].n_active = off[p + 1] - off[p];
+                bp[p].active_idx = epp[p].active_idx = b.active_idx + off[p];
+                bp[p].partial = b.partial + (size_t)off[p] * b.n_tiles * kAcc;
+                epp[p].partial = bp[p].partial;
+                sp[p] = p ? h->pstream[p - 1] : s;
             }
-        }
-        for (int p = 1; p < parts; ++p) {
-            PILOT_CUDA(cudaEventRecord(h->pjoin[p - 1], sp[p]), "join record");
-            PILOT_CUDA(cudaStreamWaitEvent(s, h->pjoin[p - 1], 0), "join wait");
+            if (parts > 1) {
+                PILOT_CUDA(cudaEventRecord(h->pfork, s), "fork record");
+                for (int p = 1; p < parts; ++p) PILOT_CUDA(cudaStreamWaitEvent(sp[p], h->pfork, 0), "fork wait");
+            }
+            for (int k = 0; k <= iters; ++k) {
+                for (int p = 0; p < parts; ++p) {
+                    epp[p].mode = (k == 0) ? kEpiInit : kEpiStep;
+                    epp[p].solve_next = k < iters;
+                    if ((st = run_build(h, f->feat_dtype, bp[p], sp[p], &epp[p], off[p])) != PILOT_OK) return st;
+                }
+            }
+            for (int p = 1; p < parts; ++p) {
+                PILOT_CUDA(cudaEventRecord(h->pjoin[p - 1], sp[p]), "join record");
+                PILOT_CUDA(cudaStreamWaitEvent(s, h->pjoin[p - 1], 0), "join wait");
+            }
         }
         hyp_iters += (long long)n_active * iters;
         const int K = c.keep_top_k[level];
@@ -911,9 +931,13 @@ pilot_status pilot_align_debug_normal_eq(pilot_align_handle* h, const pilot_fram
     DevFrame d;
     if ((st = bind_frame(h, f, s, &d, false)) != PILOT_OK) return st;
     PILOT_CUDA(cudaMemcpyAsync(h->Tin, T_cw, sizeof(double) * 12 * M, cudaMemcpyHostToDevice, s), "pose copy");
-    PILOT_CUDA(launch_set_poses(h->state, h->pose32, h->Tin, h->active[0], M, s), "set_poses launch");
     BuildParams b = build_params(h, f, d, level, M, h->active[0]);
-    if ((st = run_build(h, f->feat_dtype, b, s)) != PILOT_OK) return st;
+    const int kind = resident_kind(M, b.n_tiles);
+    if (kind == 0) {
+        PILOT_CUDA(launch_set_poses(h->state, h->pose32, h->Tin, h->active[0], M, s), "set_poses launch");
+        if ((st = run_build(h, f->feat_dtype, b, s)) != PILOT_OK) return st;
+        ++h->total_launches;
+    }
     EpilogueParams ep{};
     ep.state = h->state;
     ep.pose32 = h->pose32;
@@ -924,8 +948,15 @@ pilot_status pilot_align_debug_normal_eq(pilot_align_handle* h, const pilot_fram
     ep.mode = kEpiEval;
     ep.prior = prior_params(h->cfg, f, d);
     ep.eval_out = h->eval_out;
-    PILOT_CUDA(launch_epilogue(ep, h->min_valid, s), "epilogue launch");
-    h->total_launches += 2;
+    if (kind != 0) {
+        b.active_idx = nullptr;
+        const ResidentParams rp{b, ep, nullptr, h->Tin, 0};
+        if ((st = timed_build(h, s, [&]() { return launch_resident(f->feat_dtype, rp, kind == 2, s); })) != PILOT_OK)
+            return st;
+    } else {
+        PILOT_CUDA(launch_epilogue(ep, h->min_valid, s), "epilogue launch");
+        ++h->total_launches;
+    }
     PILOT_CUDA(cudaMemcpyAsync(out29, h->eval_out, sizeof(double) * kNumSums * M, cudaMemcpyDeviceToHost, s),
                "normal-equation copy");
     PILOT_CUDA(cudaStreamSynchronize(s), "debug_normal_eq");

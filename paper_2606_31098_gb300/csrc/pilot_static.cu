@@ -175,9 +175,6 @@ extern "C" pilot_status pilot_align_normal_eq_noalloc(const pilot_align_config* 
     const double huber_grav = cfg->huber_grav == 0.0 ? 0.1 : cfg->huber_grav;
     const double huber_range = cfg->huber_range == 0.0 ? 1.0 : cfg->huber_range;
 
-    cudaError_t e = launch_set_poses(state, pose32, T_cw, active, f->M, s);
-    if (e != cudaSuccess) return fail_msg(PILOT_ECUDA, std::string("set_poses launch: ") + cudaGetErrorString(e));
-
     BuildParams b{};
     const size_t N = (size_t)f->N;
     b.px = f->points;
@@ -210,8 +207,14 @@ extern "C" pilot_status pilot_align_normal_eq_noalloc(const pilot_align_config* 
     b.n_active = f->M;
     b.tile = kStaticTile;
     b.n_tiles = f->N > 0 ? (f->N + kStaticTile - 1) / kStaticTile : 1;
-    e = dispatch(f->feat_dtype, b, s);
-    if (e != cudaSuccess) return fail_msg(PILOT_ECUDA, std::string("build-pass launch: ") + cudaGetErrorString(e));
+    const int kind = resident_kind(f->M, b.n_tiles);
+    cudaError_t e = cudaSuccess;
+    if (kind == 0) {
+        e = launch_set_poses(state, pose32, T_cw, active, f->M, s);
+        if (e != cudaSuccess) return fail_msg(PILOT_ECUDA, std::string("set_poses launch: ") + cudaGetErrorString(e));
+        e = dispatch(f->feat_dtype, b, s);
+        if (e != cudaSuccess) return fail_msg(PILOT_ECUDA, std::string("build-pass launch: ") + cudaGetErrorString(e));
+    }
 
     EpilogueParams ep{};
     ep.state = state;
@@ -247,7 +250,12 @@ extern "C" pilot_status pilot_align_normal_eq_noalloc(const pilot_align_config* 
     pp.gate_grav = cfg->gate_grav;
     pp.gate_range = cfg->gate_range;
     pp.derive();
-    e = launch_epilogue(ep, min_valid, s);
-    if (e != cudaSuccess) return fail_msg(PILOT_ECUDA, std::string("epilogue launch: ") + cudaGetErrorString(e));
+    if (kind != 0) {
+        b.active_idx = nullptr;
+        e = launch_resident(f->feat_dtype, ResidentParams{b, ep, nullptr, T_cw, 0}, kind == 2, s);
+    } else {
+        e = launch_epilogue(ep, min_valid, s);
+    }
+    if (e != cudaSuccess) return fail_msg(PILOT_ECUDA, std::string("evaluation launch: ") + cudaGetErrorString(e));
     return PILOT_OK;
 }
