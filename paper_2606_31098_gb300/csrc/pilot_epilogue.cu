@@ -43,21 +43,66 @@ __global__ void epilogue_kernel(const EpilogueParams p, const double* min_valid_
     lm_step(p, slot, E, min_valid, threadIdx.x);
 }
 
-__global__ void hyp_init_kernel(HypState* st, const double* T_cw, int* active_idx, int M) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+// LM state of hypothesis m at the start of a solve, by one warp.
+__device__ __forceinline__ void init_hyp(HypState& s, const double* T_cw, int lane) {
+    if (lane < 12) s.T[lane] = s.Tc[lane] = T_cw[lane];
+    if (lane < 21) s.H[lane] = 0.0;
+    else if (lane < 27) s.g[lane - 21] = 0.0;
+    if (lane == 0) {
+        s.cost = 0.0;
+        s.lambda = 0.0;
+        s.n_valid = 0;
+        s.has_cand = 0;
+        s.last_fail = 0;
+        s.active = 1;
+        s.status = PILOT_HYP_OK;
+    }
+}
+
+// Number of set flags among N, by the whole block (blockDim.x a multiple of 32, at most 1024; 16
+// flags per load where aligned); on every thread.
+__device__ __forceinline__ int count_flags(const uint8_t* valid, int N) {
+    __shared__ int part[32];
+    int c = 0;
+    const int n16 = ((uintptr_t)valid & 15) == 0 ? N / 16 : 0;
+    const uint4* w = reinterpret_cast<const uint4*>(valid);
+    auto set4 = [](unsigned v) { return ((v & 0xffu) != 0) + ((v & 0xff00u) != 0) + ((v & 0xff0000u) != 0) + ((v >> 24) != 0); };
+#pragma unroll 4
+    for (int k = threadIdx.x; k < n16; k += blockDim.x) {
+        const uint4 v = w[k];
+        c += set4(v.x) + set4(v.y) + set4(v.z) + set4(v.w);
+    }
+    for (int j = n16 * 16 + threadIdx.x; j < N; j += blockDim.x) c += valid[j] != 0;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = c;
+    __syncthreads();
+    c = 0;
+    for (int k = 0; k < (int)blockDim.x / 32; ++k) c += part[k];
+    return c;
+}
+
+// Start of a plain solve: the hypotheses' states, one per warp; the tickets; and, by the last
+// block, the threshold on visible anchors.  One launch for what were three (5.7 + 5.5 us alone at
+// 65536 anchors and 64 hypotheses, 2.8 + 7.7 us at 500 and 1210).
+constexpr int kInitThreads = 256;
+__global__ void __launch_bounds__(kInitThreads)
+solve_init_kernel(HypState* st, const double* T_cw, int* active_idx, int M, unsigned* tickets, unsigned* done_ticket,
+                  const uint8_t* valid, int N, double frac, double* min_valid) {
+    if (blockIdx.x == gridDim.x - 1) {
+        const int c = valid ? count_flags(valid, N) : N;
+        if (threadIdx.x == 0) {
+            *min_valid = frac * (double)c;
+            *done_ticket = 0u;
+        }
+        return;
+    }
+    const int m = blockIdx.x * (kInitThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (m >= M) return;
-    HypState& s = st[m];
-    for (int i = 0; i < 12; ++i) s.T[i] = s.Tc[i] = T_cw[12 * m + i];
-    for (int i = 0; i < 21; ++i) s.H[i] = 0.0;
-    for (int i = 0; i < 6; ++i) s.g[i] = 0.0;
-    s.cost = 0.0;
-    s.lambda = 0.0;
-    s.n_valid = 0;
-    s.has_cand = 0;
-    s.last_fail = 0;
-    s.active = 1;
-    s.status = PILOT_HYP_OK;
-    active_idx[m] = m;
+    init_hyp(st[m], T_cw + 12 * (size_t)m, lane);
+    if (lane == 0) {
+        active_idx[m] = m;
+        tickets[m] = 0u;
+    }
 }
 
 __global__ void set_poses_kernel(HypState* st, float* pose32, const double* T_cw, int* active_idx,
@@ -100,19 +145,22 @@ __device__ __forceinline__ ulonglong2 order_key(int bad, unsigned long long c, i
 }
 
 // Top-K (Supp. "Multi-Hypothesis Refinement") over the n hypotheses listed in act[0, n) of
-// S, in two passes.  rank_mark: each thread of a block takes one listed hypothesis from
-// [s_begin, s_begin + blockDim.x), counts the listed hypotheses that rank before it (keys
-// streamed through shared memory blockDim.x at a time) and marks it pruned if that count is
-// K or more; many blocks share the n^2 comparisons.  compact_active (one block, blockDim.x a
-// multiple of 32, at most 1024, after every rank_mark block has finished): writes the
-// survivors' indices, in their order in act, to act_out[0, K) (act_out may be act) by a
-// block-wide prefix count.
+// S, in two passes.  rank_mark: LANES lanes of a block share one listed hypothesis of
+// [s_begin, s_begin + kRankThreads / LANES), count the listed hypotheses that rank before it (keys
+// streamed through shared memory kRankThreads at a time) and mark it pruned if that count is
+// K or more.  compact_active (one block, blockDim.x a multiple of 32, at most 1024, after every
+// rank_mark block has finished): writes the survivors' indices, in their order in act, to
+// act_out[0, K) (act_out may be act) by a block-wide prefix count.
+// The n^2 comparisons are spread over LANES lanes per hypothesis since five blocks of one thread
+// per hypothesis took 28.6 us for 1210 (alone); a warp each, with the compaction of the survivors (6 us)
+// in the same launch: 16 us.
 constexpr int kRankThreads = 256;
 
+template <int LANES>
 __device__ void rank_mark(HypState* S, const int* act, int n, int K, double min_valid, int s_begin) {
     __shared__ ulonglong2 kk[kRankThreads];      // order keys of the current chunk
-    const int tid = threadIdx.x;
-    const int s = s_begin + tid;
+    const int tid = threadIdx.x, sub = tid % LANES;
+    const int s = s_begin + tid / LANES;
     int m = -1, rank = 0;
     ulonglong2 key = make_ulonglong2(~0ull, ~0ull);
     if (s < n) {
@@ -135,13 +183,15 @@ __device__ void rank_mark(HypState* S, const int* act, int n, int K, double min_
         if (s < n) {
             const int lim = min(kRankThreads, n - c0);
 #pragma unroll 4
-            for (int j = 0; j < lim; ++j) {
+            for (int j = sub; j < lim; j += LANES) {
                 const ulonglong2 o = kk[j];
                 rank += (o.x < key.x) | ((o.x == key.x) & (o.y < key.y));
             }
         }
     }
-    if (s < n && rank >= K) {
+#pragma unroll
+    for (int o = LANES / 2; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    if (s < n && rank >= K && sub == 0) {
         S[m].active = 0;
         S[m].status = PILOT_HYP_PRUNED;
     }
@@ -159,7 +209,7 @@ __device__ void compact_active(const HypState* S, const int* act, int* act_out, 
         bool keep = false;
         if (s < n) {
             m = act[s];
-            keep = S[m].active != 0;
+            keep = __ldcg(&S[m].active) != 0;        // other blocks of the launch may have marked it
         }
         const unsigned bal = __ballot_sync(0xffffffffu, keep);
         if (lane == 0) wsum[warp] = __popc(bal);
@@ -177,208 +227,166 @@ __device__ void compact_active(const HypState* S, const int* act, int* act_out, 
     }
 }
 
-// Plain form: blockIdx.x ranks listed hypotheses [256 blockIdx.x, + 256).
-__global__ void prune_rank_kernel(HypState* st, const int* active_in, int n, int K, const double* min_valid_ptr) {
-    rank_mark(st, active_in, n, K, *min_valid_ptr, blockIdx.x * kRankThreads);
-}
-
-// Plain form: the survivors, in their order in active_in, to active_out.
-__global__ void prune_compact_kernel(const HypState* st, const int* active_in, int* active_out, int n) {
-    compact_active(st, active_in, active_out, n);
-}
-
-// One block of 1024 threads: number of valid anchors (4 flags per load when aligned).
-__global__ void count_valid_kernel(const uint8_t* valid, int N, double frac, double* min_valid) {
-    __shared__ int part[32];
-    int c = 0;
-    if (!valid) {
-        c = (threadIdx.x == 0) ? N : 0;
-    } else if (((uintptr_t)valid & 3) == 0) {
-        const uint32_t* w = reinterpret_cast<const uint32_t*>(valid);
-        for (int k = threadIdx.x; k < N / 4; k += blockDim.x) {
-            const uint32_t v = w[k];
-            c += ((v & 0xffu) != 0) + ((v & 0xff00u) != 0) + ((v & 0xff0000u) != 0) + ((v >> 24) != 0);
-        }
-        for (int j = (N / 4) * 4 + threadIdx.x; j < N; j += blockDim.x) c += valid[j] != 0;
-    } else {
-        for (int j = threadIdx.x; j < N; j += blockDim.x) c += valid[j] != 0;
-    }
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = c;
+// Whether this block is the last of the launch to get here (ticket zero before the launch and left
+// zero); what the other blocks wrote before is then visible.
+__device__ __forceinline__ bool last_block(unsigned* ticket, unsigned blocks) {
+    __shared__ bool last;
+    __threadfence();
     __syncthreads();
-    if (threadIdx.x < 32) {
-        int v = (threadIdx.x < (blockDim.x >> 5)) ? part[threadIdx.x] : 0;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (threadIdx.x == 0) *min_valid = frac * (double)v;
+    if (threadIdx.x == 0) {
+        last = atomicAdd(ticket, 1u) == blocks - 1u;
+        if (last) *ticket = 0u;
     }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
 }
 
-// One block (blockDim.x a power of two, at most 1024): final statuses, result block, argmin
-// (ties -> lowest index).
-__global__ void finalize_kernel(HypState* st, int M, const double* min_valid_ptr,
-                                unsigned char* res, ResultLayout lay) {
-    const double min_valid = *min_valid_ptr;
-    double* T = reinterpret_cast<double*>(res + lay.off_T);
-    double* cost = reinterpret_cast<double*>(res + lay.off_cost);
-    int* nv = reinterpret_cast<int*>(res + lay.off_nvalid);
-    int* status = reinterpret_cast<int*>(res + lay.off_status);
-    int* best = reinterpret_cast<int*>(res + lay.off_best);
-    __shared__ double bc[1024];
-    __shared__ int bi[1024];
-    double my_c = 0.0;
-    int my_i = -1;
-    for (int m = threadIdx.x; m < M; m += blockDim.x) {
-        HypState& s = st[m];
+// Plain form: a warp per listed hypothesis; the last block lists the survivors, in their order
+// in active_in, in active_out.
+constexpr int kPlainRankLanes = 32;
+__global__ void __launch_bounds__(kRankThreads)
+prune_kernel(HypState* st, const int* active_in, int* active_out, int n, int K, const double* min_valid_ptr,
+             unsigned* ticket) {
+    rank_mark<kPlainRankLanes>(st, active_in, n, K, *min_valid_ptr, blockIdx.x * (kRankThreads / kPlainRankLanes));
+    if (last_block(ticket, gridDim.x)) compact_active(st, active_in, active_out, n);
+}
+
+// Final status and outputs of one hypothesis, by one warp (output index o).
+__device__ __forceinline__ void finish_hyp(HypState& s, double min_valid, size_t o, double* T, double* cost, int* nv,
+                                           int* status, int lane) {
+    const double t = lane < 12 ? s.T[lane] : 0.0;
+    const double c = s.cost;
+    const bool finite = __all_sync(0xffffffffu, isfinite(t)) && isfinite(c);
+    if (lane < 12) T[12 * o + lane] = t;
+    if (lane == 0) {
+        int code = s.status;
         if (s.active) {
-            bool finite = isfinite(s.cost);
-            for (int i = 0; i < 12; ++i) finite = finite && isfinite(s.T[i]);
-            int code;
             if (!finite) code = PILOT_HYP_NONFINITE;
             else if (s.n_valid < min_valid) code = PILOT_HYP_FEW_VALID;
             else if (s.last_fail) code = PILOT_HYP_NOT_PD;
             else code = PILOT_HYP_OK;
             s.status = code;
         }
-        for (int i = 0; i < 12; ++i) T[12 * m + i] = s.T[i];
-        cost[m] = s.cost;
-        nv[m] = s.n_valid;
-        status[m] = s.status;
-        if (s.status == PILOT_HYP_OK && (my_i < 0 || s.cost < my_c)) {
-            my_c = s.cost;
+        cost[o] = c;
+        nv[o] = s.n_valid;
+        status[o] = code;
+    }
+}
+
+// Index of the lowest cost among M hypotheses with status OK (ties: the lowest index), or -1; by
+// the whole block of kFinishThreads, on thread 0.  Outputs other blocks wrote are read from L2.
+constexpr int kFinishThreads = 256;
+__device__ __forceinline__ int best_of(const double* cost, const int* status, int M) {
+    __shared__ double bc[kFinishThreads];
+    __shared__ int bi[kFinishThreads];
+    const int tid = threadIdx.x;
+    double my_c = 0.0;
+    int my_i = -1;
+    for (int m = tid; m < M; m += kFinishThreads) {
+        const double c = __ldcg(cost + m);
+        if (__ldcg(status + m) == PILOT_HYP_OK && (my_i < 0 || c < my_c)) {
+            my_c = c;
             my_i = m;
         }
     }
-    bc[threadIdx.x] = my_c;
-    bi[threadIdx.x] = my_i;
+    bc[tid] = my_c;
+    bi[tid] = my_i;
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
-            const int j = threadIdx.x + s;
+    for (int s = kFinishThreads / 2; s > 0; s >>= 1) {
+        if (tid < s) {
+            const int j = tid + s;
             const bool take = bi[j] >= 0 &&
-                              (bi[threadIdx.x] < 0 || bc[j] < bc[threadIdx.x] ||
-                               (bc[j] == bc[threadIdx.x] && bi[j] < bi[threadIdx.x]));
+                              (bi[tid] < 0 || bc[j] < bc[tid] || (bc[j] == bc[tid] && bi[j] < bi[tid]));
             if (take) {
-                bc[threadIdx.x] = bc[j];
-                bi[threadIdx.x] = bi[j];
+                bc[tid] = bc[j];
+                bi[tid] = bi[j];
             }
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) *best = bi[0];
+    return bi[0];
+}
+
+// Plain form: statuses and the result block, one hypothesis per warp; the last block selects.  One
+// block of a thread per hypothesis, each reading its 560-byte state alone, took 26.7 us for
+// 1210 hypotheses (alone); now 8.0 us.
+__global__ void __launch_bounds__(kFinishThreads)
+finalize_kernel(HypState* st, int M, const double* min_valid_ptr, unsigned char* res, ResultLayout lay, unsigned* ticket) {
+    double* cost = reinterpret_cast<double*>(res + lay.off_cost);
+    int* status = reinterpret_cast<int*>(res + lay.off_status);
+    const int m = blockIdx.x * (kFinishThreads / 32) + (threadIdx.x >> 5);
+    if (m < M)
+        finish_hyp(st[m], *min_valid_ptr, m, reinterpret_cast<double*>(res + lay.off_T), cost,
+                   reinterpret_cast<int*>(res + lay.off_nvalid), status, threadIdx.x & 31);
+    if (!last_block(ticket, gridDim.x)) return;
+    const int best = best_of(cost, status, M);
+    if (threadIdx.x == 0) *reinterpret_cast<int*>(res + lay.off_best) = best;
 }
 
 // ---- batched form and serving rounds: one block per frame ----
 
-__device__ void init_frame(const FrameDesc& f, HypState* st, int* active) {
-    for (int m = threadIdx.x; m < f.M; m += blockDim.x) {
-        HypState& s = st[f.hyp_offset + m];
-        for (int i = 0; i < 12; ++i) s.T[i] = s.Tc[i] = f.T_cw[12 * m + i];
-        for (int i = 0; i < 21; ++i) s.H[i] = 0.0;
-        for (int i = 0; i < 6; ++i) s.g[i] = 0.0;
-        s.cost = 0.0;
-        s.lambda = 0.0;
-        s.n_valid = 0;
-        s.has_cand = 0;
-        s.last_fail = 0;
-        s.active = 1;
-        s.status = PILOT_HYP_OK;
-        active[f.hyp_offset + m] = m;
+// The hypotheses of one frame from the first-th on, one per warp, every stride-th.
+__device__ void init_frame(const FrameDesc& f, HypState* st, int* active, int first, int stride) {
+    const int lane = threadIdx.x & 31;
+    for (int m = first; m < f.M; m += stride) {
+        init_hyp(st[f.hyp_offset + m], f.T_cw + 12 * (size_t)m, lane);
+        if (lane == 0) active[f.hyp_offset + m] = m;
     }
 }
 
-// min_valid of one frame (block-wide; blockDim.x a multiple of 32, <= 1024)
-__device__ void count_frame(const FrameDesc& f, double frac, double* min_valid) {
-    __shared__ int part[32];
-    int c = 0;
-    for (int j = threadIdx.x; j < f.N; j += blockDim.x) c += f.valid ? (f.valid[j] != 0) : 1;
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = c;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        int v = (threadIdx.x < (blockDim.x >> 5)) ? part[threadIdx.x] : 0;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (threadIdx.x == 0) *min_valid = frac * (double)v;
-    }
-    __syncthreads();
-}
-
-// Statuses, per-hypothesis outputs (at the global hypothesis index) and the argmin of
-// one frame.  blockDim.x <= 1024, a power of two.
-__device__ void finalize_frame(const FrameDesc& f, int fi, HypState* st, double mv,
-                               unsigned char* res, int max_hyps) {
+// Statuses and outputs (at the global hypothesis index) of one frame's hypotheses from the first-th
+// on, one per warp, every stride-th.
+__device__ void finish_frame(const FrameDesc& f, HypState* st, double mv, unsigned char* res, int max_hyps, int first,
+                             int stride) {
     const ResultLayout lay = ResultLayout::make(max_hyps);
-    double* T = reinterpret_cast<double*>(res + lay.off_T);
-    double* cost = reinterpret_cast<double*>(res + lay.off_cost);
-    int* nv = reinterpret_cast<int*>(res + lay.off_nvalid);
-    int* status = reinterpret_cast<int*>(res + lay.off_status);
-    int* best = reinterpret_cast<int*>(res + lay.bytes);      // one int per frame after the block
-    __shared__ double bc[1024];
-    __shared__ int bi[1024];
-    double my_c = 0.0;
-    int my_i = -1;
-    for (int m = threadIdx.x; m < f.M; m += blockDim.x) {
-        const int g = f.hyp_offset + m;
-        HypState& s = st[g];
-        if (s.active) {
-            bool finite = isfinite(s.cost);
-            for (int i = 0; i < 12; ++i) finite = finite && isfinite(s.T[i]);
-            int code;
-            if (!finite) code = PILOT_HYP_NONFINITE;
-            else if (s.n_valid < mv) code = PILOT_HYP_FEW_VALID;
-            else if (s.last_fail) code = PILOT_HYP_NOT_PD;
-            else code = PILOT_HYP_OK;
-            s.status = code;
+    for (int m = first; m < f.M; m += stride)
+        finish_hyp(st[f.hyp_offset + m], mv, (size_t)f.hyp_offset + m, reinterpret_cast<double*>(res + lay.off_T),
+                   reinterpret_cast<double*>(res + lay.off_cost), reinterpret_cast<int*>(res + lay.off_nvalid),
+                   reinterpret_cast<int*>(res + lay.off_status), threadIdx.x & 31);
+}
+
+// The selection of one frame whose outputs are written.
+__device__ void select_frame(const FrameDesc& f, int fi, unsigned char* res, int max_hyps) {
+    const ResultLayout lay = ResultLayout::make(max_hyps);
+    const int best = best_of(reinterpret_cast<double*>(res + lay.off_cost) + f.hyp_offset,
+                             reinterpret_cast<int*>(res + lay.off_status) + f.hyp_offset, f.M);
+    if (threadIdx.x == 0) reinterpret_cast<int*>(res + lay.bytes)[fi] = best;     // one int per frame after the block
+}
+
+// Blocks of kInitThreads / kFinishThreads per frame (blockIdx.y) for its set-up and its results:
+// with one block per frame, 1210 hypotheses took 54 us to set up and 28.6 us to finish (alone).
+constexpr int kFrameBlocks = 16;
+
+__global__ void __launch_bounds__(kInitThreads)
+batch_init_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st, int* active, double frac,
+                  double* min_valid, unsigned* tickets) {
+    const int fi = blockIdx.x;
+    if (fi >= hdr->n_frames) return;
+    const FrameDesc& f = frames[fi];
+    if (blockIdx.y == kFrameBlocks) {
+        const int c = f.valid ? count_flags(f.valid, f.N) : f.N;
+        if (threadIdx.x == 0) {
+            min_valid[fi] = frac * (double)c;
+            tickets[fi] = 0u;
         }
-        for (int i = 0; i < 12; ++i) T[12 * (size_t)g + i] = s.T[i];
-        cost[g] = s.cost;
-        nv[g] = s.n_valid;
-        status[g] = s.status;
-        if (s.status == PILOT_HYP_OK && (my_i < 0 || s.cost < my_c)) {
-            my_c = s.cost;
-            my_i = m;
-        }
+        return;
     }
-    bc[threadIdx.x] = my_c;
-    bi[threadIdx.x] = my_i;
-    __syncthreads();
-    for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-        if ((int)threadIdx.x < k) {
-            const int j = threadIdx.x + k;
-            const bool take = bi[j] >= 0 &&
-                              (bi[threadIdx.x] < 0 || bc[j] < bc[threadIdx.x] ||
-                               (bc[j] == bc[threadIdx.x] && bi[j] < bi[threadIdx.x]));
-            if (take) {
-                bc[threadIdx.x] = bc[j];
-                bi[threadIdx.x] = bi[j];
-            }
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) best[fi] = bi[0];
+    init_frame(f, st, active, blockIdx.y * (kInitThreads / 32) + (threadIdx.x >> 5), kFrameBlocks * (kInitThreads / 32));
 }
 
-__global__ void batch_init_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
-                                  int* active) {
-    if ((int)blockIdx.x >= hdr->n_frames) return;
-    init_frame(frames[blockIdx.x], st, active);
-}
+constexpr int kRankLanes = 8, kRankHyps = kRankThreads / kRankLanes;   // batched and served forms
 
-__global__ void batch_count_valid_kernel(const BatchHeader* hdr, const FrameDesc* frames, double frac,
-                                         double* min_valid) {
-    if ((int)blockIdx.x >= hdr->n_frames) return;
-    count_frame(frames[blockIdx.x], frac, min_valid + blockIdx.x);
-}
-
-// Batched form, top-K after a level: blockIdx.x is the frame, blockIdx.y a block of 256 of
+// Batched form, top-K after a level: blockIdx.x is the frame, blockIdx.y a block of kRankHyps of
 // its listed hypotheses (frames whose count is at most K keep all of them).
 __global__ void batch_rank_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                                   const int* active, const int* n_active, int K, const double* min_valid) {
     const int fi = blockIdx.x;
     if (fi >= hdr->n_frames) return;
     const int n = n_active[fi];
-    if (K <= 0 || K >= n || (int)blockIdx.y * kRankThreads >= n) return;
+    if (K <= 0 || K >= n || (int)blockIdx.y * kRankHyps >= n) return;
     const FrameDesc& f = frames[fi];
-    rank_mark(st + f.hyp_offset, active + f.hyp_offset, n, K, min_valid[fi], blockIdx.y * kRankThreads);
+    rank_mark<kRankLanes>(st + f.hyp_offset, active + f.hyp_offset, n, K, min_valid[fi], blockIdx.y * kRankHyps);
 }
 
 // Batched form: each pruned frame's active list compacted in place.
@@ -392,21 +400,26 @@ __global__ void batch_compact_kernel(const BatchHeader* hdr, const FrameDesc* fr
     compact_active(st + f.hyp_offset, active + f.hyp_offset, active + f.hyp_offset, n);
 }
 
-__global__ void batch_finalize_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
-                                      const double* min_valid, unsigned char* res, int max_hyps) {
+__global__ void __launch_bounds__(kFinishThreads)
+batch_finalize_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st, const double* min_valid,
+                      unsigned char* res, int max_hyps, unsigned* tickets) {
     const int fi = blockIdx.x;
     if (fi >= hdr->n_frames) return;
-    finalize_frame(frames[fi], fi, st, min_valid[fi], res, max_hyps);
+    finish_frame(frames[fi], st, min_valid[fi], res, max_hyps, blockIdx.y * (kFinishThreads / 32) + (threadIdx.x >> 5),
+                 kFrameBlocks * (kFinishThreads / 32));
+    if (last_block(tickets + fi, kFrameBlocks)) select_frame(frames[fi], fi, res, max_hyps);
 }
 
-__global__ void round_prepare_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
-                                     int* active, double frac, double* min_valid) {
+__global__ void __launch_bounds__(kInitThreads)
+round_prepare_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st, int* active, double frac,
+                     double* min_valid) {
     const int fi = blockIdx.x;
     if (fi >= hdr->n_frames) return;
     const FrameDesc& f = frames[fi];
     if (!(f.flags & kFlagInit)) return;
-    init_frame(f, st, active);
-    count_frame(f, frac, min_valid + fi);
+    init_frame(f, st, active, threadIdx.x >> 5, kInitThreads / 32);
+    const int c = f.valid ? count_flags(f.valid, f.N) : f.N;
+    if (threadIdx.x == 0) min_valid[fi] = frac * (double)c;
 }
 
 // Serving round, top-K of the frames that finished a pruning level (as batch_rank_kernel).
@@ -415,11 +428,13 @@ __global__ void round_rank_kernel(const BatchHeader* hdr, const FrameDesc* frame
     const int fi = blockIdx.x;
     if (fi >= hdr->n_frames) return;
     const FrameDesc& f = frames[fi];
-    if (!(f.flags & kFlagPrune) || (int)blockIdx.y * kRankThreads >= f.n_active) return;
-    rank_mark(st + f.hyp_offset, active + f.hyp_offset, f.n_active, f.keep, min_valid[fi], blockIdx.y * kRankThreads);
+    if (!(f.flags & kFlagPrune) || (int)blockIdx.y * kRankHyps >= f.n_active) return;
+    rank_mark<kRankLanes>(st + f.hyp_offset, active + f.hyp_offset, f.n_active, f.keep, min_valid[fi],
+                          blockIdx.y * kRankHyps);
 }
 
-__global__ void round_finish_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
+__global__ void __launch_bounds__(kFinishThreads)
+round_finish_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                                     int* active, const double* min_valid, unsigned char* res,
                                     int max_hyps) {
     const int fi = blockIdx.x;
@@ -427,7 +442,12 @@ __global__ void round_finish_kernel(const BatchHeader* hdr, const FrameDesc* fra
     const FrameDesc& f = frames[fi];
     if (f.flags & kFlagPrune)
         compact_active(st + f.hyp_offset, active + f.hyp_offset, active + f.hyp_offset, f.n_active);
-    if (f.flags & kFlagFinalize) finalize_frame(f, fi, st, min_valid[fi], res, max_hyps);
+    if (f.flags & kFlagFinalize) {
+        finish_frame(f, st, min_valid[fi], res, max_hyps, threadIdx.x >> 5, kFinishThreads / 32);
+        __threadfence();
+        __syncthreads();
+        select_frame(f, fi, res, max_hyps);
+    }
 }
 
 // Serving round with several levels: after a level's finish, every listed frame moves on to
@@ -479,21 +499,17 @@ cudaError_t launch_round_advance(const BatchHeader* hdr, FrameDesc* frames, cons
 }
 
 cudaError_t launch_batch_init(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
-                              int* active, int max_frames, cudaStream_t s) {
-    batch_init_kernel<<<max_frames, 128, 0, s>>>(hdr, frames, st, active);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_batch_count_valid(const BatchHeader* hdr, const FrameDesc* frames, double frac,
-                                     double* min_valid, int max_frames, cudaStream_t s) {
-    batch_count_valid_kernel<<<max_frames, 1024, 0, s>>>(hdr, frames, frac, min_valid);
+                              int* active, double frac, double* min_valid, unsigned* tickets, int max_frames,
+                              cudaStream_t s) {
+    batch_init_kernel<<<dim3(max_frames, kFrameBlocks + 1), kInitThreads, 0, s>>>(hdr, frames, st, active, frac, min_valid,
+                                                                                  tickets);
     return cudaGetLastError();
 }
 
 cudaError_t launch_batch_prune(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                                int* active, const int* n_active, int keep, const double* min_valid,
                                int max_frames, int max_frame_hyps, cudaStream_t s) {
-    const dim3 grid(max_frames, (max_frame_hyps + kRankThreads - 1) / kRankThreads);
+    const dim3 grid(max_frames, (max_frame_hyps + kRankHyps - 1) / kRankHyps);
     batch_rank_kernel<<<grid, kRankThreads, 0, s>>>(hdr, frames, st, active, n_active, keep, min_valid);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -503,26 +519,27 @@ cudaError_t launch_batch_prune(const BatchHeader* hdr, const FrameDesc* frames, 
 
 cudaError_t launch_batch_finalize(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                                   const double* min_valid, unsigned char* result, int max_hyps,
-                                  int max_frames, cudaStream_t s) {
-    batch_finalize_kernel<<<max_frames, 1024, 0, s>>>(hdr, frames, st, min_valid, result, max_hyps);
+                                  unsigned* tickets, int max_frames, cudaStream_t s) {
+    batch_finalize_kernel<<<dim3(max_frames, kFrameBlocks), kFinishThreads, 0, s>>>(hdr, frames, st, min_valid, result,
+                                                                                    max_hyps, tickets);
     return cudaGetLastError();
 }
 
 cudaError_t launch_round_prepare(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                                  int* active, double frac, double* min_valid, int max_frames,
                                  cudaStream_t s) {
-    round_prepare_kernel<<<max_frames, 1024, 0, s>>>(hdr, frames, st, active, frac, min_valid);
+    round_prepare_kernel<<<max_frames, kInitThreads, 0, s>>>(hdr, frames, st, active, frac, min_valid);
     return cudaGetLastError();
 }
 
 cudaError_t launch_round_finish(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                                 int* active, const double* min_valid, unsigned char* result,
                                 int max_hyps, int max_frames, int max_frame_hyps, cudaStream_t s) {
-    const dim3 grid(max_frames, (max_frame_hyps + kRankThreads - 1) / kRankThreads);
+    const dim3 grid(max_frames, (max_frame_hyps + kRankHyps - 1) / kRankHyps);
     round_rank_kernel<<<grid, kRankThreads, 0, s>>>(hdr, frames, st, active, min_valid);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    round_finish_kernel<<<max_frames, 1024, 0, s>>>(hdr, frames, st, active, min_valid, result, max_hyps);
+    round_finish_kernel<<<max_frames, kFinishThreads, 0, s>>>(hdr, frames, st, active, min_valid, result, max_hyps);
     return cudaGetLastError();
 }
 
@@ -532,10 +549,11 @@ cudaError_t launch_epilogue(const EpilogueParams& p, const double* min_valid, cu
     return cudaGetLastError();
 }
 
-cudaError_t launch_hyp_init(HypState* st, const double* T_cw, int* active_idx, int M,
-                            cudaStream_t s) {
-    if (M <= 0) return cudaSuccess;
-    hyp_init_kernel<<<(M + 127) / 128, 128, 0, s>>>(st, T_cw, active_idx, M);
+cudaError_t launch_solve_init(HypState* st, const double* T_cw, int* active_idx, int M, unsigned* tickets,
+                              unsigned* done_ticket, const uint8_t* valid, int N, double frac, double* min_valid,
+                              cudaStream_t s) {
+    solve_init_kernel<<<(M + kInitThreads / 32 - 1) / (kInitThreads / 32) + 1, kInitThreads, 0, s>>>(
+        st, T_cw, active_idx, M, tickets, done_ticket, valid, N, frac, min_valid);
     return cudaGetLastError();
 }
 
@@ -554,25 +572,18 @@ cudaError_t launch_level_init(HypState* st, float* pose32, const int* active_idx
 }
 
 cudaError_t launch_prune(HypState* st, const int* active_in, int* active_out, int n_active,
-                         int keep, const double* min_valid, cudaStream_t s) {
+                         int keep, const double* min_valid, unsigned* ticket, cudaStream_t s) {
     if (n_active <= 0) return cudaSuccess;
-    prune_rank_kernel<<<(n_active + kRankThreads - 1) / kRankThreads, kRankThreads, 0, s>>>(st, active_in, n_active,
-                                                                                            keep, min_valid);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    prune_compact_kernel<<<1, 1024, 0, s>>>(st, active_in, active_out, n_active);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_count_valid(const uint8_t* valid, int N, double frac, double* min_valid,
-                               cudaStream_t s) {
-    count_valid_kernel<<<1, 1024, 0, s>>>(valid, N, frac, min_valid);
+    constexpr int per_block = kRankThreads / kPlainRankLanes;
+    prune_kernel<<<(n_active + per_block - 1) / per_block, kRankThreads, 0, s>>>(st, active_in, active_out, n_active, keep,
+                                                                                min_valid, ticket);
     return cudaGetLastError();
 }
 
 cudaError_t launch_finalize(HypState* st, int M, const double* min_valid, unsigned char* result,
-                            ResultLayout lay, cudaStream_t s) {
-    finalize_kernel<<<1, 1024, 0, s>>>(st, M, min_valid, result, lay);
+                            ResultLayout lay, unsigned* ticket, cudaStream_t s) {
+    constexpr int per_block = kFinishThreads / 32;
+    finalize_kernel<<<(M + per_block - 1) / per_block, kFinishThreads, 0, s>>>(st, M, min_valid, result, lay, ticket);
     return cudaGetLastError();
 }
 

@@ -268,16 +268,17 @@ struct ResultLayout {
 cudaError_t launch_epilogue(const EpilogueParams& p, const double* min_valid, cudaStream_t s);
 cudaError_t launch_level_init(HypState* st, float* pose32, const int* active_idx, int n_active,
                               double lambda0, cudaStream_t s);
-cudaError_t launch_hyp_init(HypState* st, const double* T_cw, int* active_idx, int M,
-                            cudaStream_t s);
+// Start of a plain solve: states, active list, tickets (M, and done_ticket), visibility threshold.
+cudaError_t launch_solve_init(HypState* st, const double* T_cw, int* active_idx, int M, unsigned* tickets,
+                              unsigned* done_ticket, const uint8_t* valid, int N, double frac, double* min_valid,
+                              cudaStream_t s);
 cudaError_t launch_set_poses(HypState* st, float* pose32, const double* T_cw, int* active_idx,
                              int M, cudaStream_t s);
+// ticket: one word, zero before the launch and after it
 cudaError_t launch_prune(HypState* st, const int* active_in, int* active_out, int n_active,
-                         int keep, const double* min_valid, cudaStream_t s);
-cudaError_t launch_count_valid(const uint8_t* valid, int N, double frac, double* min_valid,
-                               cudaStream_t s);
+                         int keep, const double* min_valid, unsigned* ticket, cudaStream_t s);
 cudaError_t launch_finalize(HypState* st, int M, const double* min_valid, unsigned char* result,
-                            ResultLayout lay, cudaStream_t s);
+                            ResultLayout lay, unsigned* ticket, cudaStream_t s);
 
 template <pilot_dtype DT>
 cudaError_t launch_build_dtype(const BuildParams& p, cudaStream_t s);
@@ -294,17 +295,17 @@ cudaError_t launch_level_persistent_dtype(int C, int variant, const LevelArgs& a
 template <pilot_dtype DT>
 cudaError_t level_persistent_occupancy(int C, int variant, int* ctas_per_sm);
 
-// batch bookkeeping (one block per frame; frames beyond header->n_frames return)
+// batch bookkeeping (frames beyond header->n_frames return); tickets: a word per frame, reset by the
+// first for the last
 cudaError_t launch_batch_init(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
-                              int* active, int max_frames, cudaStream_t s);
-cudaError_t launch_batch_count_valid(const BatchHeader* hdr, const FrameDesc* frames, double frac,
-                                     double* min_valid, int max_frames, cudaStream_t s);
+                              int* active, double frac, double* min_valid, unsigned* tickets, int max_frames,
+                              cudaStream_t s);
 cudaError_t launch_batch_prune(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                                int* active, const int* n_active, int keep, const double* min_valid,
                                int max_frames, int max_frame_hyps, cudaStream_t s);
 cudaError_t launch_batch_finalize(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                                   const double* min_valid, unsigned char* result, int max_hyps,
-                                  int max_frames, cudaStream_t s);
+                                  unsigned* tickets, int max_frames, cudaStream_t s);
 // serving rounds: the same steps, each frame doing only what its flags ask for
 struct LevelKeep {
     int k[PILOT_MAX_LEVELS];   // keep_top_k per level

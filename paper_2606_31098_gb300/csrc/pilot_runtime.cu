@@ -2,8 +2,9 @@
 // input staging, and the per-level launch sequence of the LM solve.
 //
 // One solve of one frame (Sec. IV-E, Eq. 7-9), all on the caller's stream:
-//   count_valid  (min_valid = frac x valid anchors)    hyp_init (FP64 state from T_cw)
+//   solve_init   (min_valid = frac x valid anchors, FP64 state from T_cw)
 //   for l = L-1 .. 0:
+//     a small level: one launch (level_resident_kernel, level_spread_kernel); else
 //     level_init (lambda = lambda0, candidate = T)
 //     build(l) with the FP64 step fused (init: store E(T), solve the first candidate)
 //     repeat iters[l] times: build(l) at the candidates, fused step (accept or reject,
@@ -186,6 +187,7 @@ struct pilot_align_handle {
     size_t bres_bytes = 0;
     int* bactive = nullptr;
     double* bmin_valid = nullptr;
+    unsigned* btickets = nullptr;          // one per frame
     unsigned long long* bsync = nullptr;   // per level: item claims, barrier arrivals, generations
     unsigned* bjob_meta = nullptr;         // per job of a level launch: hypothesis | evaluate bit
     unsigned* bflags = nullptr;            // level kernel's per-job-tile flags: completed items, then published iterations
@@ -481,6 +483,7 @@ void release(pilot_align_handle* h) {
     if (h->bres_host) cudaFreeHost(h->bres_host);
     cudaFree(h->bactive);
     cudaFree(h->bmin_valid);
+    cudaFree(h->btickets);
     cudaFree(h->bsync);
     cudaFree(h->bjob_meta);
     cudaFree(h->bflags);
@@ -559,6 +562,7 @@ pilot_status batch_alloc(pilot_align_handle* h) {
     PILOT_CUDA(cudaMallocHost((void**)&h->bres_host, h->bres_bytes), "batch result staging");
     PILOT_CUDA(cudaMalloc((void**)&h->bactive, sizeof(int) * (size_t)c.max_hyps), "batch active lists");
     PILOT_CUDA(cudaMalloc((void**)&h->bmin_valid, sizeof(double) * (size_t)c.max_frames), "batch thresholds");
+    PILOT_CUDA(cudaMalloc((void**)&h->btickets, sizeof(unsigned) * (size_t)c.max_frames), "batch tickets");
     PILOT_CUDA(cudaMalloc((void**)&h->bsync, sizeof(unsigned long long) * kSyncWords * PILOT_MAX_LEVELS),
                "batch level counters");
     PILOT_CUDA(cudaMalloc((void**)&h->bjob_meta, sizeof(unsigned) * (size_t)c.max_hyps), "batch job table");
@@ -649,9 +653,8 @@ pilot_status capture_batch_graph(pilot_align_handle* h, pilot_dtype dt, int C, i
     if (e == cudaSuccess)
         e = cudaMemsetAsync(h->bsync, 0, sizeof(unsigned long long) * kSyncWords * PILOT_MAX_LEVELS, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(error, 0, sizeof(unsigned), s);
-    if (e == cudaSuccess) e = launch_batch_init(hdr, frames, h->state, h->bactive, c.max_frames, s);
     if (e == cudaSuccess)
-        e = launch_batch_count_valid(hdr, frames, c.min_valid_frac, h->bmin_valid, c.max_frames, s);
+        e = launch_batch_init(hdr, frames, h->state, h->bactive, c.min_valid_frac, h->bmin_valid, h->btickets, c.max_frames, s);
     for (int level = L - 1; level >= 0 && e == cudaSuccess; --level) {
         LevelArgs a{};
         a.header = hdr;
@@ -696,7 +699,7 @@ pilot_status capture_batch_graph(pilot_align_handle* h, pilot_dtype dt, int C, i
                                    h->bmin_valid, c.max_frames, std::min(c.max_hyps, kMaxFrameHyps), s);
     }
     if (e == cudaSuccess)
-        e = launch_batch_finalize(hdr, frames, h->state, h->bmin_valid, h->bres_dev, c.max_hyps, c.max_frames, s);
+        e = launch_batch_finalize(hdr, frames, h->state, h->bmin_valid, h->bres_dev, c.max_hyps, h->btickets, c.max_frames, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->bres_host, h->bres_dev, h->bres_bytes, cudaMemcpyDeviceToHost, s);
     cudaGraph_t g = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(s, &g);
@@ -759,7 +762,7 @@ pilot_status pilot_align_create(const pilot_align_config* cfg_in, pilot_align_ha
     ALLOC(h->Tin, sizeof(double) * 12 * M);
     ALLOC(h->eval_out, sizeof(double) * kNumSums * M);
     ALLOC(h->min_valid, sizeof(double));
-    ALLOC(h->tickets, sizeof(unsigned) * M);
+    ALLOC(h->tickets, sizeof(unsigned) * (M + 1));     // one per hypothesis (tile), then one per launch
     ALLOC(h->ones, sizeof(float) * cfg.max_channels);
     ALLOC(h->res_dev, lay.bytes);
 #undef ALLOC
@@ -768,7 +771,7 @@ pilot_status pilot_align_create(const pilot_align_config* cfg_in, pilot_align_ha
         return cuda_fail(e, "pinned result buffer");
     }
     if ((e = cudaMemcpy(h->ones, ones.data(), sizeof(float) * cfg.max_channels, cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (e = cudaMemset(h->tickets, 0, sizeof(unsigned) * M)) != cudaSuccess) {
+        (e = cudaMemset(h->tickets, 0, sizeof(unsigned) * (M + 1))) != cudaSuccess) {
         release(h);
         return cuda_fail(e, "workspace init");
     }
@@ -810,10 +813,10 @@ pilot_status pilot_align_solve(pilot_align_handle* h, const pilot_frame* f, pilo
     if ((st = bind_frame(h, f, s, &d, true, overlap ? h->cstream : nullptr, h->level_ready)) != PILOT_OK) return st;
     const int M = f->M;
 
-    PILOT_CUDA(cudaMemsetAsync(h->tickets, 0, sizeof(unsigned) * M, s), "ticket reset");
-    PILOT_CUDA(launch_count_valid(d.valid, f->N, c.min_valid_frac, h->min_valid, s), "count_valid launch");
-    PILOT_CUDA(launch_hyp_init(h->state, d.T, h->active[0], M, s), "hyp_init launch");
-    h->total_launches += 2;
+    unsigned* const done_ticket = h->tickets + c.max_hyps;
+    PILOT_CUDA(launch_solve_init(h->state, d.T, h->active[0], M, h->tickets, done_ticket, d.valid, f->N, c.min_valid_frac,
+                                 h->min_valid, s), "solve_init launch");
+    ++h->total_launches;
     int cur = 0, n_active = M;
     const PriorParams prior = prior_params(c, f, d);
 
@@ -885,15 +888,15 @@ pilot_status pilot_align_solve(pilot_align_handle* h, const pilot_frame* f, pilo
         hyp_iters += (long long)n_active * iters;
         const int K = c.keep_top_k[level];
         if (level > 0 && K > 0 && K < n_active) {
-            PILOT_CUDA(launch_prune(h->state, h->active[cur], h->active[cur ^ 1], n_active, K, h->min_valid, s),
-                       "prune launch");
+            PILOT_CUDA(launch_prune(h->state, h->active[cur], h->active[cur ^ 1], n_active, K, h->min_valid,
+                                    done_ticket, s), "prune launch");
             ++h->total_launches;
             cur ^= 1;
             n_active = K;
         }
     }
     const ResultLayout lay = ResultLayout::make(M);
-    PILOT_CUDA(launch_finalize(h->state, M, h->min_valid, h->res_dev, lay, s), "finalize launch");
+    PILOT_CUDA(launch_finalize(h->state, M, h->min_valid, h->res_dev, lay, done_ticket, s), "finalize launch");
     ++h->total_launches;
     PILOT_CUDA(cudaMemcpyAsync(h->res_host, h->res_dev, lay.bytes, cudaMemcpyDeviceToHost, s), "result copy");
     PILOT_CUDA(cudaStreamSynchronize(s), "solve");
@@ -1176,7 +1179,7 @@ pilot_status pilot_align_solve_batch(pilot_align_handle* h, const pilot_frame* f
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     PILOT_CUDA(cudaGraphLaunch(h->gexec, s), "batch graph launch");
     PILOT_CUDA(cudaStreamSynchronize(s), "batch solve");
-    h->total_launches = 4 + 2 * L + 1;
+    h->total_launches = 3 + 2 * L + 1;
     const ResultLayout rl = ResultLayout::make(c.max_hyps);
     const unsigned char* r = h->bres_host;
     const int* best = reinterpret_cast<const int*>(r + rl.bytes);
