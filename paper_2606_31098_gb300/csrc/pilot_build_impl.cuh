@@ -101,44 +101,6 @@ __device__ __forceinline__ void raw_pair(const RawVec<DT, W>& v, int e, float& l
     }
 }
 
-// Loaded and widened to FP32.
-template <pilot_dtype DT, int W>
-__device__ __forceinline__ void load_vec(const typename Storage<DT>::T* p, float* out) {
-    RawVec<DT, W> v;
-    load_raw<DT, W>(p, v);
-#pragma unroll
-    for (int e = 0; e < W; e += 2) raw_pair<DT, W>(v, e, out[e], out[e + 1]);
-}
-
-struct ChanSums {
-    float s, m00, m01, m11, b0, b1;
-};
-
-// One channel: bilinear value and in-cell gradient, residual, and the six sums.
-template <bool SCALED>
-__device__ __forceinline__ void channel(ChanSums& a, float t00, float t01, float t10, float t11,
-                                        float fr, float ax, float ay, float sq, float sr) {
-    const float bq = t01 - t00;              // d/dx along the upper row
-    const float cq = t10 - t00;              // d/dy along the left column
-    const float dq = (t11 - t10) - bq;       // bilinear cross term
-    float fu = fmaf(dq, ay, bq);             // df/du inside the cell
-    float fv = fmaf(dq, ax, cq);             // df/dv inside the cell
-    float f = fmaf(ax, fu, fmaf(ay, cq, t00));
-    if constexpr (SCALED) {
-        f *= sq;
-        fu *= sq;
-        fv *= sq;
-        fr *= sr;
-    }
-    const float r = f - fr;
-    a.s = fmaf(r, r, a.s);
-    a.m00 = fmaf(fu, fu, a.m00);
-    a.m01 = fmaf(fu, fv, a.m01);
-    a.m11 = fmaf(fv, fv, a.m11);
-    a.b0 = fmaf(fu, r, a.b0);
-    a.b1 = fmaf(fv, r, a.b1);
-}
-
 // ---- two channels per instruction: packed FP32x2 arithmetic (each lane of the pair is
 // rounded exactly like the scalar operation) ----
 typedef unsigned long long f2;
@@ -246,33 +208,55 @@ __device__ __forceinline__ LevelView level_view(const BuildParams& p) {
                      p.H, p.W, p.fx, p.fy, p.cx, p.cy, p.huber};
 }
 
-// Channel sums of one record over this lane's channels (vector k covers VW (q + k LP) ..
-// + VW): the 4 taps at t00 (row below at t00 + WC) against the reference values rr (already
-// loaded, shared by the two hypotheses of an anchor): bilinear value and in-cell gradient,
-// residual, and the six partial sums.
-template <pilot_dtype DT, int C, bool SCALED>
-__device__ __forceinline__ void record_partials(const typename Storage<DT>::T* t00, int WC, const float* rr,
-                                                float ax, float ay, int q, const float* qs, const float* rs,
-                                                float* p) {
+// The 4 taps of one record in this lane's channels (vector k covers VW (q + k LP) .. + VW).
+template <pilot_dtype DT, int C, bool SCALED> struct TapBuf {
     using G = GroupShape<DT, C, SCALED>;
-    constexpr int VW = G::VW, LP = G::LP, NV = G::NV;
-    const typename Storage<DT>::T* t10 = t00 + WC;
+    RawVec<DT, G::VW> t[G::NV][4];
+
+    __device__ __forceinline__ void load(const typename Storage<DT>::T* t00, int WC, int q) {
+#pragma unroll
+        for (int k = 0; k < G::NV; ++k) {
+            const typename Storage<DT>::T* p = t00 + G::VW * (q + k * G::LP);
+            load_raw<DT, G::VW>(p, t[k][0]);
+            load_raw<DT, G::VW>(p + C, t[k][1]);
+            load_raw<DT, G::VW>(p + WC, t[k][2]);
+            load_raw<DT, G::VW>(p + WC + C, t[k][3]);
+        }
+    }
+};
+
+// This lane's channels of one anchor's reference row.
+template <pilot_dtype DT, int C, bool SCALED> struct RefBuf {
+    using G = GroupShape<DT, C, SCALED>;
+    RawVec<DT, G::VW> r[G::NV];
+
+    __device__ __forceinline__ void load(const typename Storage<DT>::T* row, int q) {
+#pragma unroll
+        for (int k = 0; k < G::NV; ++k) load_raw<DT, G::VW>(row + G::VW * (q + k * G::LP), r[k]);
+    }
+};
+
+// Channel sums of one record over this lane's channels: the 4 taps against the anchor's
+// reference values: bilinear value and in-cell gradient, residual, and the six partial sums.
+template <pilot_dtype DT, int C, bool SCALED>
+__device__ __forceinline__ void record_partials(const TapBuf<DT, C, SCALED>& b, const RefBuf<DT, C, SCALED>& rr,
+                                                float ax, float ay, const float* qs, const float* rs, float* p) {
+    using G = GroupShape<DT, C, SCALED>;
+    constexpr int VW = G::VW;
     const f2 ax2 = pk(ax, ax), ay2 = pk(ay, ay), z2 = pk(0.f, 0.f);
     ChanSums2 cs{z2, z2, z2, z2, z2, z2};
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        const int c = VW * (q + k * LP);
-        float a00[VW], a01[VW], a10[VW], a11[VW];
-        load_vec<DT, VW>(t00 + c, a00);
-        load_vec<DT, VW>(t00 + c + C, a01);
-        load_vec<DT, VW>(t10 + c, a10);
-        load_vec<DT, VW>(t10 + c + C, a11);
-        const float* r = rr + k * VW;
+    for (int k = 0; k < G::NV; ++k) {
 #pragma unroll
-        for (int e = 0; e < VW; e += 2)
-            channel_pair<SCALED>(cs, pk(a00[e], a00[e + 1]), pk(a01[e], a01[e + 1]), pk(a10[e], a10[e + 1]),
-                                 pk(a11[e], a11[e + 1]), pk(r[e], r[e + 1]), ax2, ay2,
+        for (int e = 0; e < VW; e += 2) {
+            float a[4][2], r[2];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) raw_pair<DT, VW>(b.t[k][i], e, a[i][0], a[i][1]);
+            raw_pair<DT, VW>(rr.r[k], e, r[0], r[1]);
+            channel_pair<SCALED>(cs, pk(a[0][0], a[0][1]), pk(a[1][0], a[1][1]), pk(a[2][0], a[2][1]),
+                                 pk(a[3][0], a[3][1]), pk(r[0], r[1]), ax2, ay2,
                                  pk(qs[k * VW + e], qs[k * VW + e + 1]), pk(rs[k * VW + e], rs[k * VW + e + 1]));
+        }
     }
     p[0] = hsum(cs.s);
     p[1] = hsum(cs.m00);
@@ -399,11 +383,11 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
         float S[6];
         if constexpr (LP == 1) {
             // one lane per record: its own taps and reference row
-            float rr[C];
-            const Elem* fr = ref + (jo < j_end ? jo : j_begin) * C;
-#pragma unroll
-            for (int k = 0; k < NV; ++k) load_vec<DT, VW>(fr + VW * k, rr + VW * k);
-            record_partials<DT, C, SCALED>(qry + off, WC, rr, ax, ay, 0, qs, rs, S);
+            RefBuf<DT, C, SCALED> rr;
+            TapBuf<DT, C, SCALED> taps;
+            rr.load(ref + (jo < j_end ? jo : j_begin) * C, 0);
+            taps.load(qry + off, WC, 0);
+            record_partials<DT, C, SCALED>(taps, rr, ax, ay, qs, rs, S);
         } else {
             // 2. the group reads its records two at a time: records t and t + LP/2, one
             //    anchor (t mod APB) under two of the group's hypotheses, against one read of
@@ -412,15 +396,10 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
             //    butterfly round (xor LP/2) keeps in each lane only the record it owns, so
             //    only LP/2 partial records stay live
             constexpr int HALF = LP / 2;
-            float rra[HG > 2 ? APB : 1][CPL];
+            RefBuf<DT, C, SCALED> rra[HG > 2 ? APB : 1];
             if constexpr (HG > 2) {
 #pragma unroll
-                for (int a = 0; a < APB; ++a) {
-                    const int ja = jb + a;
-                    const Elem* fr = ref + (ja < j_end ? ja : j_begin) * C;
-#pragma unroll
-                    for (int k = 0; k < NV; ++k) load_vec<DT, VW>(fr + VW * (q + k * LP), rra[a] + k * VW);
-                }
+                for (int a = 0; a < APB; ++a) rra[a].load(ref + (jb + a < j_end ? jb + a : j_begin) * C, q);
             }
             // one butterfly step: lane keeps the record of its half and adds the partner's
             auto combine = [&](float* lo, const float* hi, int half) {
@@ -435,24 +414,19 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
             // record pair t: records t and t + HALF (one anchor, two hypotheses) against one
             // reference read, then the first butterfly round
             auto pair = [&](int t, float* Bt) {
-                float rrt[CPL];
-                const float* rr = rra[HG > 2 ? t % APB : 0];
-                if constexpr (HG <= 2) {
-                    const int ja = jb + t;
-                    const Elem* fr = ref + (ja < j_end ? ja : j_begin) * C;
-#pragma unroll
-                    for (int k = 0; k < NV; ++k) load_vec<DT, VW>(fr + VW * (q + k * LP), rrt + k * VW);
-                    rr = rrt;
-                }
+                RefBuf<DT, C, SCALED>& rr = rra[HG > 2 ? t % APB : 0];
+                if constexpr (HG <= 2) rr.load(ref + (jb + t < j_end ? jb + t : j_begin) * C, q);
                 float P2[2][6];
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     const int i = t + u * HALF;
-                    // the tap offset carries visibility: -1 when the record is not visible
-                    const int oi = __shfl_sync(gmask, vis ? off : -1, src0 + i);
+                    // (an invisible record reads the map's first cell; its sums are discarded)
+                    const int o = __shfl_sync(gmask, off, src0 + i);
                     const float axi = __shfl_sync(gmask, ax, src0 + i);
                     const float ayi = __shfl_sync(gmask, ay, src0 + i);
-                    record_partials<DT, C, SCALED>(qry + (oi >= 0 ? oi : 0), WC, rr, axi, ayi, q, qs, rs, P2[u]);
+                    TapBuf<DT, C, SCALED> taps;
+                    taps.load(qry + o, WC, q);
+                    record_partials<DT, C, SCALED>(taps, rr, axi, ayi, qs, rs, P2[u]);
                 }
                 combine(P2[0], P2[1], HALF);
 #pragma unroll
@@ -544,64 +518,6 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
             acc[28] += 1.0f;
         }
     }
-}
-
-// The 4 taps of one record in this lane's channels (vector k covers VW (q + k LP) .. + VW).
-template <pilot_dtype DT, int C, bool SCALED> struct TapBuf {
-    using G = GroupShape<DT, C, SCALED>;
-    RawVec<DT, G::VW> t[G::NV][4];
-
-    __device__ __forceinline__ void load(const typename Storage<DT>::T* t00, int WC, int q) {
-#pragma unroll
-        for (int k = 0; k < G::NV; ++k) {
-            const typename Storage<DT>::T* p = t00 + G::VW * (q + k * G::LP);
-            load_raw<DT, G::VW>(p, t[k][0]);
-            load_raw<DT, G::VW>(p + C, t[k][1]);
-            load_raw<DT, G::VW>(p + WC, t[k][2]);
-            load_raw<DT, G::VW>(p + WC + C, t[k][3]);
-        }
-    }
-};
-
-// This lane's channels of one anchor's reference row.
-template <pilot_dtype DT, int C, bool SCALED> struct RefBuf {
-    using G = GroupShape<DT, C, SCALED>;
-    RawVec<DT, G::VW> r[G::NV];
-
-    __device__ __forceinline__ void load(const typename Storage<DT>::T* row, int q) {
-#pragma unroll
-        for (int k = 0; k < G::NV; ++k) load_raw<DT, G::VW>(row + G::VW * (q + k * G::LP), r[k]);
-    }
-};
-
-// record_partials on taps and a reference row already loaded: the 4 taps against the anchor's
-// reference values: bilinear value and in-cell gradient, residual, and the six partial sums.
-template <pilot_dtype DT, int C, bool SCALED>
-__device__ __forceinline__ void raw_partials(const TapBuf<DT, C, SCALED>& b, const RefBuf<DT, C, SCALED>& rr,
-                                                float ax, float ay, const float* qs, const float* rs, float* p) {
-    using G = GroupShape<DT, C, SCALED>;
-    constexpr int VW = G::VW;
-    const f2 ax2 = pk(ax, ax), ay2 = pk(ay, ay), z2 = pk(0.f, 0.f);
-    ChanSums2 cs{z2, z2, z2, z2, z2, z2};
-#pragma unroll
-    for (int k = 0; k < G::NV; ++k) {
-#pragma unroll
-        for (int e = 0; e < VW; e += 2) {
-            float a[4][2], r[2];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) raw_pair<DT, VW>(b.t[k][i], e, a[i][0], a[i][1]);
-            raw_pair<DT, VW>(rr.r[k], e, r[0], r[1]);
-            channel_pair<SCALED>(cs, pk(a[0][0], a[0][1]), pk(a[1][0], a[1][1]), pk(a[2][0], a[2][1]),
-                                 pk(a[3][0], a[3][1]), pk(r[0], r[1]), ax2, ay2,
-                                 pk(qs[k * VW + e], qs[k * VW + e + 1]), pk(rs[k * VW + e], rs[k * VW + e + 1]));
-        }
-    }
-    p[0] = hsum(cs.s);
-    p[1] = hsum(cs.m00);
-    p[2] = hsum(cs.m01);
-    p[3] = hsum(cs.m11);
-    p[4] = hsum(cs.b0);
-    p[5] = hsum(cs.b1);
 }
 
 // ---- one hypothesis per CTA ----
@@ -781,7 +697,7 @@ __device__ __forceinline__ void accumulate_spread(const LevelView& v, const floa
                 const float axi = LP > 1 ? __shfl_sync(0xffffffffu, ax, src0 + i) : ax;
                 const float ayi = LP > 1 ? __shfl_sync(0xffffffffu, ay, src0 + i) : ay;
                 float* P = LP == 1 || k == 6 ? S : (k & 1) ? B[2] : (k == 0 ? B[0] : B[1]);
-                raw_partials<DT, C, SCALED>(taps[m], rr[m], axi, ayi, qs, rs, P);
+                record_partials<DT, C, SCALED>(taps[m], rr[m], axi, ayi, qs, rs, P);
                 if (k == 1) combine(B[0], B[2], HALF);
                 if (k == 3) {
                     combine(B[1], B[2], HALF);
@@ -887,22 +803,45 @@ __device__ __forceinline__ float cta_reduce_spread(float* acc, float (*red)[kAcc
     return v;
 }
 
-// Fixed-order CTA reduction of the lanes' 29 sums, per hypothesis slot: the lanes of a slot
+// Fixed-order CTA reduction of the lanes' 29 sums, per hypothesis slot: the eight lanes of a slot
 // are reduced by a butterfly over every lane bit but the slot bits (APB .. APB kHypTile / 2),
-// then the warps in order.  Thread t < kHypTile kAcc returns sum t mod kAcc of slot t / kAcc
-// (0 pads).
-template <int NTHREADS, int APB>
+// then the warps in order.  SCATTER: the butterfly scatters as it goes (16, 8, then 4 sums exchanged
+// instead of 29 three times: the shuffles are what the reduction costs), so a lane ends with four
+// sums; without it fewer registers are live, which the level kernels need more (batched BF16,
+// uneven frames: 15.1 ms without, 15.4 ms with).  Thread t < kHypTile kAcc returns sum t mod kAcc
+// of slot t / kAcc (0 pads).
+template <int NTHREADS, int APB, bool SCATTER = true>
 __device__ __forceinline__ float cta_reduce_slots(float* acc, float (*red)[kHypTile][kAcc]) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // the three non-slot lane bits, in the butterfly's order
+    constexpr int b0 = APB == 2 ? 1 : 4, b1 = 8, b2 = 16;
+    static_assert(APB * kHypTile == 4 || APB * kHypTile == 8, "slots of a warp");
+    if constexpr (SCATTER) {
+        auto exchange = [&](float* a, int n, int bit) {  // keeps the lower or upper half of n sums
+            const bool up = (lane & bit) != 0;
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        if (off >= APB && off < APB * kHypTile) continue;
+            for (int i = 0; i < n / 2; ++i) {
+                const float send = up ? a[i] : a[i + n / 2], keep = up ? a[i + n / 2] : a[i];
+                a[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+            }
+        };
+        float a[kAcc];
 #pragma unroll
-        for (int i = 0; i < kNumSums; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
-    }
-    if (lane % APB == 0 && lane < APB * kHypTile) {
+        for (int i = 0; i < kAcc; ++i) a[i] = i < kNumSums ? acc[i] : 0.f;
+        exchange(a, 32, b0);
+        exchange(a, 16, b1);
+        exchange(a, 8, b2);
+        const int kept = ((lane & b0) ? 16 : 0) + ((lane & b1) ? 8 : 0) + ((lane & b2) ? 4 : 0);
+        *reinterpret_cast<float4*>(&red[warp][(lane / APB) % kHypTile][kept]) = make_float4(a[0], a[1], a[2], a[3]);
+    } else {
 #pragma unroll
-        for (int i = 0; i < kNumSums; ++i) red[warp][lane / APB][i] = acc[i];
+        for (int bit : {b0, b1, b2})
+#pragma unroll
+            for (int i = 0; i < kNumSums; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], bit);
+        if (lane % APB == 0 && lane < APB * kHypTile) {
+#pragma unroll
+            for (int i = 0; i < kNumSums; ++i) red[warp][lane / APB][i] = acc[i];
+        }
     }
     __syncthreads();
     float v = 0.f;
@@ -953,7 +892,7 @@ __device__ __forceinline__ bool any_cand(const TileSlots& ts) {
 template <pilot_dtype DT, int C, bool SCALED, bool CONF>
 __global__ void __launch_bounds__(kBuildThreads, 2)
 build_kernel(const BuildParams p) {
-    __shared__ float red[kBuildThreads / 32][kHypTile][kAcc];
+    __shared__ __align__(16) float red[kBuildThreads / 32][kHypTile][kAcc];
     const TileSlots ts = tile_slots(p);
     if (!any_cand(ts)) return;                       // uniform over the CTA
     float acc[kNumSums];
@@ -976,7 +915,7 @@ template <pilot_dtype DT, int C, bool SCALED, bool CONF>
 __global__ void __launch_bounds__(kBuildThreads, 2)
 build_fused_kernel(const FusedBuildParams fp) {
     const BuildParams& p = fp.b;
-    __shared__ float red[kBuildThreads / 32][kHypTile][kAcc];
+    __shared__ __align__(16) float red[kBuildThreads / 32][kHypTile][kAcc];
     __shared__ double part[kHypTile][8][kAcc];
     __shared__ double E[kHypTile][kAcc];
     __shared__ int s_last;
@@ -1004,12 +943,15 @@ build_fused_kernel(const FusedBuildParams fp) {
     }
     if (tid < kHypTile * kAcc && hv < ts.n && ts.cand[hv])
         p.partial[((size_t)ts.slot[hv] * p.n_tiles + blockIdx.x) * kAcc + iv] = v;
-    __threadfence();
+    // one fence for the CTA's records (it is cumulative over the barrier)
     __syncthreads();
-    if (tid == 0) s_last = (atomicAdd(fp.tickets + blockIdx.y, 1u) == (unsigned)(p.n_tiles - 1));
+    if (tid == 0) {
+        __threadfence();
+        s_last = (atomicAdd(fp.tickets + blockIdx.y, 1u) == (unsigned)(p.n_tiles - 1));
+        if (s_last) __threadfence();
+    }
     __syncthreads();
     if (!s_last) return;
-    __threadfence();
     // 8 chains per slot and value: thread (h, c, i) sums tiles c, c + 8, ... of sum i of slot h
     {
         constexpr int kTPC = kBuildThreads / (kHypTile * 8);     // threads per (slot, chain)
@@ -1055,7 +997,7 @@ __global__ void __launch_bounds__(kBuildThreads, 2)
 level_resident_kernel(const __grid_constant__ ResidentParams rp) {
     namespace cg = cooperative_groups;
     const BuildParams& p = rp.b;
-    __shared__ float red[kBuildThreads / 32][kHypTile][kAcc];
+    __shared__ __align__(16) float red[kBuildThreads / 32][kHypTile][kAcc];
     __shared__ double E[kHypTile][kAcc];
     __shared__ float rec[kHypTile][kAcc];
     __shared__ float pose[kHypTile][12];

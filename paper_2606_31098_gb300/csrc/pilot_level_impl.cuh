@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kBuildThreads, 2)
 level_persistent_kernel(const __grid_constant__ LevelArgs a) {
     constexpr int kWarps = kBuildThreads / 32;
     constexpr unsigned kEval = 0x80000000u;          // job_meta: "has a pose to evaluate" bit
-    __shared__ float red[kWarps][kHypTile][kAcc];
+    __shared__ __align__(16) float red[kWarps][kHypTile][kAcc];
     __shared__ double E[kWarps][kAcc];
     __shared__ float pose[kHypTile][12];
     __shared__ unsigned s_meta[kHypTile];
@@ -256,7 +256,7 @@ level_persistent_kernel(const __grid_constant__ LevelArgs a) {
                     const int j0 = t * a.tile;
                     accumulate_anchors<DT, C, SCALED, CONF, kBuildThreads, DT == PILOT_F32, true>(
                         v, sp, j0, min(j0 + a.tile, fd->N), acc);
-                    const float val = cta_reduce_slots<kBuildThreads, GroupShape<DT, C, SCALED>::APB>(acc, red);
+                    const float val = cta_reduce_slots<kBuildThreads, GroupShape<DT, C, SCALED>::APB, false>(acc, red);
                     if (tid < kHypTile * kAcc && tid / kAcc < s_njobs)
                         a.partial[(((size_t)s_first * tpi + t) * kHypTile + tid / kAcc) * kAcc + tid % kAcc] = val;
                     if (t + 1 < s_t1) __syncthreads();
@@ -392,7 +392,7 @@ level_persistent_kernel(const __grid_constant__ LevelArgs a) {
                             // already take the registers that kernel parameters cost the plain form
                             accumulate_anchors<DT, C, SCALED, CONF, kBuildThreads, DT == PILOT_F32>(
                                 v, sp, j0, min(j0 + a.tile, fd->N), acc);
-                            const float val = cta_reduce_slots<kBuildThreads, GroupShape<DT, C, SCALED>::APB>(acc, red);
+                            const float val = cta_reduce_slots<kBuildThreads, GroupShape<DT, C, SCALED>::APB, false>(acc, red);
                             if (tid < kHypTile * kAcc && tid / kAcc < s_njobs)
                                 a.partial[(((size_t)s_first * tpi + t) * kHypTile + tid / kAcc) * kAcc + tid % kAcc] =
                                     val;

@@ -1,6 +1,6 @@
 """Levels of small frames run in one launch (one hypothesis or four per CTA, one or several anchor
-tiles per cluster): every output bitwise that of the batched form, which runs the same levels
-with a launch-wide work queue, over storage types, channels, scales, confidence maps and the
+tiles per cluster; batched: job tiles claimed for a whole level): every output bitwise that of the
+batched form in lockstep (which a frame of two anchor tiles in the batch asks for), over storage types, channels, scales, confidence maps and the
 sizes at which the layout changes (batches of 64 anchors, steps of 256, tiles of 1024)."""
 import numpy as np
 import pytest
@@ -40,16 +40,22 @@ def cut(frame, n, m, conf):
 
 
 def check(torch, frame, dt, per_channel, damping=0):
-    opts = B.Options(iters=(3, 2), max_points=max(frame.N, 1), max_hyps=frame.M, max_channels=frame.C, max_frames=1,
+    opts = B.Options(iters=(3, 2), max_points=max(frame.N, 1100), max_hyps=frame.M + 1, max_channels=frame.C, max_frames=2,
                      damping_mode=damping, keep_top_k=(0, max(1, frame.M // 2), 0, 0))
     fa = B.FrameArgs(frame, B.quantized_device_arrays(frame, dt, per_channel=per_channel), is_device=True, dtype=dt)
+    # a second frame of 1100 anchors sends the batch through the lockstep schedule
+    two = frame.replace(points=np.resize(frame.points[:, :1], (3, 1100)), point_valid=np.ones(1100, np.uint8),
+                        point_weight=np.ones(1100, np.float32),
+                        ref_feat=[np.resize(f[:1], (1100, frame.C)) for f in frame.ref_feat], T_hyps=frame.T_hyps[:1])
+    fb = B.FrameArgs(two, B.quantized_device_arrays(two, dt, per_channel=per_channel), is_device=True, dtype=dt)
     s = B.Solver(opts)
-    a, b = s.solve(fa), s.solve_batch([fa])[0]
-    np.testing.assert_array_equal(a.T_cw, b.T_cw)
-    np.testing.assert_array_equal(a.cost, b.cost)
-    np.testing.assert_array_equal(a.n_valid, b.n_valid)
-    np.testing.assert_array_equal(a.status, b.status)
-    assert a.best == b.best
+    a = s.solve(fa)
+    for b in (s.solve_batch([fa])[0], s.solve_batch([fa, fb])[0]):
+        np.testing.assert_array_equal(a.T_cw, b.T_cw)
+        np.testing.assert_array_equal(a.cost, b.cost)
+        np.testing.assert_array_equal(a.n_valid, b.n_valid)
+        np.testing.assert_array_equal(a.status, b.status)
+        assert a.best == b.best
     # the evaluation of one level, with and without a handle
     T = np.ascontiguousarray(frame.T_hyps)
     ne = s.normal_eq(fa, 1, T)
