@@ -889,22 +889,39 @@ __device__ __forceinline__ bool any_cand(const TileSlots& ts) {
     return a;
 }
 
+// Evaluation of larger frames at given poses (T_cw, M x 12): the tile records; epilogue_kernel,
+// which may start while the last of these CTAs run, sums them.  The poses are narrowed here, and
+// left in the state for the priors.  (Summing in the last CTA of each hypothesis tile, as
+// build_fused_kernel does, made 64 poses x 65536 anchors 172 us instead of 164: sixteen CTAs sum
+// what sixty-four blocks do here.)
 template <pilot_dtype DT, int C, bool SCALED, bool CONF>
 __global__ void __launch_bounds__(kBuildThreads, 2)
-build_kernel(const BuildParams p) {
+build_kernel(const BuildParams p, HypState* state, const double* T_cw) {
     __shared__ __align__(16) float red[kBuildThreads / 32][kHypTile][kAcc];
-    const TileSlots ts = tile_slots(p);
-    if (!any_cand(ts)) return;                       // uniform over the CTA
+    __shared__ float pose[kHypTile][12];
+    const int slot0 = kHypTile * (int)blockIdx.y, n = min(kHypTile, p.n_active - slot0), tid = threadIdx.x;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (tid < 12 * kHypTile) {
+        const int h = tid / 12, hyp = slot0 + (h < n ? h : 0);
+        const double t = T_cw[12 * (size_t)hyp + tid % 12];
+        pose[h][tid % 12] = narrow(t);
+        if (blockIdx.x == 0 && h < n) state[hyp].T[tid % 12] = t;
+    }
+    __syncthreads();
+    SlotPoses sp;
+#pragma unroll
+    for (int h = 0; h < kHypTile; ++h) {
+        sp.p[h] = pose[h];
+        sp.act[h] = h < n;
+    }
     float acc[kNumSums];
 #pragma unroll
     for (int i = 0; i < kNumSums; ++i) acc[i] = 0.f;
     const int j0 = blockIdx.x * p.tile;
-    accumulate_anchors<DT, C, SCALED, CONF, kBuildThreads>(level_view(p), slot_poses(p, ts), j0,
-                                                           min(j0 + p.tile, p.N), acc);
+    accumulate_anchors<DT, C, SCALED, CONF, kBuildThreads>(level_view(p), sp, j0, min(j0 + p.tile, p.N), acc);
     const float v = cta_reduce_slots<kBuildThreads, GroupShape<DT, C, SCALED>::APB>(acc, red);
-    const int h = threadIdx.x / kAcc;
-    if (threadIdx.x < kHypTile * kAcc && h < ts.n && ts.cand[h])
-        p.partial[((size_t)ts.slot[h] * p.n_tiles + blockIdx.x) * kAcc + threadIdx.x % kAcc] = v;
+    const int h = tid / kAcc;
+    if (tid < kHypTile * kAcc && h < n) p.partial[((size_t)(slot0 + h) * p.n_tiles + blockIdx.x) * kAcc + tid % kAcc] = v;
 }
 
 // The same pass with the per-hypothesis FP64 step fused in: the CTA that takes the last
@@ -1159,16 +1176,16 @@ level_spread_kernel(const __grid_constant__ ResidentParams rp) {
 }
 
 template <pilot_dtype DT, int C>
-cudaError_t launch_build_typed(const BuildParams& p, cudaStream_t s) {
+cudaError_t launch_build_typed(const BuildParams& p, HypState* state, const double* T_cw, cudaStream_t s) {
     dim3 grid(p.n_tiles, (p.n_active + kHypTile - 1) / kHypTile);
     if (p.qscale && p.conf)
-        build_kernel<DT, C, true, true><<<grid, kBuildThreads, 0, s>>>(p);
+        build_kernel<DT, C, true, true><<<grid, kBuildThreads, 0, s>>>(p, state, T_cw);
     else if (p.qscale)
-        build_kernel<DT, C, true, false><<<grid, kBuildThreads, 0, s>>>(p);
+        build_kernel<DT, C, true, false><<<grid, kBuildThreads, 0, s>>>(p, state, T_cw);
     else if (p.conf)
-        build_kernel<DT, C, false, true><<<grid, kBuildThreads, 0, s>>>(p);
+        build_kernel<DT, C, false, true><<<grid, kBuildThreads, 0, s>>>(p, state, T_cw);
     else
-        build_kernel<DT, C, false, false><<<grid, kBuildThreads, 0, s>>>(p);
+        build_kernel<DT, C, false, false><<<grid, kBuildThreads, 0, s>>>(p, state, T_cw);
     return cudaGetLastError();
 }
 
@@ -1223,13 +1240,13 @@ cudaError_t launch_resident_dtype(const ResidentParams& p, bool spread, cudaStre
 }
 
 template <pilot_dtype DT>
-cudaError_t launch_build_dtype(const BuildParams& p, cudaStream_t s) {
+cudaError_t launch_build_dtype(const BuildParams& p, HypState* state, const double* T_cw, cudaStream_t s) {
     switch (p.C) {
-        case 4: return launch_build_typed<DT, 4>(p, s);
-        case 8: return launch_build_typed<DT, 8>(p, s);
-        case 16: return launch_build_typed<DT, 16>(p, s);
-        case 32: return launch_build_typed<DT, 32>(p, s);
-        case 64: return launch_build_typed<DT, 64>(p, s);
+        case 4: return launch_build_typed<DT, 4>(p, state, T_cw, s);
+        case 8: return launch_build_typed<DT, 8>(p, state, T_cw, s);
+        case 16: return launch_build_typed<DT, 16>(p, state, T_cw, s);
+        case 32: return launch_build_typed<DT, 32>(p, state, T_cw, s);
+        case 64: return launch_build_typed<DT, 64>(p, state, T_cw, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -18,29 +18,25 @@ namespace pilot {
 
 namespace {
 
-// One block of 256 threads per hypothesis slot: FP64 sum of the tile records (8 partial
-// chains per value, combined in a fixed order), then the FP64 LM step on warp 0.
-__global__ void epilogue_kernel(const EpilogueParams p, const double* min_valid_ptr) {
+// One block of 256 threads per pose: FP64 sum of the tile records (8 partial chains per value,
+// combined in a fixed order), then the priors on warp 0.  Launched while the build pass before it
+// still runs.
+__global__ void epilogue_kernel(const EpilogueParams p) {
     const int slot = blockIdx.x;
     __shared__ double part[8][kAcc];
     __shared__ double E[kAcc];
     const int v = threadIdx.x & 31, c = threadIdx.x >> 5;
-    const HypState& st = p.state[p.active_idx[slot]];
-    const bool evaluated = (p.mode == kEpiStep) ? (st.has_cand != 0) : true;
-    if (evaluated) {
-        const float* src = p.partial + (size_t)slot * p.n_tiles * kAcc + v;
-        part[c][v] = chain_sum([&](int t) { return src[(size_t)t * kAcc]; }, c, p.n_tiles);
-        __syncthreads();
-        if (threadIdx.x < kAcc) {
-            double sum = part[0][threadIdx.x];
-            for (int k = 1; k < min(8, p.n_tiles); ++k) sum += part[k][threadIdx.x];
-            E[threadIdx.x] = sum;
-        }
-    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const float* src = p.partial + (size_t)slot * p.n_tiles * kAcc + v;
+    part[c][v] = chain_sum([&](int t) { return __ldcg(src + (size_t)t * kAcc); }, c, p.n_tiles);
     __syncthreads();
-    if (threadIdx.x >= 32) return;                 // warp 0 runs the FP64 step
-    const double min_valid = (p.mode == kEpiEval) ? 0.0 : *min_valid_ptr;
-    lm_step(p, slot, E, min_valid, threadIdx.x);
+    if (threadIdx.x >= 32) return;                 // warp 0
+    double sum = part[0][v];
+    for (int k = 1; k < min(8, p.n_tiles); ++k) sum += part[k][v];
+    E[v] = sum;
+    __syncwarp();
+    lm_update(p.state[slot], kEpiEval, 0, p.damping_mode, p.prior, E, 0.0, nullptr,
+              p.eval_out + (size_t)slot * kNumSums, v);
 }
 
 // LM state of hypothesis m at the start of a solve, by one warp.
@@ -103,16 +99,6 @@ solve_init_kernel(HypState* st, const double* T_cw, int* active_idx, int M, unsi
         active_idx[m] = m;
         tickets[m] = 0u;
     }
-}
-
-__global__ void set_poses_kernel(HypState* st, float* pose32, const double* T_cw, int* active_idx,
-                                 int M) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= M) return;
-    for (int i = 0; i < 12; ++i) st[m].T[i] = T_cw[12 * m + i];
-    store_pose32(pose32 + 12 * m, st[m].T);
-    st[m].has_cand = 1;
-    active_idx[m] = m;
 }
 
 __global__ void level_init_kernel(HypState* st, float* pose32, const int* active_idx, int n_active,
@@ -543,10 +529,18 @@ cudaError_t launch_round_finish(const BatchHeader* hdr, const FrameDesc* frames,
     return cudaGetLastError();
 }
 
-cudaError_t launch_epilogue(const EpilogueParams& p, const double* min_valid, cudaStream_t s) {
+cudaError_t launch_epilogue(const EpilogueParams& p, cudaStream_t s) {
     if (p.n_active <= 0) return cudaSuccess;
-    epilogue_kernel<<<p.n_active, 256, 0, s>>>(p, min_valid);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(p.n_active);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, epilogue_kernel, p);
 }
 
 cudaError_t launch_solve_init(HypState* st, const double* T_cw, int* active_idx, int M, unsigned* tickets,
@@ -554,13 +548,6 @@ cudaError_t launch_solve_init(HypState* st, const double* T_cw, int* active_idx,
                               cudaStream_t s) {
     solve_init_kernel<<<(M + kInitThreads / 32 - 1) / (kInitThreads / 32) + 1, kInitThreads, 0, s>>>(
         st, T_cw, active_idx, M, tickets, done_ticket, valid, N, frac, min_valid);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_set_poses(HypState* st, float* pose32, const double* T_cw, int* active_idx,
-                             int M, cudaStream_t s) {
-    if (M <= 0) return cudaSuccess;
-    set_poses_kernel<<<(M + 127) / 128, 128, 0, s>>>(st, pose32, T_cw, active_idx, M);
     return cudaGetLastError();
 }
 

@@ -265,23 +265,24 @@ struct ResultLayout {
 };
 
 // ---- launchers (each returns the cudaError_t of its launch) ----
-cudaError_t launch_epilogue(const EpilogueParams& p, const double* min_valid, cudaStream_t s);
+cudaError_t launch_epilogue(const EpilogueParams& p, cudaStream_t s);    // after launch_build
 cudaError_t launch_level_init(HypState* st, float* pose32, const int* active_idx, int n_active,
                               double lambda0, cudaStream_t s);
 // Start of a plain solve: states, active list, tickets (M, and done_ticket), visibility threshold.
 cudaError_t launch_solve_init(HypState* st, const double* T_cw, int* active_idx, int M, unsigned* tickets,
                               unsigned* done_ticket, const uint8_t* valid, int N, double frac, double* min_valid,
                               cudaStream_t s);
-cudaError_t launch_set_poses(HypState* st, float* pose32, const double* T_cw, int* active_idx,
-                             int M, cudaStream_t s);
 // ticket: one word, zero before the launch and after it
 cudaError_t launch_prune(HypState* st, const int* active_in, int* active_out, int n_active,
                          int keep, const double* min_valid, unsigned* ticket, cudaStream_t s);
 cudaError_t launch_finalize(HypState* st, int M, const double* min_valid, unsigned char* result,
                             ResultLayout lay, unsigned* ticket, cudaStream_t s);
 
+// Tile records at given poses (T_cw, M x 12, device), slot s being hypothesis s; the poses are left
+// in state.  launch_epilogue after it sums them.
 template <pilot_dtype DT>
-cudaError_t launch_build_dtype(const BuildParams& p, cudaStream_t s);
+cudaError_t launch_build_dtype(const BuildParams& p, HypState* state, const double* T_cw, cudaStream_t s);
+cudaError_t launch_build(pilot_dtype dt, const BuildParams& p, HypState* state, const double* T_cw, cudaStream_t s);
 template <pilot_dtype DT>
 cudaError_t launch_build_fused_dtype(const FusedBuildParams& p, cudaStream_t s);
 

@@ -374,16 +374,6 @@ PriorParams prior_params(const pilot_align_config& c, const pilot_frame* f, cons
     return pp;
 }
 
-cudaError_t dispatch_build(pilot_dtype dt, const BuildParams& b, cudaStream_t s) {
-    switch (dt) {
-        case PILOT_F32: return launch_build_dtype<PILOT_F32>(b, s);
-        case PILOT_BF16: return launch_build_dtype<PILOT_BF16>(b, s);
-        case PILOT_F16: return launch_build_dtype<PILOT_F16>(b, s);
-        case PILOT_FP8E4M3: return launch_build_dtype<PILOT_FP8E4M3>(b, s);
-    }
-    return cudaErrorInvalidValue;
-}
-
 cudaError_t dispatch_build_fused(pilot_dtype dt, const FusedBuildParams& b, cudaStream_t s) {
     switch (dt) {
         case PILOT_F32: return launch_build_fused_dtype<PILOT_F32>(b, s);
@@ -414,12 +404,11 @@ pilot_status timed_build(pilot_align_handle* h, cudaStream_t s, Launch launch) {
     return PILOT_OK;
 }
 
-// One build launch, plain (ep == nullptr) or with the FP64 step fused in.
+// One build launch with the FP64 step fused in.
 pilot_status run_build(pilot_align_handle* h, pilot_dtype dt, const BuildParams& b, cudaStream_t s,
-                       const EpilogueParams* ep = nullptr, int slot_offset = 0) {
+                       const EpilogueParams& ep, int slot_offset) {
     return timed_build(h, s, [&]() {
-        return ep ? dispatch_build_fused(dt, FusedBuildParams{b, *ep, h->tickets + slot_offset, h->min_valid}, s)
-                  : dispatch_build(dt, b, s);
+        return dispatch_build_fused(dt, FusedBuildParams{b, ep, h->tickets + slot_offset, h->min_valid}, s);
     });
 }
 
@@ -595,6 +584,15 @@ cudaError_t level_occupancy(pilot_dtype dt, int C, int variant, int* n) {
 }  // namespace
 
 namespace pilot {
+cudaError_t launch_build(pilot_dtype dt, const BuildParams& b, HypState* state, const double* T_cw, cudaStream_t s) {
+    switch (dt) {
+        case PILOT_F32: return launch_build_dtype<PILOT_F32>(b, state, T_cw, s);
+        case PILOT_BF16: return launch_build_dtype<PILOT_BF16>(b, state, T_cw, s);
+        case PILOT_F16: return launch_build_dtype<PILOT_F16>(b, state, T_cw, s);
+        case PILOT_FP8E4M3: return launch_build_dtype<PILOT_FP8E4M3>(b, state, T_cw, s);
+    }
+    return cudaErrorInvalidValue;
+}
 cudaError_t launch_resident(pilot_dtype dt, const ResidentParams& p, bool spread, cudaStream_t s) {
     switch (dt) {
         case PILOT_F32: return launch_resident_dtype<PILOT_F32>(p, spread, s);
@@ -877,7 +875,7 @@ pilot_status pilot_align_solve(pilot_align_handle* h, const pilot_frame* f, pilo
                 for (int p = 0; p < parts; ++p) {
                     epp[p].mode = (k == 0) ? kEpiInit : kEpiStep;
                     epp[p].solve_next = k < iters;
-                    if ((st = run_build(h, f->feat_dtype, bp[p], sp[p], &epp[p], off[p])) != PILOT_OK) return st;
+                    if ((st = run_build(h, f->feat_dtype, bp[p], sp[p], epp[p], off[p])) != PILOT_OK) return st;
                 }
             }
             for (int p = 1; p < parts; ++p) {
@@ -936,28 +934,23 @@ pilot_status pilot_align_debug_normal_eq(pilot_align_handle* h, const pilot_fram
     PILOT_CUDA(cudaMemcpyAsync(h->Tin, T_cw, sizeof(double) * 12 * M, cudaMemcpyHostToDevice, s), "pose copy");
     BuildParams b = build_params(h, f, d, level, M, h->active[0]);
     const int kind = resident_kind(M, b.n_tiles);
-    if (kind == 0) {
-        PILOT_CUDA(launch_set_poses(h->state, h->pose32, h->Tin, h->active[0], M, s), "set_poses launch");
-        if ((st = run_build(h, f->feat_dtype, b, s)) != PILOT_OK) return st;
-        ++h->total_launches;
-    }
+    b.active_idx = nullptr;
     EpilogueParams ep{};
     ep.state = h->state;
     ep.pose32 = h->pose32;
     ep.partial = h->partial;
-    ep.active_idx = h->active[0];
     ep.n_active = M;
     ep.n_tiles = b.n_tiles;
     ep.mode = kEpiEval;
     ep.prior = prior_params(h->cfg, f, d);
     ep.eval_out = h->eval_out;
-    if (kind != 0) {
-        b.active_idx = nullptr;
-        const ResidentParams rp{b, ep, nullptr, h->Tin, 0};
-        if ((st = timed_build(h, s, [&]() { return launch_resident(f->feat_dtype, rp, kind == 2, s); })) != PILOT_OK)
-            return st;
-    } else {
-        PILOT_CUDA(launch_epilogue(ep, h->min_valid, s), "epilogue launch");
+    st = timed_build(h, s, [&]() {
+        return kind != 0 ? launch_resident(f->feat_dtype, ResidentParams{b, ep, nullptr, h->Tin, 0}, kind == 2, s)
+                         : launch_build(f->feat_dtype, b, h->state, h->Tin, s);
+    });
+    if (st != PILOT_OK) return st;
+    if (kind == 0) {
+        PILOT_CUDA(launch_epilogue(ep, s), "epilogue launch");
         ++h->total_launches;
     }
     PILOT_CUDA(cudaMemcpyAsync(out29, h->eval_out, sizeof(double) * kNumSums * M, cudaMemcpyDeviceToHost, s),

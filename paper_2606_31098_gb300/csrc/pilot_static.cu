@@ -35,10 +35,7 @@ constexpr int kStaticMaxPoints = kStaticMaxTiles * kStaticTile;
 
 constexpr size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 constexpr size_t kOffState = 0;
-constexpr size_t kOffPose = align256(kOffState + sizeof(HypState) * kStaticMaxHyps);
-constexpr size_t kOffActive = align256(kOffPose + sizeof(float) * 12 * kStaticMaxHyps);
-constexpr size_t kOffMinValid = align256(kOffActive + sizeof(int) * kStaticMaxHyps);
-constexpr size_t kOffPartial = align256(kOffMinValid + sizeof(double));
+constexpr size_t kOffPartial = align256(kOffState + sizeof(HypState) * kStaticMaxHyps);
 constexpr size_t kScratchBytes =
     align256(kOffPartial + sizeof(float) * kAcc * kStaticMaxTiles * (size_t)kStaticMaxHyps);
 
@@ -123,16 +120,6 @@ pilot_status scratch_address(unsigned char** scratch, float** ones) {
     return PILOT_OK;
 }
 
-cudaError_t dispatch(pilot_dtype dt, const BuildParams& b, cudaStream_t s) {
-    switch (dt) {
-        case PILOT_F32: return launch_build_dtype<PILOT_F32>(b, s);
-        case PILOT_BF16: return launch_build_dtype<PILOT_BF16>(b, s);
-        case PILOT_F16: return launch_build_dtype<PILOT_F16>(b, s);
-        case PILOT_FP8E4M3: return launch_build_dtype<PILOT_FP8E4M3>(b, s);
-    }
-    return cudaErrorInvalidValue;
-}
-
 }  // namespace
 }  // namespace pilot
 
@@ -166,9 +153,6 @@ extern "C" pilot_status pilot_align_normal_eq_noalloc(const pilot_align_config* 
     if ((st = scratch_address(&base, &ones)) != PILOT_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     HypState* state = reinterpret_cast<HypState*>(base + kOffState);
-    float* pose32 = reinterpret_cast<float*>(base + kOffPose);
-    int* active = reinterpret_cast<int*>(base + kOffActive);
-    double* min_valid = reinterpret_cast<double*>(base + kOffMinValid);
     float* partial = reinterpret_cast<float*>(base + kOffPartial);
 
     const double huber_photo = cfg->huber_photo == 0.0 ? 0.1 : cfg->huber_photo;
@@ -200,27 +184,14 @@ extern "C" pilot_status pilot_align_normal_eq_noalloc(const pilot_align_config* 
     b.cx = (float)(f->cx * sc);
     b.cy = (float)(f->cy * sc);
     b.huber = (float)huber_photo;
-    b.pose32 = pose32;
-    b.active_idx = active;
     b.state = state;
     b.partial = partial;
     b.n_active = f->M;
     b.tile = kStaticTile;
     b.n_tiles = f->N > 0 ? (f->N + kStaticTile - 1) / kStaticTile : 1;
-    const int kind = resident_kind(f->M, b.n_tiles);
-    cudaError_t e = cudaSuccess;
-    if (kind == 0) {
-        e = launch_set_poses(state, pose32, T_cw, active, f->M, s);
-        if (e != cudaSuccess) return fail_msg(PILOT_ECUDA, std::string("set_poses launch: ") + cudaGetErrorString(e));
-        e = dispatch(f->feat_dtype, b, s);
-        if (e != cudaSuccess) return fail_msg(PILOT_ECUDA, std::string("build-pass launch: ") + cudaGetErrorString(e));
-    }
-
     EpilogueParams ep{};
     ep.state = state;
-    ep.pose32 = pose32;
     ep.partial = partial;
-    ep.active_idx = active;
     ep.n_active = f->M;
     ep.n_tiles = b.n_tiles;
     ep.mode = kEpiEval;
@@ -250,12 +221,10 @@ extern "C" pilot_status pilot_align_normal_eq_noalloc(const pilot_align_config* 
     pp.gate_grav = cfg->gate_grav;
     pp.gate_range = cfg->gate_range;
     pp.derive();
-    if (kind != 0) {
-        b.active_idx = nullptr;
-        e = launch_resident(f->feat_dtype, ResidentParams{b, ep, nullptr, T_cw, 0}, kind == 2, s);
-    } else {
-        e = launch_epilogue(ep, min_valid, s);
-    }
+    const int kind = resident_kind(f->M, b.n_tiles);
+    cudaError_t e = kind != 0 ? launch_resident(f->feat_dtype, ResidentParams{b, ep, nullptr, T_cw, 0}, kind == 2, s)
+                              : launch_build(f->feat_dtype, b, state, T_cw, s);
+    if (e == cudaSuccess && kind == 0) e = launch_epilogue(ep, s);
     if (e != cudaSuccess) return fail_msg(PILOT_ECUDA, std::string("evaluation launch: ") + cudaGetErrorString(e));
     return PILOT_OK;
 }
