@@ -1005,16 +1005,17 @@ build_fused_kernel(const FusedBuildParams fp) {
 // Why: with few anchors an iteration is a chain of latencies -- the launch, eight or more
 // dependent batches of gathers, the FP64 step.  One launch per level drops the launches, and
 // level_spread_kernel shortens the rest while SMs would be idle.  solve_small (4096 anchors, 1
-// hypothesis, 20 iterations): 752 -> 381 us; paper's schedule (500 anchors, 1210 -> 128
-// hypotheses, 12 evaluations): 552 -> 343 us (with the FP64 step's own gain).
+// hypothesis, 20 iterations): 752 -> 378 us; paper's schedule (500 anchors, 1210 -> 128
+// hypotheses, 12 evaluations): 552 -> 284 us (with the FP64 step's own gain).
 
-// kHypTile hypotheses per CTA.
+// kHypTile hypotheses per CTA, hypothesis h stepped by warp h.
 template <pilot_dtype DT, int C, bool SCALED, bool CONF>
 __global__ void __launch_bounds__(kBuildThreads, 2)
 level_resident_kernel(const __grid_constant__ ResidentParams rp) {
     namespace cg = cooperative_groups;
     const BuildParams& p = rp.b;
     __shared__ __align__(16) float red[kBuildThreads / 32][kHypTile][kAcc];
+    __shared__ ResidentHyp hyps[kHypTile];
     __shared__ double E[kHypTile][kAcc];
     __shared__ float rec[kHypTile][kAcc];
     __shared__ float pose[kHypTile][12];
@@ -1023,27 +1024,20 @@ level_resident_kernel(const __grid_constant__ ResidentParams rp) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = blockIdx.x, slot0 = kHypTile * (int)blockIdx.y, n = min(kHypTile, p.n_active - slot0);
     const int iters = rp.iters;
-    auto hyp_of = [&](int h) { return p.active_idx ? p.active_idx[slot0 + h] : slot0 + h; };
+    const bool steps = rank == 0 && warp < n;
     auto all_ctas = [&]() {
         if (p.n_tiles > 1) cluster.sync();
         else __syncthreads();
     };
-    // level start: damping and flags by the stepping warps, the FP32 poses by every CTA
-    if (rank == 0 && warp < n) {
-        HypState& st = rp.ep.state[hyp_of(warp)];
-        if (rp.T_cw && lane < 12) st.T[lane] = rp.T_cw[12 * (size_t)hyp_of(warp) + lane];
-        if (lane == 0) {
-            st.lambda = rp.ep.lambda0;
-            st.last_fail = 0;
-            st.has_cand = 1;
-        }
-        __syncwarp();
+    int hyp = 0;
+    if (warp < kHypTile) {
+        const int slot = slot0 + (warp < n ? warp : 0);
+        hyp = p.active_idx ? p.active_idx[slot] : slot;
+        const double T = lane < 12 ? (rp.T_cw ? rp.T_cw[12 * (size_t)hyp + lane] : __ldcg(rp.ep.state[hyp].T + lane)) : 0.0;
+        if (steps) resident_begin(hyps[warp], T, rp.ep.lambda0, lane);
+        if (lane < 12) pose[warp][lane] = narrow(T);
+        if (lane == 0) s_cand[warp] = warp < n;
     }
-    if (tid < 12 * kHypTile) {
-        const int h = tid / 12, hyp = hyp_of(h < n ? h : 0);
-        pose[h][tid % 12] = narrow(rp.T_cw ? rp.T_cw[12 * (size_t)hyp + tid % 12] : __ldcg(rp.ep.state[hyp].T + tid % 12));
-    }
-    if (tid < kHypTile) s_cand[tid] = tid < n;
     __syncthreads();
     for (int k = 0; k <= iters; ++k) {
         SlotPoses sp;
@@ -1055,6 +1049,7 @@ level_resident_kernel(const __grid_constant__ ResidentParams rp) {
             any = any || sp.act[h];
         }
         if (any) {                                       // the same in every CTA of the cluster
+            if (steps && s_cand[warp]) resident_priors(hyps[warp], rp.ep.prior, k == 0, lane);
             float acc[kNumSums];
 #pragma unroll
             for (int i = 0; i < kNumSums; ++i) acc[i] = 0.f;
@@ -1071,11 +1066,13 @@ level_resident_kernel(const __grid_constant__ ResidentParams rp) {
                 (&E[0][0])[tid] = sum;
             }
             __syncthreads();
-            if (warp < n) {
-                const int mode = rp.T_cw ? kEpiEval : (k == 0 ? kEpiInit : kEpiStep);
-                const int cand = lm_update(rp.ep.state[hyp_of(warp)], mode, k < iters, rp.ep.damping_mode, rp.ep.prior,
-                                           E[warp], rp.T_cw ? 0.0 : *rp.min_valid, pose[warp],
-                                           rp.T_cw ? rp.ep.eval_out + (size_t)(slot0 + warp) * kNumSums : nullptr, lane);
+            if (steps && rp.T_cw) {
+                if (lane < kNumSums)
+                    rp.ep.eval_out[(size_t)(slot0 + warp) * kNumSums + lane] =
+                        with_priors(E[warp][lane], hyps[warp].terms[lane]);
+            } else if (steps) {
+                const int cand = resident_step(hyps[warp], E[warp], k == 0 ? kEpiInit : kEpiStep, k < iters,
+                                               rp.ep.damping_mode, *rp.min_valid, pose[warp], lane);
                 if (lane == 0) s_cand[warp] = cand;
             }
         }
@@ -1086,6 +1083,7 @@ level_resident_kernel(const __grid_constant__ ResidentParams rp) {
             __syncthreads();
         }
     }
+    if (steps && !rp.T_cw) resident_end(hyps[warp], rp.ep.state[hyp], lane);
 }
 
 // One hypothesis per CTA, and a ninth warp for its FP64 work: the warp keeps the LM state on its

@@ -405,6 +405,86 @@ static __device__ __noinline__ int lm_update(HypState& st, int mode, int solve_n
     return s.has_cand;
 }
 
+// A hypothesis whose LM state stays in shared memory through a level, and what its priors add to
+// the sums at the pose being evaluated (lane l's factors in terms[l]).
+struct ResidentHyp {
+    double T[12], Tc[12], hg[27], cost, lambda;
+    PriorTerms terms[32];
+    int n_valid, has_cand, last_fail, pad;
+};
+
+// Level start, by one warp: T is lane l's entry of the pose (l < 12).
+__device__ __forceinline__ void resident_begin(ResidentHyp& h, double T, double lambda0, int lane) {
+    if (lane < 12) h.T[lane] = T;
+    if (lane == 0) {
+        h.lambda = lambda0;
+        h.cost = 0.0;
+        h.n_valid = 0;
+        h.has_cand = 1;
+        h.last_fail = 0;
+    }
+}
+
+// The priors at the pose to be evaluated (first: T, else the candidate), by the hypothesis' warp
+// before the gathers: they depend on the pose only, and the other warps gather meanwhile.
+static __device__ __noinline__ void resident_priors(ResidentHyp& h, const PriorParams& prior, int first, int lane) {
+    int ta = 0, tb = 0;
+    if (lane < 21) tri_pair(lane, &ta, &tb);
+    const double T = lane < 12 ? (first ? h.T[lane] : h.Tc[lane]) : 0.0;
+    h.terms[lane] = prior_terms(prior, T, lane, ta, tb);
+}
+
+// The LM step on the photo sums E (29, shared memory), by the hypothesis' warp; the next candidate's
+// FP32 pose goes to pose.  Returns whether there is one.
+static __device__ __noinline__ int resident_step(ResidentHyp& h, const double* E, int mode, int solve_next,
+                                                 int damping_mode, double min_valid, float* pose, int lane) {
+    int ta = 0, tb = 0;
+    if (lane < 21) tri_pair(lane, &ta, &tb);
+    LmLanes s;
+    s.T = lane < 12 ? h.T[lane] : 0.0;
+    s.Tc = lane < 12 && mode == kEpiStep ? h.Tc[lane] : 0.0;
+    s.hg = lane < 27 && mode == kEpiStep ? h.hg[lane] : 0.0;
+    s.cost = h.cost;
+    s.lambda = h.lambda;
+    s.n_valid = h.n_valid;
+    s.last_fail = h.last_fail;
+    const bool evaluated = h.has_cand != 0;
+    double e = 0.0;
+    if (evaluated) e = with_priors(lane < kNumSums ? E[lane] : 0.0, h.terms[lane]);
+    bool take;
+    lm_lanes_step(s, mode, evaluated, solve_next, damping_mode, e, min_valid, lane, ta, tb, &take);
+    __syncwarp();
+    if (lane < 12) {
+        h.T[lane] = s.T;
+        if (s.has_cand) {
+            h.Tc[lane] = s.Tc;
+            pose[lane] = narrow(s.Tc);
+        }
+    }
+    if (lane < 27) h.hg[lane] = s.hg;
+    if (lane == 0) {
+        h.cost = s.cost;
+        h.lambda = s.lambda;
+        h.n_valid = s.n_valid;
+        h.has_cand = s.has_cand;
+        h.last_fail = s.last_fail;
+    }
+    __syncwarp();
+    return s.has_cand;
+}
+
+// Level end: what the next level, the top-K and the selection read.
+__device__ __forceinline__ void resident_end(const ResidentHyp& h, HypState& st, int lane) {
+    if (lane < 12) st.T[lane] = h.T[lane];
+    if (lane == 0) {
+        st.cost = h.cost;
+        st.lambda = h.lambda;
+        st.n_valid = h.n_valid;
+        st.has_cand = h.has_cand;
+        st.last_fail = h.last_fail;
+    }
+}
+
 // lm_update for slot `slot` of a launch described by p (candidate written to p.pose32); all
 // 32 lanes of one warp call it.
 __device__ inline void lm_step(const EpilogueParams& p, int slot, const double* E, double min_valid, int lane) {

@@ -240,6 +240,7 @@ struct LevelArgs {
     unsigned* error;           // set to 1 when a barrier wait gives up
     unsigned long long barrier_timeout_ns;   // longest barrier wait
     int barrier_extra;         // 0; > 0 only in the failure self-tests: a grid barrier (lockstep) or a job tile's flag (barrier-free schedule) that cannot complete
+    int small;                 // 1: every listed frame has one anchor tile at most (level_small_kernel)
     int level;                 // >= 0: every frame runs this level; -1: each its own level
     int list_index;            // which header->n_listed entry counts this launch's frames
     int iters[PILOT_MAX_LEVELS];

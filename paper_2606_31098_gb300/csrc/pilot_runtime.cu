@@ -612,18 +612,18 @@ cudaError_t level_occupancy_query(pilot_dtype dt, int C, int variant, int* n) {
 
 namespace {
 
-// flow_mask bit l: level l runs the level kernel's schedule without grid barriers; selftest:
-// the graph of the flag self-test
-long long graph_key(pilot_dtype dt, int C, int variant, int L, const pilot_schedule& sc, int flow_mask,
+// flow_mask bit l: level l runs the level kernel's schedule without grid barriers; small: every
+// frame has one anchor tile at most; selftest: the graph of the flag self-test
+long long graph_key(pilot_dtype dt, int C, int variant, int L, const pilot_schedule& sc, int flow_mask, bool small,
                     bool selftest) {
-    return ((long long)selftest << 62) | ((long long)dt << 44) | ((long long)C << 36) | ((long long)variant << 32) |
+    return ((long long)selftest << 62) | ((long long)small << 48) | ((long long)dt << 44) | ((long long)C << 36) | ((long long)variant << 32) |
            ((long long)L << 28) | ((long long)flow_mask << 22) | ((long long)sc.tile << 8) | (long long)sc.ctas_per_sm;
 }
 
 // Records the whole batched solve on h->bstream: descriptor upload, per-frame set-up,
 // one persistent launch per level (+ per-frame top-K), selection, result download.
 pilot_status capture_batch_graph(pilot_align_handle* h, pilot_dtype dt, int C, int variant, int L,
-                                 const pilot_schedule& sc, int flow_mask) {
+                                 const pilot_schedule& sc, int flow_mask, bool small) {
     const pilot_align_config& c = h->cfg;
     const BatchLayout lay = BatchLayout::make(c.max_frames, c.max_hyps);
     int dev = 0, sms = 0, per_sm = 0;
@@ -667,6 +667,7 @@ pilot_status capture_batch_graph(pilot_align_handle* h, pilot_dtype dt, int C, i
         a.job_meta = h->bjob_meta;
         a.partial = h->partial;
         a.sync = h->bsync + (size_t)level * kSyncWords;
+        a.small = small ? 1 : 0;
         // gather-heavy levels: the schedule without grid barriers (its per-job-tile flags)
         const bool flow = (flow_mask >> level) & 1;
         a.tile_done = flow ? h->bflags : nullptr;
@@ -708,7 +709,7 @@ pilot_status capture_batch_graph(pilot_align_handle* h, pilot_dtype dt, int C, i
     if (e2 != cudaSuccess) return cuda_fail(e2, "graph capture end");
     h->graph = g;
     PILOT_CUDA(cudaGraphInstantiate(&h->gexec, g, 0), "graph instantiate");
-    h->graph_key = graph_key(dt, C, variant, L, sc, flow_mask, h->flag_selftest_ms > 0);
+    h->graph_key = graph_key(dt, C, variant, L, sc, flow_mask, small, h->flag_selftest_ms > 0);
     return PILOT_OK;
 }
 
@@ -1134,6 +1135,8 @@ pilot_status pilot_align_solve_batch(pilot_align_handle* h, const pilot_frame* f
     std::vector<long long> hyp_iters(n, 0);
     std::vector<int> cur(n);
     int flow_mask = 0;     // levels that run without grid barriers
+    bool small = true;     // no frame has more than one anchor tile
+    for (int i = 0; i < n; ++i) small = small && frames[i].N <= sc.tile;
     for (int i = 0; i < n; ++i) cur[i] = frames[i].M;
     for (int level = L - 1; level >= 0; --level) {
         int* list = fr_list + (size_t)level * lay.max_frames;
@@ -1148,6 +1151,7 @@ pilot_status pilot_align_solve_batch(pilot_align_handle* h, const pilot_frame* f
             items[oi + 1] = items[oi] + frame_items(cur[i], frames[i].N, sc.tile, tpi);
         }
         hdr->n_listed[level] = n;
+        // one-tile frames: job tiles claimed for the whole level.  Else
         // the schedule without grid barriers for levels with much gather work per iteration, or
         // at least one work item of anchors per job on average (few steps per gather); the
         // lockstep schedule where the FP64 steps dominate (e.g. 500 anchors per job)
@@ -1156,7 +1160,7 @@ pilot_status pilot_align_solve_batch(pilot_align_handle* h, const pilot_frame* f
             units += (long long)frames[i].N * cur[i];
             n_jobs += cur[i];
         }
-        if (units >= kSplitUnits || (n_jobs > 0 && units >= (long long)kItemAnchors * n_jobs))
+        if (!small && (units >= kSplitUnits || (n_jobs > 0 && units >= (long long)kItemAnchors * n_jobs)))
             flow_mask |= 1 << level;
         for (int i = 0; i < n; ++i) {
             hyp_iters[i] += (long long)cur[i] * c.iters_per_level[level];
@@ -1166,9 +1170,9 @@ pilot_status pilot_align_solve_batch(pilot_align_handle* h, const pilot_frame* f
     }
     if (h->flag_selftest_ms > 0 && flow_mask == 0)
         return fail(PILOT_EINVAL, "flag self-test: no level of this batch runs without grid barriers");
-    const long long key = graph_key(f0.feat_dtype, f0.C, variant, L, sc, flow_mask, h->flag_selftest_ms > 0);
+    const long long key = graph_key(f0.feat_dtype, f0.C, variant, L, sc, flow_mask, small, h->flag_selftest_ms > 0);
     if (!h->gexec || h->graph_key != key)
-        if ((st = capture_batch_graph(h, f0.feat_dtype, f0.C, variant, L, sc, flow_mask)) != PILOT_OK) return st;
+        if ((st = capture_batch_graph(h, f0.feat_dtype, f0.C, variant, L, sc, flow_mask, small)) != PILOT_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     PILOT_CUDA(cudaGraphLaunch(h->gexec, s), "batch graph launch");
     PILOT_CUDA(cudaStreamSynchronize(s), "batch solve");
