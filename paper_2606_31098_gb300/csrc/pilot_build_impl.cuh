@@ -134,21 +134,26 @@ struct ChanSums2 {
     f2 s, m00, m01, m11, b0, b1;
 };
 
-// Two channels at once: the same operations as channel(), in packed form.
+// Two channels at once.  The differences of the taps of a cell ...
+struct CellDiffs {
+    f2 t00, bq, cq, dq;
+};
+__device__ __forceinline__ CellDiffs cell_diffs(f2 t00, f2 t01, f2 t10, f2 t11) {
+    const f2 bq = sub2(t01, t00);                    // d/dx along the upper row
+    const f2 cq = sub2(t10, t00);                    // d/dy along the left column
+    return CellDiffs{t00, bq, cq, sub2(sub2(t11, t10), bq)};   // bilinear cross term
+}
+// ... and the value, in-cell gradient, residual (fr: the reference value, scaled) and six sums of
+// one position in it.
 template <bool SCALED>
-__device__ __forceinline__ void channel_pair(ChanSums2& a, f2 t00, f2 t01, f2 t10, f2 t11, f2 fr,
-                                             f2 ax, f2 ay, f2 sq, f2 sr) {
-    const f2 bq = sub2(t01, t00);
-    const f2 cq = sub2(t10, t00);
-    const f2 dq = sub2(sub2(t11, t10), bq);
-    f2 fu = fma2(dq, ay, bq);
-    f2 fv = fma2(dq, ax, cq);
-    f2 f = fma2(ax, fu, fma2(ay, cq, t00));
+__device__ __forceinline__ void channel_pair(ChanSums2& a, const CellDiffs& d, f2 fr, f2 ax, f2 ay, f2 sq) {
+    f2 fu = fma2(d.dq, ay, d.bq);                    // df/du inside the cell
+    f2 fv = fma2(d.dq, ax, d.cq);                    // df/dv inside the cell
+    f2 f = fma2(ax, fu, fma2(ay, d.cq, d.t00));
     if constexpr (SCALED) {
         f = mul2(f, sq);
         fu = mul2(fu, sq);
         fv = mul2(fv, sq);
-        fr = mul2(fr, sr);
     }
     const f2 r = sub2(f, fr);
     a.s = fma2(r, r, a.s);
@@ -236,15 +241,24 @@ template <pilot_dtype DT, int C, bool SCALED> struct RefBuf {
     }
 };
 
-// Channel sums of one record over this lane's channels: the 4 taps against the anchor's
-// reference values: bilinear value and in-cell gradient, residual, and the six partial sums.
-template <pilot_dtype DT, int C, bool SCALED>
+// Channel sums of R records of one cell over this lane's channels: the 4 taps against the anchor's
+// reference values: bilinear value and in-cell gradient at each record's (ax, ay), residual, and
+// the six partial sums p[record].
+template <pilot_dtype DT, int C, bool SCALED, int R>
 __device__ __forceinline__ void record_partials(const TapBuf<DT, C, SCALED>& b, const RefBuf<DT, C, SCALED>& rr,
-                                                float ax, float ay, const float* qs, const float* rs, float* p) {
+                                                const float (&ax)[R], const float (&ay)[R], const float* qs,
+                                                const float* rs, float (*p)[6]) {
     using G = GroupShape<DT, C, SCALED>;
     constexpr int VW = G::VW;
-    const f2 ax2 = pk(ax, ax), ay2 = pk(ay, ay), z2 = pk(0.f, 0.f);
-    ChanSums2 cs{z2, z2, z2, z2, z2, z2};
+    const f2 z2 = pk(0.f, 0.f);
+    f2 ax2[R], ay2[R];
+    ChanSums2 cs[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        ax2[i] = pk(ax[i], ax[i]);
+        ay2[i] = pk(ay[i], ay[i]);
+        cs[i] = ChanSums2{z2, z2, z2, z2, z2, z2};
+    }
 #pragma unroll
     for (int k = 0; k < G::NV; ++k) {
 #pragma unroll
@@ -253,17 +267,23 @@ __device__ __forceinline__ void record_partials(const TapBuf<DT, C, SCALED>& b, 
 #pragma unroll
             for (int i = 0; i < 4; ++i) raw_pair<DT, VW>(b.t[k][i], e, a[i][0], a[i][1]);
             raw_pair<DT, VW>(rr.r[k], e, r[0], r[1]);
-            channel_pair<SCALED>(cs, pk(a[0][0], a[0][1]), pk(a[1][0], a[1][1]), pk(a[2][0], a[2][1]),
-                                 pk(a[3][0], a[3][1]), pk(r[0], r[1]), ax2, ay2,
-                                 pk(qs[k * VW + e], qs[k * VW + e + 1]), pk(rs[k * VW + e], rs[k * VW + e + 1]));
+            const CellDiffs d = cell_diffs(pk(a[0][0], a[0][1]), pk(a[1][0], a[1][1]), pk(a[2][0], a[2][1]), pk(a[3][0], a[3][1]));
+            f2 fr = pk(r[0], r[1]);
+            const f2 sq = pk(qs[k * VW + e], qs[k * VW + e + 1]);
+            if constexpr (SCALED) fr = mul2(fr, pk(rs[k * VW + e], rs[k * VW + e + 1]));
+#pragma unroll
+            for (int i = 0; i < R; ++i) channel_pair<SCALED>(cs[i], d, fr, ax2[i], ay2[i], sq);
         }
     }
-    p[0] = hsum(cs.s);
-    p[1] = hsum(cs.m00);
-    p[2] = hsum(cs.m01);
-    p[3] = hsum(cs.m11);
-    p[4] = hsum(cs.b0);
-    p[5] = hsum(cs.b1);
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        p[i][0] = hsum(cs[i].s);
+        p[i][1] = hsum(cs[i].m00);
+        p[i][2] = hsum(cs[i].m01);
+        p[i][3] = hsum(cs[i].m11);
+        p[i][4] = hsum(cs[i].b0);
+        p[i][5] = hsum(cs[i].b1);
+    }
 }
 
 // Accumulate anchors [j_begin, j_end) under the CTA's kHypTile hypotheses into this lane's
@@ -292,7 +312,7 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
     const int slot = (lane / APB) % kHypTile;        // this lane's hypothesis slot
     const int qa = q % APB;                          // this lane's anchor in the batch
     const int src0 = lane & ~(LP - 1);
-    const unsigned gmask = LP > 1 ? (((1u << LP) - 1u) << src0) : (1u << lane);
+    constexpr unsigned all = 0xffffffffu;            // every lane runs every batch
 
     const float* P = sp.p[0];
     bool act = sp.act[0];
@@ -333,7 +353,8 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
         nok = act && (!v.valid || v.valid[j]);
         nX = __ldg(v.px + j), nY = __ldg(v.py + j), nZ = __ldg(v.pz + j);
     }
-    for (int jb = jfirst; jb < j_end; jb += ASTEP) {
+    const int batches = (j_end - j_begin + ASTEP - 1) / ASTEP;
+    for (int b = 0, jb = jfirst; b < batches; ++b, jb += ASTEP) {
         // 1. every lane projects its own record: anchor jb + qa under its hypothesis
         const int jo = jb + qa;
         float X = nX, Y = nY, Z = nZ;
@@ -350,7 +371,7 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
             X = __ldg(v.px + jo), Y = __ldg(v.py + jo), Z = __ldg(v.pz + jo);
         }
         bool vis = false;
-        int off = 0;
+        int off = -1;                                // tap offset; -1: not visible
         float ax = 0.f, ay = 0.f, x = 0.f, y = 0.f, z = 1.f, iz = 1.f, wq = 1.f;
         if (ok) {
             // p = R P + t  (world -> camera)
@@ -386,8 +407,11 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
             RefBuf<DT, C, SCALED> rr;
             TapBuf<DT, C, SCALED> taps;
             rr.load(ref + (jo < j_end ? jo : j_begin) * C, 0);
-            taps.load(qry + off, WC, 0);
-            record_partials<DT, C, SCALED>(taps, rr, ax, ay, qs, rs, S);
+            taps.load(qry + max(off, 0), WC, 0);
+            float P[1][6];
+            record_partials<DT, C, SCALED, 1>(taps, rr, {ax}, {ay}, qs, rs, P);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) S[k] = P[0][k];
         } else {
             // 2. the group reads its records two at a time: records t and t + LP/2, one
             //    anchor (t mod APB) under two of the group's hypotheses, against one read of
@@ -408,7 +432,7 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
                 for (int k = 0; k < 6; ++k) {
                     const float send = upper ? lo[k] : hi[k];
                     const float keep = upper ? hi[k] : lo[k];
-                    lo[k] = keep + __shfl_xor_sync(gmask, send, half);
+                    lo[k] = keep + __shfl_xor_sync(all, send, half);
                 }
             };
             // record pair t: records t and t + HALF (one anchor, two hypotheses) against one
@@ -417,16 +441,21 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
                 RefBuf<DT, C, SCALED>& rr = rra[HG > 2 ? t % APB : 0];
                 if constexpr (HG <= 2) rr.load(ref + (jb + t < j_end ? jb + t : j_begin) * C, q);
                 float P2[2][6];
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int i = t + u * HALF;
-                    // (an invisible record reads the map's first cell; its sums are discarded)
-                    const int o = __shfl_sync(gmask, off, src0 + i);
-                    const float axi = __shfl_sync(gmask, ax, src0 + i);
-                    const float ayi = __shfl_sync(gmask, ay, src0 + i);
-                    TapBuf<DT, C, SCALED> taps;
-                    taps.load(qry + o, WC, q);
-                    record_partials<DT, C, SCALED>(taps, rr, axi, ayi, qs, rs, P2[u]);
+                const int o0 = __shfl_sync(all, off, src0 + t), o1 = __shfl_sync(all, off, src0 + t + HALF);
+                const float ax2[2] = {__shfl_sync(all, ax, src0 + t), __shfl_sync(all, ax, src0 + t + HALF)};
+                const float ay2[2] = {__shfl_sync(all, ay, src0 + t), __shfl_sync(all, ay, src0 + t + HALF)};
+                TapBuf<DT, C, SCALED> taps;
+                // hypotheses that agree to a fraction of a pixel read the same cell: one load and
+                // one set of tap differences for both (an invisible record's sums are discarded, so
+                // it goes with the other)
+                if (__all_sync(all, o0 == o1 || (o0 | o1) < 0)) {
+                    taps.load(qry + max(max(o0, o1), 0), WC, q);
+                    record_partials<DT, C, SCALED, 2>(taps, rr, ax2, ay2, qs, rs, P2);
+                } else {
+                    taps.load(qry + max(o0, 0), WC, q);
+                    record_partials<DT, C, SCALED, 1>(taps, rr, {ax2[0]}, {ay2[0]}, qs, rs, P2);
+                    taps.load(qry + max(o1, 0), WC, q);
+                    record_partials<DT, C, SCALED, 1>(taps, rr, {ax2[1]}, {ay2[1]}, qs, rs, P2 + 1);
                 }
                 combine(P2[0], P2[1], HALF);
 #pragma unroll
@@ -697,7 +726,7 @@ __device__ __forceinline__ void accumulate_spread(const LevelView& v, const floa
                 const float axi = LP > 1 ? __shfl_sync(0xffffffffu, ax, src0 + i) : ax;
                 const float ayi = LP > 1 ? __shfl_sync(0xffffffffu, ay, src0 + i) : ay;
                 float* P = LP == 1 || k == 6 ? S : (k & 1) ? B[2] : (k == 0 ? B[0] : B[1]);
-                record_partials<DT, C, SCALED>(taps[m], rr[m], axi, ayi, qs, rs, P);
+                record_partials<DT, C, SCALED, 1>(taps[m], rr[m], {axi}, {ayi}, qs, rs, reinterpret_cast<float(*)[6]>(P));
                 if (k == 1) combine(B[0], B[2], HALF);
                 if (k == 3) {
                     combine(B[1], B[2], HALF);
