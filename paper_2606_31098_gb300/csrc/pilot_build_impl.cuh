@@ -76,6 +76,12 @@ __device__ __forceinline__ void load_raw(const typename Storage<DT>::T* p, RawVe
     }
 }
 
+// One row of a pose (16-byte aligned), by a volatile load: a loop reads it again in every pass
+// instead of holding it in registers.
+__device__ __forceinline__ void load_row(const float* p, float& x, float& y, float& z, float& t) {
+    asm volatile("ld.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x), "=f"(y), "=f"(z), "=f"(t) : "l"(p));
+}
+
 // Channels e and e + 1 (e even) widened to FP32.
 template <pilot_dtype DT, int W>
 __device__ __forceinline__ void raw_pair(const RawVec<DT, W>& v, int e, float& lo, float& hi) {
@@ -295,7 +301,13 @@ __device__ __forceinline__ void record_partials(const TapBuf<DT, C, SCALED>& b, 
 // through the loop; the sums are the same either way).  FRESH_TID: read the thread index
 // through a volatile move, so that the lane layout derived from it is recomputed at each call
 // instead of being hoisted into an enclosing loop and held across that loop's function calls.
-template <pilot_dtype DT, int C, bool SCALED, bool CONF, int NTHREADS, bool PREFETCH = true, bool FRESH_TID = false>
+// REREAD: read the pose again for every batch (three 16-byte loads) instead of holding it in
+// twelve registers through the gathers.  Held against read again, 64 hypotheses x 65536 anchors:
+// 16-bit maps 3739 -> 3703 us a solve, an uneven batch 13.54 -> 13.31 ms, eight frames of the
+// paper's schedule 1212 -> 1160 us; FP32 evaluation 158.5 -> 153.6 us, but FP32 solves 3824 ->
+// 3846 us and FP8 ones 4433 -> 4480 us, which therefore hold it.
+template <pilot_dtype DT, int C, bool SCALED, bool CONF, int NTHREADS, bool PREFETCH = true, bool FRESH_TID = false,
+          bool REREAD = DT == PILOT_BF16 || DT == PILOT_F16>
 __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const SlotPoses& sp, int j_begin, int j_end,
                                                    float* acc) {
     using Elem = typename Storage<DT>::T;
@@ -322,9 +334,12 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
             P = sp.p[h];
             act = sp.act[h];
         }
-    const float R00 = P[0], R01 = P[1], R02 = P[2], T0 = P[3];
-    const float R10 = P[4], R11 = P[5], R12 = P[6], T1 = P[7];
-    const float R20 = P[8], R21 = P[9], R22 = P[10], T2 = P[11];
+    float R00, R01, R02, T0, R10, R11, R12, T1, R20, R21, R22, T2;
+    if constexpr (!REREAD) {
+        R00 = P[0], R01 = P[1], R02 = P[2], T0 = P[3];
+        R10 = P[4], R11 = P[5], R12 = P[6], T1 = P[7];
+        R20 = P[8], R21 = P[9], R22 = P[10], T2 = P[11];
+    }
 
     // channels owned by this lane: vector k covers VW (q + k LP) .. + VW
     float qs[CPL], rs[CPL];
@@ -374,6 +389,11 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
         int off = -1;                                // tap offset; -1: not visible
         float ax = 0.f, ay = 0.f, x = 0.f, y = 0.f, z = 1.f, iz = 1.f, wq = 1.f;
         if (ok) {
+            if constexpr (REREAD) {
+                load_row(P, R00, R01, R02, T0);
+                load_row(P + 4, R10, R11, R12, T1);
+                load_row(P + 8, R20, R21, R22, T2);
+            }
             // p = R P + t  (world -> camera)
             x = fmaf(R00, X, fmaf(R01, Y, fmaf(R02, Z, T0)));
             y = fmaf(R10, X, fmaf(R11, Y, fmaf(R12, Z, T1)));
@@ -927,7 +947,7 @@ template <pilot_dtype DT, int C, bool SCALED, bool CONF>
 __global__ void __launch_bounds__(kBuildThreads, 2)
 build_kernel(const BuildParams p, HypState* state, const double* T_cw) {
     __shared__ __align__(16) float red[kBuildThreads / 32][kHypTile][kAcc];
-    __shared__ float pose[kHypTile][12];
+    __shared__ __align__(16) float pose[kHypTile][12];
     const int slot0 = kHypTile * (int)blockIdx.y, n = min(kHypTile, p.n_active - slot0), tid = threadIdx.x;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (tid < 12 * kHypTile) {
@@ -947,7 +967,8 @@ build_kernel(const BuildParams p, HypState* state, const double* T_cw) {
 #pragma unroll
     for (int i = 0; i < kNumSums; ++i) acc[i] = 0.f;
     const int j0 = blockIdx.x * p.tile;
-    accumulate_anchors<DT, C, SCALED, CONF, kBuildThreads>(level_view(p), sp, j0, min(j0 + p.tile, p.N), acc);
+    accumulate_anchors<DT, C, SCALED, CONF, kBuildThreads, true, false, DT != PILOT_FP8E4M3>(
+        level_view(p), sp, j0, min(j0 + p.tile, p.N), acc);
     const float v = cta_reduce_slots<kBuildThreads, GroupShape<DT, C, SCALED>::APB>(acc, red);
     const int h = tid / kAcc;
     if (tid < kHypTile * kAcc && h < n) p.partial[((size_t)(slot0 + h) * p.n_tiles + blockIdx.x) * kAcc + tid % kAcc] = v;
@@ -1047,7 +1068,7 @@ level_resident_kernel(const __grid_constant__ ResidentParams rp) {
     __shared__ ResidentHyp hyps[kHypTile];
     __shared__ double E[kHypTile][kAcc];
     __shared__ float rec[kHypTile][kAcc];
-    __shared__ float pose[kHypTile][12];
+    __shared__ __align__(16) float pose[kHypTile][12];
     __shared__ int s_cand[kHypTile];
     cg::cluster_group cluster = cg::this_cluster();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;

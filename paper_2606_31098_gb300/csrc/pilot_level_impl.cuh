@@ -109,7 +109,7 @@ level_persistent_kernel(const __grid_constant__ LevelArgs a) {
     constexpr unsigned kEval = 0x80000000u;          // job_meta: "has a pose to evaluate" bit
     __shared__ __align__(16) float red[kWarps][kHypTile][kAcc];
     __shared__ double E[kWarps][kAcc];
-    __shared__ float pose[kHypTile][12];
+    __shared__ __align__(16) float pose[kHypTile][12];
     __shared__ unsigned s_meta[kHypTile];
     // the claimed work item: its frame, first record slot, tile range and job tile (s_item < 0:
     // none left in this phase)
@@ -420,7 +420,7 @@ level_small_kernel(const __grid_constant__ LevelArgs a) {
     __shared__ __align__(16) float red[kBuildThreads / 32][kHypTile][kAcc];
     __shared__ ResidentHyp hyps[kHypTile];
     __shared__ double E[kHypTile][kAcc];
-    __shared__ float pose[kHypTile][12];
+    __shared__ __align__(16) float pose[kHypTile][12];
     __shared__ int s_cand[kHypTile];
     __shared__ int s_frame, s_level, s_slot, s_n;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
