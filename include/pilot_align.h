@@ -174,7 +174,8 @@ typedef struct {
     int tile;         /* anchors per reduction tile: 512, 1024, 2048 or 4096 */
     int ctas_per_sm;  /* batched form: persistent CTAs per SM; 0 = as many as fit */
     int job_order;    /* batched form: 0 = frames with more anchors first, 1 = frames in the caller's order */
-    int streams;      /* plain form: 1 = one launch per LM iteration over all hypotheses;
+    int streams;      /* plain form, levels of larger frames (a small level is one launch whatever
+                         this says): 1 = one launch per LM iteration over all hypotheses;
                          2..4 = the hypotheses in that many parts, each launched on its own
                          stream, so that the FP64 steps ending one part's launch overlap the
                          other parts' gathers; 0 = 2.  Bitwise the same results. */
@@ -202,7 +203,9 @@ pilot_status pilot_align_get_schedule(const pilot_align_handle* h, const pilot_f
                                       int n_frames, int batched, pilot_schedule* out);
 
 /* Batched form: solve n_frames independent frames (uneven N, M, map sizes, intrinsics,
- * priors) in one pass per pyramid level.  Each level is one persistent cooperative launch
+ * priors) in one pass per pyramid level.  When every frame's anchors fit one tile, each level is
+ * one launch whose CTAs claim tiles of jobs and run the whole level for each, no CTA waiting for
+ * another.  Otherwise each level is one persistent cooperative launch
  * that runs the level's LM iterations over all (frame, hypothesis) jobs; its CTAs claim work
  * items (runs of anchor tiles of one tile of jobs, frames with more anchors first unless the
  * schedule says otherwise) from one counter.  A level with at least 2^23 anchor x hypothesis

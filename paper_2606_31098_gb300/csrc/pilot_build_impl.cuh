@@ -31,6 +31,16 @@
 // it takes or on the other hypotheses (the lanes of all slots run the same anchors in the
 // same order, and the reduction trees are translates of one another), so the result is
 // deterministic and independent of the grid shape and of how hypotheses are grouped.
+//
+// What bounds it: issue and the latency of the L1 gathers, at two CTAs (16 warps) per SM, which 128
+// registers allow; the frame's maps stay in L2, and DRAM is idle.  So the taps and reference rows
+// stay in registers as they were loaded and are widened where they are used, and two records of an
+// anchor whose hypotheses agree to a pixel -- most, once a solve converges -- share one cell's
+// loads and tap differences (64 hypotheses x 65536 anchors: a solve 4158 -> 3738 us, one
+// evaluation 163.8 -> 156.5 us; uneven BF16 batch 15.06 -> 13.60 ms).  Not faster: a third or
+// fourth CTA per SM with the sums in tensor memory (solve 4.3 - 4.6 ms, read-modify-write of 29
+// words per record), the same with the loads of a cell shared by all four hypotheses (4.2 ms), the
+// shared taps held for the second pair (4.1 ms, spills), L1 prefetches a batch ahead (no change).
 #pragma once
 
 #include <cooperative_groups.h>
@@ -942,7 +952,7 @@ __device__ __forceinline__ bool any_cand(const TileSlots& ts) {
 // which may start while the last of these CTAs run, sums them.  The poses are narrowed here, and
 // left in the state for the priors.  (Summing in the last CTA of each hypothesis tile, as
 // build_fused_kernel does, made 64 poses x 65536 anchors 172 us instead of 164: sixteen CTAs sum
-// what sixty-four blocks do here.)
+// what sixty-four blocks do here.)  With the shared cells and the pose read again per batch 153.6 us.
 template <pilot_dtype DT, int C, bool SCALED, bool CONF>
 __global__ void __launch_bounds__(kBuildThreads, 2)
 build_kernel(const BuildParams p, HypState* state, const double* T_cw) {
@@ -1054,8 +1064,8 @@ build_fused_kernel(const FusedBuildParams fp) {
 //
 // Why: with few anchors an iteration is a chain of latencies -- the launch, eight or more
 // dependent batches of gathers, the FP64 step.  One launch per level drops the launches, and
-// level_spread_kernel shortens the rest while SMs would be idle.  solve_small (4096 anchors, 1
-// hypothesis, 20 iterations): 752 -> 378 us; paper's schedule (500 anchors, 1210 -> 128
+// level_spread_kernel shortens the rest while SMs would be idle.  4096 anchors, 1
+// hypothesis, 20 iterations: 752 -> 378 us; paper's schedule (500 anchors, 1210 -> 128
 // hypotheses, 12 evaluations): 552 -> 284 us (with the FP64 step's own gain).
 
 // kHypTile hypotheses per CTA, hypothesis h stepped by warp h.

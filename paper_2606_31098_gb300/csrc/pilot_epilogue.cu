@@ -1,4 +1,5 @@
-// Per-hypothesis FP64 epilogue of each build pass, and the small bookkeeping kernels.
+// FP64 epilogue of an evaluation at given poses, and the small kernels around the levels: set-up,
+// top-K, selection.
 //
 //   tile sums     FP64 sum of the build pass' FP32 partial records, fixed order
 //   gravity term  Eq. 3: r = R gamma^W - gamma^imu, J = [0 | -[a]x], a = R gamma^W

@@ -1,5 +1,5 @@
-// FP64 per-hypothesis part of an LM iteration (device functions shared by the
-// separately launched epilogue and by the build pass' fused last-CTA epilogue).
+// FP64 per-hypothesis part of an LM iteration (device functions shared by the evaluation's
+// epilogue, the build pass' fused last-CTA epilogue and the kernels that run whole levels).
 //
 //   gravity term  Eq. 3: r = R gamma^W - gamma^imu, J = [0 | -[a]x], a = R gamma^W
 //   range term    Eq. 4-6: P = R^T (q - t), r = P_z - D(P_x, P_y), J = [-n | n x q]

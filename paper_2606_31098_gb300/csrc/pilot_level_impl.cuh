@@ -1,7 +1,8 @@
-// Batched form's persistent level kernel (one cooperative launch per pyramid level for a
-// whole batch of frames, or for a serving round).  It reuses the build pass' anchor loop
-// (accumulate_anchors, cta_reduce) and the FP64 step (lm_update), in the plain form's
-// summation order, so a frame's results are bitwise those of its plain solve.
+// Batched form's level kernels: level_persistent_kernel (one cooperative launch per pyramid level
+// for a whole batch of frames, or for a serving round) and level_small_kernel (frames of one anchor
+// tile, no CTA waits for another).  They reuse the build pass' anchor loop (accumulate_anchors,
+// cta_reduce_slots) and the FP64 step, in the plain form's summation order, so a frame's results
+// are bitwise those of its plain solve.
 #pragma once
 
 #include "pilot_build_impl.cuh"
@@ -413,7 +414,8 @@ level_persistent_kernel(const __grid_constant__ LevelArgs a) {
 // CTAs, so a CTA claims a job tile and runs the whole level for it (build pass, FP64 steps on one
 // warp per job, candidates through shared memory), then claims the next.  No barrier and no flag,
 // and the CTAs of an SM drift apart, one stepping on the FP64 pipe while another gathers.  Eight
-// paper-schedule frames (500 anchors, 1210 -> 128 hypotheses): 1540 us in lockstep, 1255 us so.
+// paper-schedule frames (500 anchors, 1210 -> 128 hypotheses): 1540 us in lockstep, 1255 us so; 1160
+// us with the shared cells and the pose read again per batch.
 template <pilot_dtype DT, int C, bool SCALED, bool CONF>
 __global__ void __launch_bounds__(kBuildThreads, 2)
 level_small_kernel(const __grid_constant__ LevelArgs a) {

@@ -5,7 +5,7 @@
 // an external pool or allocator it must go through, or a latency-bound loop (a flight
 // controller, a serving thread) that may not risk an allocation's implicit device
 // synchronisation.  This entry point allocates nothing.  Its scratch (hypothesis
-// state, FP32 candidate poses, slot list and the per-tile partial sums) lives in one
+// state and the per-tile partial sums) lives in one
 // file-scope __device__ array of fixed size; every GPU that loads the library holds that
 // array until the process exits.  The caller passes device pointers for all inputs and
 // for the output.
@@ -40,7 +40,7 @@ constexpr size_t kScratchBytes =
     align256(kOffPartial + sizeof(float) * kAcc * kStaticMaxTiles * (size_t)kStaticMaxHyps);
 
 // The scratch: about 2.3 MB per device.  Every word a call reads is written earlier in
-// the same call (poses, flags and slot list by set_poses, every partial record by the
+// the same call (poses and every partial record by the
 // build pass), so nothing needs clearing between calls.
 __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
