@@ -104,3 +104,9 @@ def test_f32_scales_and_non_finite_maps(torch, frames):
         np.testing.assert_array_equal(a.cost, b.cost)
         np.testing.assert_array_equal(a.status, b.status)
         s.close()
+
+
+@pytest.mark.parametrize("m,n", [(15, 8000), (16, 8000), (76, 2000), (77, 2000), (116, 7500), (117, 7500), (152, 1000)])
+def test_lines_between_the_forms(torch, frames, m, n):
+    """Around the hypotheses x tiles at which a level leaves one CTA per hypothesis, and one launch."""
+    check(torch, cut(frames(32), n, m, False), B.F32, False)
