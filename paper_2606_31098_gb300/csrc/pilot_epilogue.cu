@@ -78,6 +78,10 @@ __device__ __forceinline__ int count_flags(const uint8_t* valid, int N) {
     return c;
 }
 
+// Threshold on visible anchors for the fraction frac of c; never -0.0 (a fraction of -0.0 is accepted
+// as 0), because the LM step compares it with a count by their words.
+__device__ __forceinline__ double visible_threshold(double frac, int c) { return fabs(frac) * (double)c; }
+
 // Start of a plain solve: the hypotheses' states, one per warp; the tickets; and, by the last
 // block, the threshold on visible anchors.  One launch for what were three (5.7 + 5.5 us alone at
 // 65536 anchors and 64 hypotheses, 2.8 + 7.7 us at 500 and 1210).
@@ -88,7 +92,7 @@ solve_init_kernel(HypState* st, const double* T_cw, int* active_idx, int M, unsi
     if (blockIdx.x == gridDim.x - 1) {
         const int c = valid ? count_flags(valid, N) : N;
         if (threadIdx.x == 0) {
-            *min_valid = frac * (double)c;
+            *min_valid = visible_threshold(frac, c);
             *done_ticket = 0u;
         }
         return;
@@ -354,7 +358,7 @@ batch_init_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
     if (blockIdx.y == kFrameBlocks) {
         const int c = f.valid ? count_flags(f.valid, f.N) : f.N;
         if (threadIdx.x == 0) {
-            min_valid[fi] = frac * (double)c;
+            min_valid[fi] = visible_threshold(frac, c);
             tickets[fi] = 0u;
         }
         return;
@@ -406,7 +410,7 @@ round_prepare_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* 
     if (!(f.flags & kFlagInit)) return;
     init_frame(f, st, active, threadIdx.x >> 5, kInitThreads / 32);
     const int c = f.valid ? count_flags(f.valid, f.N) : f.N;
-    if (threadIdx.x == 0) min_valid[fi] = frac * (double)c;
+    if (threadIdx.x == 0) min_valid[fi] = visible_threshold(frac, c);
 }
 
 // Serving round, top-K of the frames that finished a pruning level (as batch_rank_kernel).

@@ -10,6 +10,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "pilot_align.h"
@@ -112,8 +113,11 @@ struct PriorParams {
     double dsm_x0, dsm_y0, dsm_gsd, dsm_inv_gsd;   // inv = 1 / gsd
     double dsm_wmax, dsm_hmax;      // dsm_W - 1, dsm_H - 1
 
-    // the fields that follow from the others
+    // the fields that follow from the others; gates of -0.0 are 0 (off): the step tests and compares
+    // the gates by their words
     void derive() {
+        gate_grav = fabs(gate_grav);
+        gate_range = fabs(gate_range);
         huber_grav2 = huber_grav * huber_grav;
         huber_range2 = huber_range * huber_range;
         gate_grav2 = gate_grav * gate_grav;
