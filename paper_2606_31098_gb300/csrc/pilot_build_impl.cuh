@@ -986,8 +986,10 @@ build_kernel(const BuildParams p, HypState* state, const double* T_cw) {
 
 // The same pass with the per-hypothesis FP64 step fused in: the CTA that takes the last
 // ticket of its hypothesis tile sums the tile records of its hypotheses (FP64, 8 chains per
-// value, fixed order) and runs lm_step for hypothesis h on warp h.  A tile of hypotheses with
-// no candidate runs its steps in tile 0's CTA.
+// value, fixed order) and runs lm_step for hypothesis h on warp h.  A step may set has_cand and
+// write the next pose, which a tile's CTAs read when they start, so the last ticket is also the
+// one of a tile of hypotheses with no candidate, where there is nothing to sum: its step may find
+// one (a larger lambda), and a CTA of the launch that had not started yet would evaluate it.
 template <pilot_dtype DT, int C, bool SCALED, bool CONF>
 __global__ void __launch_bounds__(kBuildThreads, 2)
 build_fused_kernel(const FusedBuildParams fp) {
@@ -998,8 +1000,22 @@ build_fused_kernel(const FusedBuildParams fp) {
     __shared__ int s_last;
     const TileSlots ts = tile_slots(p);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // whether this CTA is the last of its hypothesis tile to get here (one fence for what its
+    // threads read and wrote: it is cumulative over the barrier)
+    auto last_of_tile = [&]() {
+        __syncthreads();
+        if (tid == 0) {
+            __threadfence();
+            s_last = (atomicAdd(fp.tickets + blockIdx.y, 1u) == (unsigned)(p.n_tiles - 1));
+            if (s_last) __threadfence();
+        }
+        __syncthreads();
+        return s_last != 0;
+    };
     if (!any_cand(ts)) {                             // uniform over the CTA
-        if (blockIdx.x == 0 && warp < ts.n) lm_step(fp.ep, ts.slot[warp], E[warp], *fp.min_valid, lane);
+        if (p.n_tiles > 1 && !last_of_tile()) return;
+        if (warp < ts.n) lm_step(fp.ep, ts.slot[warp], E[warp], *fp.min_valid, lane);
+        if (p.n_tiles > 1 && tid == 0) fp.tickets[blockIdx.y] = 0u;
         return;
     }
     float acc[kNumSums];
@@ -1020,15 +1036,7 @@ build_fused_kernel(const FusedBuildParams fp) {
     }
     if (tid < kHypTile * kAcc && hv < ts.n && ts.cand[hv])
         p.partial[((size_t)ts.slot[hv] * p.n_tiles + blockIdx.x) * kAcc + iv] = v;
-    // one fence for the CTA's records (it is cumulative over the barrier)
-    __syncthreads();
-    if (tid == 0) {
-        __threadfence();
-        s_last = (atomicAdd(fp.tickets + blockIdx.y, 1u) == (unsigned)(p.n_tiles - 1));
-        if (s_last) __threadfence();
-    }
-    __syncthreads();
-    if (!s_last) return;
+    if (!last_of_tile()) return;
     // 8 chains per slot and value: thread (h, c, i) sums tiles c, c + 8, ... of sum i of slot h
     {
         constexpr int kTPC = kBuildThreads / (kHypTile * 8);     // threads per (slot, chain)
