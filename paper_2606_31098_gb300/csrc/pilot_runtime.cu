@@ -1135,7 +1135,9 @@ pilot_status pilot_align_solve_batch(pilot_align_handle* h, const pilot_frame* f
     std::vector<long long> hyp_iters(n, 0);
     std::vector<int> cur(n);
     int flow_mask = 0;     // levels that run without grid barriers
-    bool small = true;     // no frame has more than one anchor tile
+    // no frame has more than one anchor tile (the flag self-test is of the schedule without grid
+    // barriers, whatever the frames)
+    bool small = h->flag_selftest_ms <= 0;
     for (int i = 0; i < n; ++i) small = small && frames[i].N <= sc.tile;
     for (int i = 0; i < n; ++i) cur[i] = frames[i].M;
     for (int level = L - 1; level >= 0; --level) {
