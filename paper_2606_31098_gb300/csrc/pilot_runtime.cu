@@ -1135,10 +1135,19 @@ pilot_status pilot_align_solve_batch(pilot_align_handle* h, const pilot_frame* f
     std::vector<long long> hyp_iters(n, 0);
     std::vector<int> cur(n);
     int flow_mask = 0;     // levels that run without grid barriers
-    // no frame has more than one anchor tile (the flag self-test is of the schedule without grid
-    // barriers, whatever the frames)
-    bool small = h->flag_selftest_ms <= 0;
-    for (int i = 0; i < n; ++i) small = small && frames[i].N <= sc.tile;
+    // No frame has more than one anchor tile, and not every job is a whole work item: job tiles are
+    // claimed for the level.  The level's time is then a whole number of job tiles per CTA.  Jobs of
+    // kItemAnchors anchors lose by that and keep the schedule without grid barriers (4096 anchors x
+    // 1600 hypotheses: FP32 4043 us claimed so, 2763 without barriers, BF16 3155 and 2636; x 16: 2204
+    // and 1568, 1957 and 1467; only a full wave gains, BF16 x 1216: 2058 and 2129); smaller
+    // ones would run in lockstep and gain (4000 anchors x 1600: FP32 4503 in lockstep, 4011 so).
+    // The flag self-test is of the schedule without grid barriers, whatever the frames.
+    bool small = h->flag_selftest_ms <= 0, items_only = true;
+    for (int i = 0; i < n; ++i) {
+        small = small && frames[i].N <= sc.tile;
+        items_only = items_only && frames[i].N >= kItemAnchors;
+    }
+    small = small && !items_only;
     for (int i = 0; i < n; ++i) cur[i] = frames[i].M;
     for (int level = L - 1; level >= 0; --level) {
         int* list = fr_list + (size_t)level * lay.max_frames;
