@@ -587,51 +587,53 @@ constexpr int kRowWords = 29;
 enum RowCell { kRowW0 = 0, kRowW1 = 6, kRowB0 = 12, kRowB1 = 18, kRowb0 = 24, kRowb1 = 25, kRowRho = 26, kRowOne = 27,
                kRowZero = 1 /* W0[1] */ };
 
-// The 29 sums over four lanes (the slots of a quad), eight each: four of the form
-// acc = fma(x, y, acc) (the first two rows of H, their g, the cost, the count) and four of the form
-// acc = fma(x, y, fma(z, w, acc)).  Entry: the sum's index, then its cells.
+// The 29 sums over the kHypTile lanes of the slots (four, a quad), 2 kRoleSums each: kRoleSums of
+// the form acc = fma(x, y, acc) (the first two rows of H, their g, the cost, the count) and
+// kRoleSums of the form acc = fma(x, y, fma(z, w, acc)).  Entry: the sum's index, then its cells.
+constexpr int kRoleSums = 16 / kHypTile;
 struct RoleTable {
-    unsigned char sum[4][8], cell[4][24];
+    unsigned char sum[kHypTile][2 * kRoleSums], cell[kHypTile][6 * kRoleSums];
 };
 constexpr RoleTable make_roles() {
+    constexpr int K = kRoleSums;
     RoleTable t{};
     int n1 = 0, n2 = 0;
-    for (int i = 0; i < 32; ++i) {
-        t.sum[i / 8][i % 8] = kNumSums;                      // none
+    for (int l = 0; l < kHypTile; ++l) {
+        for (int i = 0; i < 2 * K; ++i) t.sum[l][i] = kNumSums;                // none
+        for (int i = 0; i < 6 * K; ++i) t.cell[l][i] = kRowZero;
     }
-    for (int i = 0; i < 96; ++i) t.cell[i / 24][i % 24] = kRowZero;
     int e = 0;
     for (int a = 0; a < 6; ++a)
         for (int b = a; b < 6; ++b, ++e) {
             if (a < 2) {
-                t.sum[n1 / 4][n1 % 4] = e;
-                t.cell[n1 / 4][2 * (n1 % 4)] = (a == 0 ? kRowW0 : kRowW1) + a;
-                t.cell[n1 / 4][2 * (n1 % 4) + 1] = (a == 0 ? kRowB0 : kRowB1) + b;
+                t.sum[n1 / K][n1 % K] = e;
+                t.cell[n1 / K][2 * (n1 % K)] = (a == 0 ? kRowW0 : kRowW1) + a;
+                t.cell[n1 / K][2 * (n1 % K) + 1] = (a == 0 ? kRowB0 : kRowB1) + b;
                 ++n1;
             } else {
-                unsigned char* c = t.cell[n2 / 4] + 8 + 4 * (n2 % 4);
-                t.sum[n2 / 4][4 + n2 % 4] = e;
+                unsigned char* c = t.cell[n2 / K] + 2 * K + 4 * (n2 % K);
+                t.sum[n2 / K][K + n2 % K] = e;
                 c[0] = kRowW0 + a, c[1] = kRowB0 + b, c[2] = kRowW1 + a, c[3] = kRowB1 + b;
                 ++n2;
             }
         }
     for (int a = 0; a < 6; ++a) {
         if (a < 2) {
-            t.sum[n1 / 4][n1 % 4] = 21 + a;
-            t.cell[n1 / 4][2 * (n1 % 4)] = (a == 0 ? kRowW0 : kRowW1) + a;
-            t.cell[n1 / 4][2 * (n1 % 4) + 1] = a == 0 ? kRowb0 : kRowb1;
+            t.sum[n1 / K][n1 % K] = 21 + a;
+            t.cell[n1 / K][2 * (n1 % K)] = (a == 0 ? kRowW0 : kRowW1) + a;
+            t.cell[n1 / K][2 * (n1 % K) + 1] = a == 0 ? kRowb0 : kRowb1;
             ++n1;
         } else {
-            unsigned char* c = t.cell[n2 / 4] + 8 + 4 * (n2 % 4);
-            t.sum[n2 / 4][4 + n2 % 4] = 21 + a;
+            unsigned char* c = t.cell[n2 / K] + 2 * K + 4 * (n2 % K);
+            t.sum[n2 / K][K + n2 % K] = 21 + a;
             c[0] = kRowW0 + a, c[1] = kRowb0, c[2] = kRowW1 + a, c[3] = kRowb1;
             ++n2;
         }
     }
     for (int i = 0; i < 2; ++i) {                            // cost, count
-        t.sum[n1 / 4][n1 % 4] = 27 + i;
-        t.cell[n1 / 4][2 * (n1 % 4)] = i == 0 ? kRowRho : kRowOne;
-        t.cell[n1 / 4][2 * (n1 % 4) + 1] = kRowOne;
+        t.sum[n1 / K][n1 % K] = 27 + i;
+        t.cell[n1 / K][2 * (n1 % K)] = i == 0 ? kRowRho : kRowOne;
+        t.cell[n1 / K][2 * (n1 % K) + 1] = kRowOne;
         ++n1;
     }
     return t;
@@ -643,7 +645,7 @@ static __constant__ RoleTable kRoles = make_roles();
 // h-th), so that a step covers four batches, all of their taps in flight at once.  The records'
 // factors pass through shared memory (rows, one per thread) and a quad's lanes add them in the
 // order of their anchors, eight sums each: the same sums in the same order as with four
-// hypotheses per CTA.  acc: this lane's eight (kRoles.sum[slot]).
+// hypotheses per CTA.  acc: this lane's eight, 2 kRoleSums (kRoles.sum[slot]).
 template <pilot_dtype DT, int C, bool SCALED, bool CONF>
 __device__ __forceinline__ void accumulate_spread(const LevelView& v, const float* pose, int j_begin, int j_end,
                                                   float (*rows)[kRowWords], float* acc) {
@@ -671,11 +673,12 @@ __device__ __forceinline__ void accumulate_spread(const LevelView& v, const floa
     const Elem* ref = static_cast<const Elem*>(v.ref);
     const int WC = v.W * C;
     const float xmax = (float)(v.W - 1), ymax = (float)(v.H - 1), d2 = v.huber * v.huber;
-    int cell[24];
+    constexpr int K = kRoleSums;
+    int cell[6 * K];
 #pragma unroll
-    for (int i = 0; i < 24; ++i) cell[i] = kRoles.cell[slot][i];
+    for (int i = 0; i < 6 * K; ++i) cell[i] = kRoles.cell[slot][i];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+    for (int i = 0; i < 2 * K; ++i) acc[i] = 0.f;
     float* row = rows[tid];
 
     float nX = 0.f, nY = 0.f, nZ = 0.f;
@@ -825,10 +828,10 @@ __device__ __forceinline__ void accumulate_spread(const LevelView& v, const floa
         for (int h = 0; h < kHypTile; ++h) {
             const float* r = quad + h * APB * kRowWords;
 #pragma unroll
-            for (int m = 0; m < 4; ++m) {
+            for (int m = 0; m < K; ++m) {
+                const int* c = cell + 2 * K + 4 * m;
                 acc[m] = fmaf(r[cell[2 * m]], r[cell[2 * m + 1]], acc[m]);
-                acc[4 + m] = fmaf(r[cell[8 + 4 * m]], r[cell[9 + 4 * m]],
-                                  fmaf(r[cell[10 + 4 * m]], r[cell[11 + 4 * m]], acc[4 + m]));
+                acc[K + m] = fmaf(r[c[0]], r[c[1]], fmaf(r[c[2]], r[c[3]], acc[K + m]));
             }
         }
         __syncwarp();
@@ -844,11 +847,11 @@ __device__ __forceinline__ float cta_reduce_spread(float* acc, float (*red)[kAcc
     for (int off = 1; off < 32; off <<= 1) {
         if (off >= APB && off < APB * kHypTile) continue;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
+        for (int i = 0; i < 2 * kRoleSums; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
     }
     if (lane % APB == 0 && lane < APB * kHypTile) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < 2 * kRoleSums; ++i) {
             const int s = kRoles.sum[lane / APB][i];
             if (s < kNumSums) red[warp][s] = acc[i];
         }
@@ -862,41 +865,51 @@ __device__ __forceinline__ float cta_reduce_spread(float* acc, float (*red)[kAcc
     return v;
 }
 
-// Fixed-order CTA reduction of the lanes' 29 sums, per hypothesis slot: the eight lanes of a slot
-// are reduced by a butterfly over every lane bit but the slot bits (APB .. APB kHypTile / 2),
+// Fixed-order CTA reduction of the lanes' 29 sums, per hypothesis slot: the 32 / kHypTile lanes of a
+// slot are reduced by a butterfly over every lane bit but the slot bits (APB .. APB kHypTile / 2),
 // then the warps in order.  SCATTER: the butterfly scatters as it goes (16, 8, then 4 sums exchanged
-// instead of 29 three times: the shuffles are what the reduction costs), so a lane ends with four
-// sums; without it fewer registers are live, which the level kernels need more (batched BF16,
-// uneven frames: 15.1 ms without, 15.4 ms with).  Thread t < kHypTile kAcc returns sum t mod kAcc
-// of slot t / kAcc (0 pads).
+// instead of 29 three times: the shuffles are what the reduction costs), so a lane ends with
+// kHypTile sums; without it fewer registers are live, which the level kernels need more (batched
+// BF16, uneven frames: 15.1 ms without, 15.4 ms with).  Thread t < kHypTile kAcc returns sum t mod
+// kAcc of slot t / kAcc (0 pads).
 template <int NTHREADS, int APB, bool SCATTER = true>
 __device__ __forceinline__ float cta_reduce_slots(float* acc, float (*red)[kHypTile][kAcc]) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // the three non-slot lane bits, in the butterfly's order
-    constexpr int b0 = APB == 2 ? 1 : 4, b1 = 8, b2 = 16;
-    static_assert(APB * kHypTile == 4 || APB * kHypTile == 8, "slots of a warp");
+    constexpr int slot_bits = APB * (kHypTile - 1);
+    static_assert(APB * kHypTile <= 32, "slots of a warp");
     if constexpr (SCATTER) {
-        auto exchange = [&](float* a, int n, int bit) {  // keeps the lower or upper half of n sums
-            const bool up = (lane & bit) != 0;
-#pragma unroll
-            for (int i = 0; i < n / 2; ++i) {
-                const float send = up ? a[i] : a[i + n / 2], keep = up ? a[i + n / 2] : a[i];
-                a[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
-            }
-        };
         float a[kAcc];
 #pragma unroll
         for (int i = 0; i < kAcc; ++i) a[i] = i < kNumSums ? acc[i] : 0.f;
-        exchange(a, 32, b0);
-        exchange(a, 16, b1);
-        exchange(a, 8, b2);
-        const int kept = ((lane & b0) ? 16 : 0) + ((lane & b1) ? 8 : 0) + ((lane & b2) ? 4 : 0);
-        *reinterpret_cast<float4*>(&red[warp][(lane / APB) % kHypTile][kept]) = make_float4(a[0], a[1], a[2], a[3]);
+        int n = kAcc, kept = 0;                      // sums held, and the first one's index
+#pragma unroll
+        for (int bit = 1; bit < 32; bit <<= 1) {
+            if (bit & slot_bits) continue;
+            n /= 2;                                  // keeps the lower or upper half
+            const bool up = (lane & bit) != 0;
+#pragma unroll
+            for (int i = 0; i < kAcc / 2; ++i) {
+                if (i >= n) break;
+                const float send = up ? a[i] : a[i + n], keep = up ? a[i + n] : a[i];
+                a[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+            }
+            if (up) kept += n;
+        }
+        float* dst = &red[warp][(lane / APB) % kHypTile][kept];
+        if constexpr (kHypTile == 2) {
+            *reinterpret_cast<float2*>(dst) = make_float2(a[0], a[1]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < kHypTile; i += 4)
+                *reinterpret_cast<float4*>(dst + i) = make_float4(a[i], a[i + 1], a[i + 2], a[i + 3]);
+        }
     } else {
 #pragma unroll
-        for (int bit : {b0, b1, b2})
+        for (int bit = 1; bit < 32; bit <<= 1) {
+            if (bit & slot_bits) continue;
 #pragma unroll
             for (int i = 0; i < kNumSums; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], bit);
+        }
         if (lane % APB == 0 && lane < APB * kHypTile) {
 #pragma unroll
             for (int i = 0; i < kNumSums; ++i) red[warp][lane / APB][i] = acc[i];
@@ -1195,7 +1208,7 @@ level_spread_kernel(const __grid_constant__ ResidentParams rp) {
         PriorTerms terms{};
         if (warp < kBuildThreads / 32) {
             if (cand) {
-                float acc[8];
+                float acc[2 * kRoleSums];
                 const int j0 = rank * p.tile;
                 accumulate_spread<DT, C, SCALED, CONF>(level_view(p), pose, j0, min(j0 + p.tile, p.N), rows, acc);
                 const float v = cta_reduce_spread<GroupShape<DT, C, SCALED>::APB>(acc, red);
