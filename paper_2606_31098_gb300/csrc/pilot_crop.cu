@@ -43,7 +43,22 @@ namespace {
 
 constexpr int kRayThreads = 128;
 constexpr int kRayCluster = 16;     // CTAs per corner ray (a thread-block cluster of the largest size)
-constexpr int kWarpThreads = 448;   // a 256^2 crop is 147 CTAs: one per SM, 14 warps on each
+constexpr int kWarpMaxThreads = 1024;
+
+// Threads per CTA of crop_warp_kernel for n pixels.  A sub-partition's time is its number of warps
+// (the FP64 pipe), and every CTA works the homography out once more, the other warps waiting for
+// it: the pixels spread evenly over the SMs in one CTA each, of at least one warp per sub-partition.
+// Crops of more warps per SM than a CTA takes run in CTAs of 14 warps, three to an SM by their
+// registers, so that one CTA's homography falls into another's pixels.  Whole crop of a 4096^2 map
+// in a row of calls, against 448 threads at every size (us): 64^2 23.2 -> 18.4, 96^2 25.0 -> 18.8,
+// 128^2 24.2 -> 20.9, 192^2 25.1 -> 25.2, 256^2 25.0 (the same 448), 320^2 35.5 -> 31.2, 384^2
+// 47.6 -> 37.5; with 256 threads beyond 394^2, 512^2 54.0, 768^2 115, 2048^2 659; with 448 55.8,
+// 113, 648.
+int warp_threads(long long n) {
+    constexpr int kSms = 152;
+    const long long per_sm = ((n + 31) / 32 + kSms - 1) / kSms;
+    return per_sm > kWarpMaxThreads / 32 ? 448 : 32 * (int)(per_sm > 4 ? per_sm : 4);
+}
 
 // A divisor and its correctly rounded reciprocal; exact: a power of two, whose quotients are
 // products with the reciprocal.
@@ -260,7 +275,7 @@ __device__ __forceinline__ bool crop_geometry(const double* g, double* out) {
     return ok;
 }
 
-__global__ void __launch_bounds__(kWarpThreads)
+__global__ void __launch_bounds__(kWarpMaxThreads)
 crop_warp_kernel(const MapView m, int S, const Divisor side, double* geometry, float* points, unsigned char* valid,
                  float* rgb) {
     __shared__ double H[11];
@@ -377,8 +392,9 @@ extern "C" pilot_status pilot_crop_reference(const pilot_map* map, const pilot_c
         attr[0] = cudaLaunchAttribute{};
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.gridDim = dim3((unsigned)((NP + kWarpThreads - 1) / kWarpThreads));
-        cfg.blockDim = dim3(kWarpThreads);
+        const int threads = warp_threads(NP);
+        cfg.gridDim = dim3((unsigned)((NP + threads - 1) / threads));
+        cfg.blockDim = dim3(threads);
         e = cudaLaunchKernelEx(&cfg, crop_warp_kernel, m, p->S, divisor(p->S), geometry, points, valid, rgb);
     }
     if (e != cudaSuccess) return crop_fail(PILOT_ECUDA, cudaGetErrorString(e));
