@@ -12,10 +12,12 @@
 // memory is allocated.  Without scaling (unscaled BF16 / FP16) there is one launch only.
 //
 // What bounds it: HBM and L2 (the conversion re-reads a map that fits the 129 MB L2), and at a
-// map's size still the launches.  480 x 640 x 32 FP32 to FP8: 32.6 us with four shared-memory
-// atomics per 16 bytes, a division per element and byte stores; 26.5 us with running
-// maxima in registers (a thread's channels stay the same when C divides 4 kQuantThreads), one
-// reciprocal per channel, packed conversions and programmatic dependent launches.
+// map's size still the launches.  480 x 640 x 32 FP32 to FP8: 28.7 us in a row of calls (31 to 33
+// alone) with four shared-memory atomics per 16 bytes, a division per element and byte stores;
+// 20.5 us (25 to 28 alone) with running maxima in registers (a thread's channels stay the same: its
+// stride is a multiple of C), one reciprocal per channel, packed conversions and programmatic
+// dependent launches.  As many values in 48 channels 27.2 -> 25.1 us, in 12 32.9 -> 20.5, in 2048
+// 37.1 -> 18.6.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
@@ -35,62 +37,52 @@ constexpr int kQuantUnroll = 4;      // 16-byte loads in flight per thread
 __device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// FIXED: 4 blockDim.x is a multiple of C, so that a thread's four channels never change and
-// their maxima are kept in registers.
-template <bool FIXED>
+// Both passes: `stride` threads work (the launch's, less a remainder), a multiple of C / 4, each
+// taking every stride-th vector of four values, so that its four channels never change.
+
+// The maxima are kept in registers.
 __global__ void __launch_bounds__(kQuantThreads)
-absmax_kernel(const float* __restrict__ src, long long rows, int C, unsigned* __restrict__ bits) {
+absmax_kernel(const float* __restrict__ src, long long rows, int C, long long stride, unsigned* __restrict__ bits) {
     extern __shared__ unsigned smax[];
     start_next();
     for (int c = threadIdx.x; c < C; c += blockDim.x) smax[c] = 0u;
     __syncthreads();
-    const long long n4 = rows * C / 4, stride = (long long)gridDim.x * blockDim.x;
+    const long long n4 = rows * C / 4;
     const uint4* s4 = reinterpret_cast<const uint4*>(src);
     const long long k0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if constexpr (FIXED) {
-        uint4 m = make_uint4(0u, 0u, 0u, 0u);
-        auto take = [&](const uint4& v) {
-            m.x = max(m.x, v.x & 0x7fffffffu);
-            m.y = max(m.y, v.y & 0x7fffffffu);
-            m.z = max(m.z, v.z & 0x7fffffffu);
-            m.w = max(m.w, v.w & 0x7fffffffu);
-        };
-        long long k = k0;
-        for (; k + (kQuantUnroll - 1) * stride < n4; k += kQuantUnroll * stride) {
-            uint4 v[kQuantUnroll];
+    uint4 m = make_uint4(0u, 0u, 0u, 0u);
+    auto take = [&](const uint4& v) {
+        m.x = max(m.x, v.x & 0x7fffffffu);
+        m.y = max(m.y, v.y & 0x7fffffffu);
+        m.z = max(m.z, v.z & 0x7fffffffu);
+        m.w = max(m.w, v.w & 0x7fffffffu);
+    };
+    long long k = k0 < stride ? k0 : n4;
+    for (; k + (kQuantUnroll - 1) * stride < n4; k += kQuantUnroll * stride) {
+        uint4 v[kQuantUnroll];
 #pragma unroll
-            for (int u = 0; u < kQuantUnroll; ++u) v[u] = __ldg(s4 + k + u * stride);
+        for (int u = 0; u < kQuantUnroll; ++u) v[u] = __ldg(s4 + k + u * stride);
 #pragma unroll
-            for (int u = 0; u < kQuantUnroll; ++u) take(v[u]);
-        }
-        for (; k < n4; k += stride) take(__ldg(s4 + k));
-        // lanes that hold the same channels (uniform over the warp), then one atomic per channel
-        int holders = 32;
+        for (int u = 0; u < kQuantUnroll; ++u) take(v[u]);
+    }
+    for (; k < n4; k += stride) take(__ldg(s4 + k));
+    // lanes that hold the same channels (uniform over the warp), then one atomic per channel
+    int holders = 32;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            if ((4 * o) % C != 0) break;
-            m.x = max(m.x, __shfl_xor_sync(0xffffffffu, m.x, o));
-            m.y = max(m.y, __shfl_xor_sync(0xffffffffu, m.y, o));
-            m.z = max(m.z, __shfl_xor_sync(0xffffffffu, m.z, o));
-            m.w = max(m.w, __shfl_xor_sync(0xffffffffu, m.w, o));
-            holders = o;
-        }
-        if ((int)(threadIdx.x & 31) < holders) {
-            const int c = (int)((4 * threadIdx.x) % C);
-            atomicMax(&smax[c], m.x);
-            atomicMax(&smax[c + 1], m.y);
-            atomicMax(&smax[c + 2], m.z);
-            atomicMax(&smax[c + 3], m.w);
-        }
-    } else {
-        for (long long k = k0; k < n4; k += stride) {
-            const uint4 v = __ldg(s4 + k);
-            const int c = (int)((k * 4) % C);
-            atomicMax(&smax[c], v.x & 0x7fffffffu);
-            atomicMax(&smax[c + 1], v.y & 0x7fffffffu);
-            atomicMax(&smax[c + 2], v.z & 0x7fffffffu);
-            atomicMax(&smax[c + 3], v.w & 0x7fffffffu);
-        }
+    for (int o = 16; o > 0; o >>= 1) {
+        if ((4 * o) % C != 0) break;
+        m.x = max(m.x, __shfl_xor_sync(0xffffffffu, m.x, o));
+        m.y = max(m.y, __shfl_xor_sync(0xffffffffu, m.y, o));
+        m.z = max(m.z, __shfl_xor_sync(0xffffffffu, m.z, o));
+        m.w = max(m.w, __shfl_xor_sync(0xffffffffu, m.w, o));
+        holders = o;
+    }
+    if ((int)(threadIdx.x & 31) < holders) {
+        const int c = (int)(4u * (unsigned)k0 % (unsigned)C);
+        atomicMax(&smax[c], m.x);
+        atomicMax(&smax[c + 1], m.y);
+        atomicMax(&smax[c + 2], m.z);
+        atomicMax(&smax[c + 3], m.w);
     }
     __syncthreads();
     for (int c = threadIdx.x; c < C; c += blockDim.x)
@@ -137,13 +129,13 @@ __device__ __forceinline__ void store4(void* dst, long long k, bool wide, float 
 }
 
 // SCALED: the scales derived from the absmax bits in `scale` (by absmax_kernel); else the values
-// as they are, and `scale` is set to ones.  FIXED as in absmax_kernel.
-template <pilot_dtype DT, bool SCALED, bool FIXED>
+// as they are, and `scale` is set to ones.
+template <pilot_dtype DT, bool SCALED>
 __global__ void __launch_bounds__(kQuantThreads, 6)
-convert_kernel(const float* __restrict__ src, long long rows, int C, float* scale, float qmax,
+convert_kernel(const float* __restrict__ src, long long rows, int C, long long stride, float* scale, float qmax,
                void* __restrict__ dst) {
     start_next();
-    const long long n4 = rows * C / 4, stride = (long long)gridDim.x * blockDim.x;
+    const long long n4 = rows * C / 4;
     const float4* s4 = reinterpret_cast<const float4*>(src);
     const long long k0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const bool wide = ((uintptr_t)dst & 7) == 0;
@@ -153,23 +145,18 @@ convert_kernel(const float* __restrict__ src, long long rows, int C, float* scal
     } else {
         wait_previous();
     }
-    const unsigned* bits = reinterpret_cast<const unsigned*>(scale);
-    // the products are with the reciprocal of the scale
-    auto inverse = [&](int c) { return 1.0f / scale_of(__ldcg(bits + c), qmax, 1); };
+    // the products are with the reciprocals of the scales
     float i0 = 1.0f, i1 = 1.0f, i2 = 1.0f, i3 = 1.0f;
-    if constexpr (SCALED && FIXED) {
-        const int c = (int)((4 * threadIdx.x) % C);
-        i0 = inverse(c), i1 = inverse(c + 1), i2 = inverse(c + 2), i3 = inverse(c + 3);
+    if constexpr (SCALED) {
+        const unsigned* bits = reinterpret_cast<const unsigned*>(scale) + 4u * (unsigned)k0 % (unsigned)C;
+        auto inverse = [&](int c) { return 1.0f / scale_of(__ldcg(bits + c), qmax, 1); };
+        i0 = inverse(0), i1 = inverse(1), i2 = inverse(2), i3 = inverse(3);
     }
     auto convert = [&](long long k, const float4& v) {
-        if constexpr (SCALED && !FIXED) {
-            const int c = (int)((k * 4) % C);
-            i0 = inverse(c), i1 = inverse(c + 1), i2 = inverse(c + 2), i3 = inverse(c + 3);
-        }
         if constexpr (SCALED) store4<DT>(dst, k, wide, v.x * i0, v.y * i1, v.z * i2, v.w * i3);
         else store4<DT>(dst, k, wide, v.x, v.y, v.z, v.w);
     };
-    long long k = k0;
+    long long k = k0 < stride ? k0 : n4;
     for (; k + (kQuantUnroll - 1) * stride < n4; k += kQuantUnroll * stride) {
         float4 v[kQuantUnroll];
 #pragma unroll
@@ -184,6 +171,13 @@ int grid_for(long long n4, int per_sm) {
     long long b = (n4 + kQuantThreads - 1) / kQuantThreads;
     if (b > 152 * per_sm) b = 152 * per_sm;
     return b < 1 ? 1 : (int)b;
+}
+
+// The threads of `grid` CTAs that take part: a multiple of C / 4, and of 8 too (whole 128-byte lines
+// per step) where that leaves most of them.
+long long stride_for(int grid, int C) {
+    const long long threads = (long long)grid * kQuantThreads, quads = C / 4, lines = 8 * quads;
+    return threads >= 8 * lines ? threads / lines * lines : threads / quads * quads;
 }
 
 // One launch that may begin while the kernel before it in the stream still runs; the kernels
@@ -208,12 +202,11 @@ cudaError_t launch_convert(const float* src, long long rows, int C, bool scaled,
                            cudaStream_t s) {
     const int grid = grid_for(rows * C / 4, 6);    // one wave
     if (!scaled) {
-        convert_kernel<DT, false, true><<<grid, kQuantThreads, 0, s>>>(src, rows, C, scale, qmax, dst);
+        convert_kernel<DT, false><<<grid, kQuantThreads, 0, s>>>(src, rows, C, (long long)grid * kQuantThreads, scale, qmax, dst);
         return cudaGetLastError();
     }
-    return (4 * kQuantThreads) % C == 0
-               ? launch_after(convert_kernel<DT, true, true>, grid, kQuantThreads, 0, s, src, rows, C, scale, qmax, dst)
-               : launch_after(convert_kernel<DT, true, false>, grid, kQuantThreads, 0, s, src, rows, C, scale, qmax, dst);
+    return launch_after(convert_kernel<DT, true>, grid, kQuantThreads, 0, s, src, rows, C, stride_for(grid, C), scale, qmax,
+                        dst);
 }
 
 pilot_status qfail(pilot_status st, const std::string& m) {
@@ -243,9 +236,9 @@ extern "C" pilot_status pilot_quantize_features(const float* src, long long rows
     // absmax: four CTAs per SM (each adds one atomic per channel at its end)
     if (use_absmax || n4 == 0) e = cudaMemsetAsync(scale, 0, sizeof(float) * C, s);
     if (e == cudaSuccess && use_absmax && n4 > 0) {
-        const auto kernel = (4 * kQuantThreads) % C == 0 ? absmax_kernel<true> : absmax_kernel<false>;
-        kernel<<<grid_for(n4, 4), kQuantThreads, sizeof(unsigned) * C, s>>>(src, rows, C,
-                                                                            reinterpret_cast<unsigned*>(scale));
+        const int grid = grid_for(n4, 4);
+        absmax_kernel<<<grid, kQuantThreads, sizeof(unsigned) * C, s>>>(src, rows, C, stride_for(grid, C),
+                                                                        reinterpret_cast<unsigned*>(scale));
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && n4 > 0) {
