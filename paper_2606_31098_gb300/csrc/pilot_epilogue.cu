@@ -71,6 +71,7 @@ __device__ __forceinline__ int count_flags(const uint8_t* valid, int N) {
     }
     for (int j = n16 * 16 + threadIdx.x; j < N; j += blockDim.x) c += valid[j] != 0;
     c = __reduce_add_sync(0xffffffffu, c);
+    __syncthreads();                                   // a count before this one has been read
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = c;
     __syncthreads();
     c = 0;
@@ -401,16 +402,25 @@ batch_finalize_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState*
     if (last_block(tickets + fi, kFrameBlocks)) select_frame(frames[fi], fi, res, max_hyps);
 }
 
+// Serving rounds, blocks as frame_grid lays them out: of a frame's, all but the last take its hypotheses
+// and the last one its count of valid anchors.
 __global__ void __launch_bounds__(kInitThreads)
 round_prepare_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st, int* active, double frac,
-                     double* min_valid) {
-    const int fi = blockIdx.x;
-    if (fi >= hdr->n_frames) return;
-    const FrameDesc& f = frames[fi];
-    if (!(f.flags & kFlagInit)) return;
-    init_frame(f, st, active, threadIdx.x >> 5, kInitThreads / 32);
-    const int c = f.valid ? count_flags(f.valid, f.N) : f.N;
-    if (threadIdx.x == 0) min_valid[fi] = visible_threshold(frac, c);
+                     double* min_valid, unsigned* tickets) {
+    const int warps = kInitThreads / 32, parts = gridDim.y - 1;
+    for (int fi = blockIdx.x; fi < hdr->n_frames; fi += gridDim.x) {
+        const FrameDesc& f = frames[fi];
+        if (!(f.flags & kFlagInit)) continue;
+        if ((int)blockIdx.y < parts) {
+            init_frame(f, st, active, blockIdx.y * warps + (threadIdx.x >> 5), parts * warps);
+        } else {
+            const int c = f.valid ? count_flags(f.valid, f.N) : f.N;
+            if (threadIdx.x == 0) {
+                min_valid[fi] = visible_threshold(frac, c);
+                tickets[fi] = 0u;
+            }
+        }
+    }
 }
 
 // Serving round, top-K of the frames that finished a pruning level (as batch_rank_kernel).
@@ -424,20 +434,22 @@ __global__ void round_rank_kernel(const BatchHeader* hdr, const FrameDesc* frame
                           blockIdx.y * kRankHyps);
 }
 
+// The end of a round's level, blocks as in round_prepare_kernel: the last one of a frame's compacts the
+// active list after a pruning level, the others write a finished frame's results, and the last of
+// those to be done selects.
 __global__ void __launch_bounds__(kFinishThreads)
-round_finish_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
-                                    int* active, const double* min_valid, unsigned char* res,
-                                    int max_hyps) {
-    const int fi = blockIdx.x;
-    if (fi >= hdr->n_frames) return;
-    const FrameDesc& f = frames[fi];
-    if (f.flags & kFlagPrune)
-        compact_active(st + f.hyp_offset, active + f.hyp_offset, active + f.hyp_offset, f.n_active);
-    if (f.flags & kFlagFinalize) {
-        finish_frame(f, st, min_valid[fi], res, max_hyps, threadIdx.x >> 5, kFinishThreads / 32);
-        __threadfence();
-        __syncthreads();
-        select_frame(f, fi, res, max_hyps);
+round_finish_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st, int* active, const double* min_valid,
+                    unsigned char* res, int max_hyps, unsigned* tickets) {
+    const int warps = kFinishThreads / 32, parts = gridDim.y - 1;
+    for (int fi = blockIdx.x; fi < hdr->n_frames; fi += gridDim.x) {
+        const FrameDesc& f = frames[fi];
+        if ((int)blockIdx.y == parts) {
+            if (f.flags & kFlagPrune)
+                compact_active(st + f.hyp_offset, active + f.hyp_offset, active + f.hyp_offset, f.n_active);
+        } else if (f.flags & kFlagFinalize) {
+            finish_frame(f, st, min_valid[fi], res, max_hyps, blockIdx.y * warps + (threadIdx.x >> 5), parts * warps);
+            if (last_block(tickets + fi, parts)) select_frame(f, fi, res, max_hyps);
+        }
     }
 }
 
@@ -516,21 +528,29 @@ cudaError_t launch_batch_finalize(const BatchHeader* hdr, const FrameDesc* frame
     return cudaGetLastError();
 }
 
+// Blocks over the frames (x) and over one frame's hypotheses (y, and one more): sixteen per frame while
+// a few thousand blocks are enough, then fewer, then several frames per block.
+static dim3 frame_grid(int max_frames) {
+    const int x = max_frames < 1024 ? max_frames : 1024;
+    return dim3(x, (x <= 256 ? kFrameBlocks : 4096 / x) + 1);
+}
+
 cudaError_t launch_round_prepare(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
-                                 int* active, double frac, double* min_valid, int max_frames,
+                                 int* active, double frac, double* min_valid, unsigned* tickets, int max_frames,
                                  cudaStream_t s) {
-    round_prepare_kernel<<<max_frames, kInitThreads, 0, s>>>(hdr, frames, st, active, frac, min_valid);
+    round_prepare_kernel<<<frame_grid(max_frames), kInitThreads, 0, s>>>(hdr, frames, st, active, frac, min_valid, tickets);
     return cudaGetLastError();
 }
 
 cudaError_t launch_round_finish(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                                 int* active, const double* min_valid, unsigned char* result,
-                                int max_hyps, int max_frames, int max_frame_hyps, cudaStream_t s) {
+                                int max_hyps, unsigned* tickets, int max_frames, int max_frame_hyps, cudaStream_t s) {
     const dim3 grid(max_frames, (max_frame_hyps + kRankHyps - 1) / kRankHyps);
     round_rank_kernel<<<grid, kRankThreads, 0, s>>>(hdr, frames, st, active, min_valid);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    round_finish_kernel<<<max_frames, kFinishThreads, 0, s>>>(hdr, frames, st, active, min_valid, result, max_hyps);
+    round_finish_kernel<<<frame_grid(max_frames), kFinishThreads, 0, s>>>(hdr, frames, st, active, min_valid, result, max_hyps,
+                                                                          tickets);
     return cudaGetLastError();
 }
 

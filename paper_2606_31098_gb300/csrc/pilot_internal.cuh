@@ -318,18 +318,19 @@ cudaError_t launch_batch_prune(const BatchHeader* hdr, const FrameDesc* frames, 
 cudaError_t launch_batch_finalize(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                                   const double* min_valid, unsigned char* result, int max_hyps,
                                   unsigned* tickets, int max_frames, cudaStream_t s);
-// serving rounds: the same steps, each frame doing only what its flags ask for
+// serving rounds: the same steps, each frame doing only what its flags ask for (tickets: a word per
+// frame, reset by launch_round_prepare for the frames that start)
 struct LevelKeep {
     int k[PILOT_MAX_LEVELS];   // keep_top_k per level
 };
 cudaError_t launch_round_advance(const BatchHeader* hdr, FrameDesc* frames, const int* fr_list, int* fr_item,
                                  int* fr_job, const LevelKeep& keep, int tile, int tpi, cudaStream_t s);
 cudaError_t launch_round_prepare(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
-                                 int* active, double frac, double* min_valid, int max_frames,
+                                 int* active, double frac, double* min_valid, unsigned* tickets, int max_frames,
                                  cudaStream_t s);
 cudaError_t launch_round_finish(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                                 int* active, const double* min_valid, unsigned char* result,
-                                int max_hyps, int max_frames, int max_frame_hyps, cudaStream_t s);
+                                int max_hyps, unsigned* tickets, int max_frames, int max_frame_hyps, cudaStream_t s);
 
 // Sets the message pilot_align_last_error() returns on the calling thread.
 void record_error(const char* msg);

@@ -147,6 +147,7 @@ struct pilot_server {
     HypState* state = nullptr;
     int* active = nullptr;
     double* min_valid = nullptr;
+    unsigned* tickets = nullptr;           // one per slot
     unsigned long long* sync = nullptr;   // level kernel: item claims, barrier arrivals, generations
     float* pose32 = nullptr;              // [job][12] FP32 poses to evaluate
     unsigned* job_meta = nullptr;         // [job] hypothesis | evaluate bit
@@ -193,6 +194,7 @@ void release_buffers(pilot_server* s) {
     cudaFree(s->state);
     cudaFree(s->active);
     cudaFree(s->min_valid);
+    cudaFree(s->tickets);
     cudaFree(s->sync);
     cudaFree(s->pose32);
     cudaFree(s->job_meta);
@@ -274,7 +276,7 @@ cudaError_t capture_round(pilot_server* s) {
     if (e == cudaSuccess) e = cudaMemsetAsync(error, 0, sizeof(unsigned), s->stream);
     if (e == cudaSuccess)
         e = launch_round_prepare(hdr, frames, s->state, s->active, s->cfg.min_valid_frac, s->min_valid,
-                                 s->max_slots, s->stream);
+                                 s->tickets, s->max_slots, s->stream);
     LevelArgs a{};
     a.header = hdr;
     a.frames = frames;
@@ -319,7 +321,7 @@ cudaError_t capture_round(pilot_server* s) {
         if (e == cudaSuccess) e = level_launch(s->dt, s->C, s->variant, a, s->grid, s->stream);
         if (e == cudaSuccess)
             e = launch_round_finish(hdr, frames, s->state, s->active, s->min_valid, s->res_dev, s->cfg.max_hyps,
-                                    s->max_slots, std::min(s->cfg.max_hyps, kMaxFrameHyps), s->stream);
+                                    s->tickets, s->max_slots, std::min(s->cfg.max_hyps, kMaxFrameHyps), s->stream);
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(s->res_host, s->res_dev, s->res_bytes, cudaMemcpyDeviceToHost, s->stream);
     cudaGraph_t g = nullptr;
@@ -570,6 +572,7 @@ pilot_status pilot_serve_create(const pilot_align_config* cfg_in, size_t hbm_bud
     if ((e = cudaMalloc((void**)&s->state, sizeof(HypState) * H)) != cudaSuccess) return bad("state allocation");
     if ((e = cudaMalloc((void**)&s->active, sizeof(int) * H)) != cudaSuccess) return bad("active lists");
     if ((e = cudaMalloc((void**)&s->min_valid, sizeof(double) * (size_t)max_slots)) != cudaSuccess) return bad("thresholds");
+    if ((e = cudaMalloc((void**)&s->tickets, sizeof(unsigned) * (size_t)max_slots)) != cudaSuccess) return bad("tickets");
     if ((e = cudaMalloc((void**)&s->sync, sizeof(unsigned long long) * kSyncWords)) != cudaSuccess)
         return bad("level counters");
     if ((e = cudaMalloc((void**)&s->pose32, sizeof(float) * 12 * H)) != cudaSuccess) return bad("candidates");
