@@ -316,7 +316,7 @@ finalize_kernel(HypState* st, int M, const double* min_valid_ptr, unsigned char*
     if (threadIdx.x == 0) *reinterpret_cast<int*>(res + lay.off_best) = best;
 }
 
-// ---- batched form and serving rounds: one block per frame ----
+// ---- batched form and serving rounds ----
 
 // The hypotheses of one frame from the first-th on, one per warp, every stride-th.
 __device__ void init_frame(const FrameDesc& f, HypState* st, int* active, int first, int stride) {
@@ -346,60 +346,101 @@ __device__ void select_frame(const FrameDesc& f, int fi, unsigned char* res, int
     if (threadIdx.x == 0) reinterpret_cast<int*>(res + lay.bytes)[fi] = best;     // one int per frame after the block
 }
 
-// Blocks of kInitThreads / kFinishThreads per frame (blockIdx.y) for its set-up and its results:
-// with one block per frame, 1210 hypotheses took 54 us to set up and 28.6 us to finish (alone).
+// Grids over the frames (x) and over one frame's hypotheses (y).  A handle's or a server's launches
+// are captured for all the frames it may hold, so their grids are bounded: blocks that find no work
+// still take their turn (eight frames in a handle for 65536: 2234 us with a block per frame, 10275
+// with every block of every frame, 719 so).
 constexpr int kFrameBlocks = 16;
+constexpr int kMaxFrameBlocks = 1024;      // frames side by side; more take turns
+
+// Set-up and results, a warp per hypothesis, and one more block: sixteen blocks per frame (with one,
+// 1210 hypotheses took 54 us to set up and 28.6 us to finish, alone) while a few thousand are enough.
+dim3 frame_grid(int max_frames) {
+    const int x = max_frames < kMaxFrameBlocks ? max_frames : kMaxFrameBlocks;
+    return dim3(x, (x <= 256 ? kFrameBlocks : 4096 / x) + 1);
+}
+
+// Ranking, kRankHyps hypotheses per turn of a block.  Turns are numbered frame after frame, as if every
+// frame had max_frame_hyps; block b takes turns b, b + gridDim.x, ... of those a frame has, so that a
+// frame's turns go to different blocks, and by the blocks' prime number different frames' first turns
+// too.
+constexpr int kRankLanes = 8, kRankHyps = kRankThreads / kRankLanes;   // batched and served forms
+constexpr int kRankBlocks = 2039;
+int rank_turns(int max_frame_hyps) { return (max_frame_hyps + kRankHyps - 1) / kRankHyps; }
+int rank_blocks(int max_frames, int turns) {
+    const long long n = (long long)max_frames * turns;
+    return n < kRankBlocks ? (int)n : kRankBlocks;
+}
+
+// body(frame, first hypothesis) for this block's turns, count(frame) being a frame's hypotheses to
+// rank; a thread looks up one turn.  All threads of the block of kRankThreads.
+template <typename Count, typename Body>
+__device__ __forceinline__ void each_rank_turn(int n_frames, int turns, Count count, Body body) {
+    __shared__ int2 list[kRankThreads];
+    __shared__ int listed;
+    const long long all = (long long)n_frames * turns;
+    for (long long w0 = blockIdx.x; w0 < all; w0 += (long long)gridDim.x * kRankThreads) {
+        __syncthreads();
+        if (threadIdx.x == 0) listed = 0;
+        __syncthreads();
+        const long long w = w0 + (long long)threadIdx.x * gridDim.x;
+        if (w < all) {
+            const int fi = (int)(w / turns), s0 = (int)(w % turns) * kRankHyps;
+            if (s0 < count(fi)) list[atomicAdd(&listed, 1)] = make_int2(fi, s0);
+        }
+        __syncthreads();
+        for (int i = 0; i < listed; ++i) body(list[i].x, list[i].y);
+    }
+}
 
 __global__ void __launch_bounds__(kInitThreads)
 batch_init_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st, int* active, double frac,
                   double* min_valid, unsigned* tickets) {
-    const int fi = blockIdx.x;
-    if (fi >= hdr->n_frames) return;
-    const FrameDesc& f = frames[fi];
-    if (blockIdx.y == kFrameBlocks) {
-        const int c = f.valid ? count_flags(f.valid, f.N) : f.N;
-        if (threadIdx.x == 0) {
-            min_valid[fi] = visible_threshold(frac, c);
-            tickets[fi] = 0u;
+    const int warps = kInitThreads / 32, parts = gridDim.y - 1;
+    for (int fi = blockIdx.x; fi < hdr->n_frames; fi += gridDim.x) {
+        const FrameDesc& f = frames[fi];
+        if ((int)blockIdx.y < parts) {
+            init_frame(f, st, active, blockIdx.y * warps + (threadIdx.x >> 5), parts * warps);
+        } else {
+            const int c = f.valid ? count_flags(f.valid, f.N) : f.N;
+            if (threadIdx.x == 0) {
+                min_valid[fi] = visible_threshold(frac, c);
+                tickets[fi] = 0u;
+            }
         }
-        return;
     }
-    init_frame(f, st, active, blockIdx.y * (kInitThreads / 32) + (threadIdx.x >> 5), kFrameBlocks * (kInitThreads / 32));
 }
 
-constexpr int kRankLanes = 8, kRankHyps = kRankThreads / kRankLanes;   // batched and served forms
-
-// Batched form, top-K after a level: blockIdx.x is the frame, blockIdx.y a block of kRankHyps of
-// its listed hypotheses (frames whose count is at most K keep all of them).
-__global__ void batch_rank_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
-                                  const int* active, const int* n_active, int K, const double* min_valid) {
-    const int fi = blockIdx.x;
-    if (fi >= hdr->n_frames) return;
-    const int n = n_active[fi];
-    if (K <= 0 || K >= n || (int)blockIdx.y * kRankHyps >= n) return;
-    const FrameDesc& f = frames[fi];
-    rank_mark<kRankLanes>(st + f.hyp_offset, active + f.hyp_offset, n, K, min_valid[fi], blockIdx.y * kRankHyps);
+// Batched form, top-K after a level (frames whose count is at most K keep all of them).
+__global__ void __launch_bounds__(kRankThreads)
+batch_rank_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st, const int* active,
+                  const int* n_active, int turns, int K, const double* min_valid) {
+    if (K <= 0) return;
+    each_rank_turn(hdr->n_frames, turns, [&](int fi) { return K < n_active[fi] ? n_active[fi] : 0; }, [&](int fi, int s0) {
+        const FrameDesc& f = frames[fi];
+        rank_mark<kRankLanes>(st + f.hyp_offset, active + f.hyp_offset, n_active[fi], K, min_valid[fi], s0);
+    });
 }
 
 // Batched form: each pruned frame's active list compacted in place.
 __global__ void batch_compact_kernel(const BatchHeader* hdr, const FrameDesc* frames, const HypState* st,
                                      int* active, const int* n_active, int K) {
-    const int fi = blockIdx.x;
-    if (fi >= hdr->n_frames) return;
-    const int n = n_active[fi];
-    if (K <= 0 || K >= n) return;
-    const FrameDesc& f = frames[fi];
-    compact_active(st + f.hyp_offset, active + f.hyp_offset, active + f.hyp_offset, n);
+    for (int fi = blockIdx.x; fi < hdr->n_frames; fi += gridDim.x) {
+        const int n = n_active[fi];
+        if (K <= 0 || K >= n) continue;
+        const FrameDesc& f = frames[fi];
+        compact_active(st + f.hyp_offset, active + f.hyp_offset, active + f.hyp_offset, n);
+    }
 }
 
 __global__ void __launch_bounds__(kFinishThreads)
 batch_finalize_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st, const double* min_valid,
                       unsigned char* res, int max_hyps, unsigned* tickets) {
-    const int fi = blockIdx.x;
-    if (fi >= hdr->n_frames) return;
-    finish_frame(frames[fi], st, min_valid[fi], res, max_hyps, blockIdx.y * (kFinishThreads / 32) + (threadIdx.x >> 5),
-                 kFrameBlocks * (kFinishThreads / 32));
-    if (last_block(tickets + fi, kFrameBlocks)) select_frame(frames[fi], fi, res, max_hyps);
+    const int warps = kFinishThreads / 32, parts = gridDim.y;
+    for (int fi = blockIdx.x; fi < hdr->n_frames; fi += gridDim.x) {
+        finish_frame(frames[fi], st, min_valid[fi], res, max_hyps, blockIdx.y * warps + (threadIdx.x >> 5), parts * warps);
+        if (last_block(tickets + fi, parts)) select_frame(frames[fi], fi, res, max_hyps);
+    }
 }
 
 // Serving rounds, blocks as frame_grid lays them out: of a frame's, all but the last take its hypotheses
@@ -424,14 +465,14 @@ round_prepare_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* 
 }
 
 // Serving round, top-K of the frames that finished a pruning level (as batch_rank_kernel).
-__global__ void round_rank_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
-                                  const int* active, const double* min_valid) {
-    const int fi = blockIdx.x;
-    if (fi >= hdr->n_frames) return;
-    const FrameDesc& f = frames[fi];
-    if (!(f.flags & kFlagPrune) || (int)blockIdx.y * kRankHyps >= f.n_active) return;
-    rank_mark<kRankLanes>(st + f.hyp_offset, active + f.hyp_offset, f.n_active, f.keep, min_valid[fi],
-                          blockIdx.y * kRankHyps);
+__global__ void __launch_bounds__(kRankThreads)
+round_rank_kernel(const BatchHeader* hdr, const FrameDesc* frames, HypState* st, const int* active, int turns,
+                  const double* min_valid) {
+    each_rank_turn(hdr->n_frames, turns, [&](int fi) { return frames[fi].flags & kFlagPrune ? frames[fi].n_active : 0; },
+                   [&](int fi, int s0) {
+        const FrameDesc& f = frames[fi];
+        rank_mark<kRankLanes>(st + f.hyp_offset, active + f.hyp_offset, f.n_active, f.keep, min_valid[fi], s0);
+    });
 }
 
 // The end of a round's level, blocks as in round_prepare_kernel: the last one of a frame's compacts the
@@ -504,35 +545,29 @@ cudaError_t launch_round_advance(const BatchHeader* hdr, FrameDesc* frames, cons
 cudaError_t launch_batch_init(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                               int* active, double frac, double* min_valid, unsigned* tickets, int max_frames,
                               cudaStream_t s) {
-    batch_init_kernel<<<dim3(max_frames, kFrameBlocks + 1), kInitThreads, 0, s>>>(hdr, frames, st, active, frac, min_valid,
-                                                                                  tickets);
+    batch_init_kernel<<<frame_grid(max_frames), kInitThreads, 0, s>>>(hdr, frames, st, active, frac, min_valid, tickets);
     return cudaGetLastError();
 }
 
 cudaError_t launch_batch_prune(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                                int* active, const int* n_active, int keep, const double* min_valid,
                                int max_frames, int max_frame_hyps, cudaStream_t s) {
-    const dim3 grid(max_frames, (max_frame_hyps + kRankHyps - 1) / kRankHyps);
-    batch_rank_kernel<<<grid, kRankThreads, 0, s>>>(hdr, frames, st, active, n_active, keep, min_valid);
+    const int turns = rank_turns(max_frame_hyps);
+    batch_rank_kernel<<<rank_blocks(max_frames, turns), kRankThreads, 0, s>>>(hdr, frames, st, active, n_active, turns, keep,
+                                                                              min_valid);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    batch_compact_kernel<<<max_frames, 1024, 0, s>>>(hdr, frames, st, active, n_active, keep);
+    batch_compact_kernel<<<frame_grid(max_frames).x, 1024, 0, s>>>(hdr, frames, st, active, n_active, keep);
     return cudaGetLastError();
 }
 
 cudaError_t launch_batch_finalize(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                                   const double* min_valid, unsigned char* result, int max_hyps,
                                   unsigned* tickets, int max_frames, cudaStream_t s) {
-    batch_finalize_kernel<<<dim3(max_frames, kFrameBlocks), kFinishThreads, 0, s>>>(hdr, frames, st, min_valid, result,
-                                                                                    max_hyps, tickets);
+    const dim3 grid = frame_grid(max_frames);
+    batch_finalize_kernel<<<dim3(grid.x, grid.y - 1), kFinishThreads, 0, s>>>(hdr, frames, st, min_valid, result, max_hyps,
+                                                                              tickets);
     return cudaGetLastError();
-}
-
-// Blocks over the frames (x) and over one frame's hypotheses (y, and one more): sixteen per frame while
-// a few thousand blocks are enough, then fewer, then several frames per block.
-static dim3 frame_grid(int max_frames) {
-    const int x = max_frames < 1024 ? max_frames : 1024;
-    return dim3(x, (x <= 256 ? kFrameBlocks : 4096 / x) + 1);
 }
 
 cudaError_t launch_round_prepare(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
@@ -545,8 +580,8 @@ cudaError_t launch_round_prepare(const BatchHeader* hdr, const FrameDesc* frames
 cudaError_t launch_round_finish(const BatchHeader* hdr, const FrameDesc* frames, HypState* st,
                                 int* active, const double* min_valid, unsigned char* result,
                                 int max_hyps, unsigned* tickets, int max_frames, int max_frame_hyps, cudaStream_t s) {
-    const dim3 grid(max_frames, (max_frame_hyps + kRankHyps - 1) / kRankHyps);
-    round_rank_kernel<<<grid, kRankThreads, 0, s>>>(hdr, frames, st, active, min_valid);
+    const int turns = rank_turns(max_frame_hyps);
+    round_rank_kernel<<<rank_blocks(max_frames, turns), kRankThreads, 0, s>>>(hdr, frames, st, active, turns, min_valid);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     round_finish_kernel<<<frame_grid(max_frames), kFinishThreads, 0, s>>>(hdr, frames, st, active, min_valid, result, max_hyps,
