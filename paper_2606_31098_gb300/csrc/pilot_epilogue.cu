@@ -234,13 +234,18 @@ __device__ __forceinline__ bool last_block(unsigned* ticket, unsigned blocks) {
     return last;
 }
 
-// Plain form: a warp per listed hypothesis; the last block lists the survivors, in their order
-// in active_in, in active_out.
-constexpr int kPlainRankLanes = 32;
+// Plain form: the last block lists the survivors, in their order in active_in, in active_out.  A warp
+// per listed hypothesis, but eight lanes beyond kWideRank of them and one beyond kThinRank: every
+// block reads every key, n^2 LANES / 256 reads, and they are then what the launch takes.  Solves of
+// 100 anchors, one iteration per level, with a warp and as it is: 8193 hypotheses 479 and 469 us,
+// 20000 1373 and 1115, 60000 6406 and 4209 (4616 with eight lanes), 150000 30.9 and 14.1 ms
+// (18.1).
+constexpr int kWideRank = 8192, kThinRank = 32768;
+template <int LANES>
 __global__ void __launch_bounds__(kRankThreads)
 prune_kernel(HypState* st, const int* active_in, int* active_out, int n, int K, const double* min_valid_ptr,
              unsigned* ticket) {
-    rank_mark<kPlainRankLanes>(st, active_in, n, K, *min_valid_ptr, blockIdx.x * (kRankThreads / kPlainRankLanes));
+    rank_mark<LANES>(st, active_in, n, K, *min_valid_ptr, blockIdx.x * (kRankThreads / LANES));
     if (last_block(ticket, gridDim.x)) compact_active(st, active_in, active_out, n);
 }
 
@@ -621,9 +626,14 @@ cudaError_t launch_level_init(HypState* st, float* pose32, const int* active_idx
 cudaError_t launch_prune(HypState* st, const int* active_in, int* active_out, int n_active,
                          int keep, const double* min_valid, unsigned* ticket, cudaStream_t s) {
     if (n_active <= 0) return cudaSuccess;
-    constexpr int per_block = kRankThreads / kPlainRankLanes;
-    prune_kernel<<<(n_active + per_block - 1) / per_block, kRankThreads, 0, s>>>(st, active_in, active_out, n_active, keep,
-                                                                                min_valid, ticket);
+    auto launch = [&](auto kernel, int lanes) {
+        const int per_block = kRankThreads / lanes;
+        kernel<<<(n_active + per_block - 1) / per_block, kRankThreads, 0, s>>>(st, active_in, active_out, n_active, keep,
+                                                                              min_valid, ticket);
+    };
+    if (n_active <= kWideRank) launch(prune_kernel<32>, 32);
+    else if (n_active <= kThinRank) launch(prune_kernel<8>, 8);
+    else launch(prune_kernel<1>, 1);
     return cudaGetLastError();
 }
 
