@@ -57,19 +57,20 @@ __device__ __forceinline__ void init_hyp(HypState& s, const double* T_cw, int la
 }
 
 // Number of set flags among N, by the whole block (blockDim.x a multiple of 32, at most 1024; 16
-// flags per load where aligned); on every thread.
+// flags per load between 16-byte boundaries); on every thread.
 __device__ __forceinline__ int count_flags(const uint8_t* valid, int N) {
     __shared__ int part[32];
     int c = 0;
-    const int n16 = ((uintptr_t)valid & 15) == 0 ? N / 16 : 0;
-    const uint4* w = reinterpret_cast<const uint4*>(valid);
+    const int head = min(N, (int)((0u - (unsigned)(uintptr_t)valid) & 15u)), n16 = (N - head) / 16;
+    const uint4* w = reinterpret_cast<const uint4*>(valid + head);
     auto set4 = [](unsigned v) { return ((v & 0xffu) != 0) + ((v & 0xff00u) != 0) + ((v & 0xff0000u) != 0) + ((v >> 24) != 0); };
 #pragma unroll 4
     for (int k = threadIdx.x; k < n16; k += blockDim.x) {
         const uint4 v = w[k];
         c += set4(v.x) + set4(v.y) + set4(v.z) + set4(v.w);
     }
-    for (int j = n16 * 16 + threadIdx.x; j < N; j += blockDim.x) c += valid[j] != 0;
+    // the bytes before and behind (fewer than 32)
+    for (int j = threadIdx.x; j < N - 16 * n16; j += blockDim.x) c += valid[j < head ? j : j + 16 * n16] != 0;
     c = __reduce_add_sync(0xffffffffu, c);
     __syncthreads();                                   // a count before this one has been read
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = c;
