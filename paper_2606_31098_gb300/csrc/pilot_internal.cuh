@@ -170,22 +170,23 @@ constexpr int kMaxCluster = 8;     // anchor tiles of a level run that way (port
 
 // Whether a level of n_active hypotheses over n_tiles anchor tiles runs in one launch, and with one
 // hypothesis per CTA (2, level_spread_kernel) or kHypTile (1, level_resident_kernel); 0: a launch
-// per iteration.  One hypothesis per CTA while every CTA has an SM of its own, else kHypTile, with
-// one tile always (no CTA waits for another), with more while all clusters are resident at once.
-// A cluster of more than two CTAs has to fit one GPC, so fewer of them than there are slots do: a
-// second wave of clusters takes as long as the first.  Solves of three levels x 11 evaluations,
-// hypotheses x tiles: 152x1 609 us (1224 with kHypTile per CTA, 1371 a launch per iteration), 76x2
-// 667 (1292, 1517), 30x4 683 (1263, 1504), 10x8 685 (1207, 1430), but 38x4 1271 (1261, 1485) and
-// 19x8 1324 (1241, 1479); with kHypTile 64x3 1255 (a launch per iteration 1499), 228x4 1625 (1822),
-// 114x8 1619 (1789), 152x6 1612 (1806), 600x2 1702 (1985), but 300x4 2480 (1910) and 152x8 2557
-// (1907).
+// per iteration.  One hypothesis per CTA while every CTA has an SM of its own, else kHypTile while
+// all CTAs are resident at once: a second wave takes as long as the first, where launches per
+// iteration overlap theirs.  A cluster of more than two CTAs has to fit one GPC, so fewer of them
+// than there are slots do.  Solves of three levels x 11 evaluations, hypotheses x tiles: 152x1 609 us
+// (1224 with kHypTile per CTA, 1371 a launch per iteration), 76x2 667 (1292, 1517), 30x4 683 (1263,
+// 1504), 10x8 685 (1207, 1430), but 38x4 1271 (1261, 1485) and 19x8 1324 (1241, 1479); with kHypTile
+// 64x3 1255 (a launch per iteration 1499), 228x4 1625 (1822), 114x8 1619 (1789), 152x6 1612 (1806),
+// 600x2 1702 (1985), but 300x4 2480 (1910) and 152x8 2557 (1907).  One tile of 1000 anchors beyond
+// one wave: 1230x1 2360 in one launch, 1833 a launch per iteration, 2000x1 2853 and 2339, two full
+// waves 2432x1 2879 and 2752.
 inline int resident_kind(int n_active, int n_tiles) {
     constexpr int kSms = 152;
     constexpr int kSpreadClusters = 120, kResidentClusters = 232;    // CTAs in clusters of more than two
     if (n_tiles > kMaxCluster) return 0;
     if ((long long)n_active * n_tiles <= (n_tiles <= 2 ? kSms : kSpreadClusters)) return 2;
     const long long ctas = (long long)((n_active + kHypTile - 1) / kHypTile) * n_tiles;
-    return n_tiles == 1 || ctas <= (n_tiles == 2 ? 2 * kSms : kResidentClusters) ? 1 : 0;
+    return ctas <= (n_tiles <= 2 ? 2 * kSms : kResidentClusters) ? 1 : 0;
 }
 
 // ---- batched form: many frames, one persistent launch per pyramid level ----
