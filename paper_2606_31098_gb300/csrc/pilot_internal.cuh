@@ -189,6 +189,17 @@ inline int resident_kind(int n_active, int n_tiles) {
     return ctas <= (n_tiles <= 2 ? 2 * kSms : kResidentClusters) ? 1 : 0;
 }
 
+// The same for one evaluation at given poses (0: a build pass and an epilogue).  It has no iterations to
+// gain by: clusters of more than two CTAs of kHypTile only when there are more CTAs than SMs anyway.
+// With fewer some share an SM for want of room in their GPC (FP32, poses x tiles, in clusters and so:
+// 64x8 50.3 and 37.6 us, 64x7 50.7 and 37.6, 152x4 51.7 and 37.5, 200x3 51.7 and 37.6, 128x4 41.5 and 37.5;
+// BF16 64x8 48.2 and 35.7; but 100x8 52.2 and 54.7, 180x5 52.0 and 54.4).
+inline int evaluation_kind(int n_poses, int n_tiles) {
+    constexpr int kSms = 152;
+    const int kind = resident_kind(n_poses, n_tiles);
+    return kind == 1 && n_tiles > 2 && (n_poses + kHypTile - 1) / kHypTile * n_tiles <= kSms ? 0 : kind;
+}
+
 // ---- batched form: many frames, one persistent launch per pyramid level ----
 
 // One frame of a batch, as the device kernels see it.

@@ -934,7 +934,7 @@ pilot_status pilot_align_debug_normal_eq(pilot_align_handle* h, const pilot_fram
     if ((st = bind_frame(h, f, s, &d, false)) != PILOT_OK) return st;
     PILOT_CUDA(cudaMemcpyAsync(h->Tin, T_cw, sizeof(double) * 12 * M, cudaMemcpyHostToDevice, s), "pose copy");
     BuildParams b = build_params(h, f, d, level, M, h->active[0]);
-    const int kind = resident_kind(M, b.n_tiles);
+    const int kind = evaluation_kind(M, b.n_tiles);
     b.active_idx = nullptr;
     EpilogueParams ep{};
     ep.state = h->state;

@@ -221,7 +221,7 @@ extern "C" pilot_status pilot_align_normal_eq_noalloc(const pilot_align_config* 
     pp.gate_grav = cfg->gate_grav;
     pp.gate_range = cfg->gate_range;
     pp.derive();
-    const int kind = resident_kind(f->M, b.n_tiles);
+    const int kind = evaluation_kind(f->M, b.n_tiles);
     cudaError_t e = kind != 0 ? launch_resident(f->feat_dtype, ResidentParams{b, ep, nullptr, T_cw, 0}, kind == 2, s)
                               : launch_build(f->feat_dtype, b, state, T_cw, s);
     if (e == cudaSuccess && kind == 0) e = launch_epilogue(ep, s);
