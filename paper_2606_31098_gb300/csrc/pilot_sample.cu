@@ -10,7 +10,7 @@
 //   z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9; z = (z ^ (z >> 27)) * 0x94D049BB133111EB;
 //   output z ^ (z >> 31).
 //
-// One cluster of 8 CTAs.  A pass over an 11-bit digit of the keys (one shared-memory histogram
+// One cluster of 8 CTAs (one CTA for small crops).  A pass over an 11-bit digit of the keys (one shared-memory histogram
 // per CTA, summed through distributed shared memory) finds the bin that holds the n_select-th
 // smallest key; with uniform keys the first digit leaves about n / 2048 candidates, which are
 // gathered and ranked against one another (more digits follow only while more than 1024 keys
@@ -22,7 +22,9 @@
 // passes and re-hashing every pixel in each took 162 us for 500 of 65536 pixels (174 us alone
 // under ncu); a cluster of 8 CTAs that keeps the hashed halves of the keys in shared memory (up to
 // 20 per thread, 163840 pixels; larger crops hash again per pass) takes 18.4 us, most of
-// it the launch, five cluster barriers and the scans between them.
+// it the launch, five cluster barriers and the scans between them.  Crops of up to 4096 pixels need no
+// second CTA: 500 of 1000 pixels 8.5 us (12.6 with the cluster, 26.8 before it), all of 1000 6.5
+// (11.4, 6.3), 500 of 4096 12.5 (12.6, 22.9), all of 4096 8.5 (10.6, 10.4).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -34,10 +36,9 @@ namespace cg = cooperative_groups;
 namespace pilot {
 namespace {
 
-constexpr int kSampleCtas = 8;                    // one cluster
+constexpr int kSampleCtas = 8;                    // one cluster (one CTA for small crops)
 constexpr int kSampleThreads = 1024;
 constexpr int kSampleWarps = kSampleThreads / 32;
-constexpr int kSampleStep = kSampleCtas * kSampleThreads;   // pixels taken per step of all threads
 constexpr int kSampleBins = 2048;                 // 11-bit digits
 constexpr int kSampleList = 1024;                 // candidates ranked directly
 static_assert(kSampleBins == 2 * kSampleThreads, "two bins per thread");
@@ -72,37 +73,60 @@ __device__ __forceinline__ unsigned cta_scan(unsigned v, unsigned* s_warp, unsig
 }
 
 constexpr int kSampleKeep = 20;                   // most steps whose keys are kept
+constexpr int kSampleOne = 4096;                  // most pixels that one CTA takes
 
-// KEEP: at most kSampleKeep steps of kSampleStep pixels, the hashed halves of the keys kept in
-// (dynamic) shared memory; else any number, hashed again where they are read.
-template <bool KEEP>
-__global__ void __cluster_dims__(kSampleCtas, 1, 1) __launch_bounds__(kSampleThreads)
+// KEEP: at most kSampleKeep steps of CTAS kSampleThreads pixels, the hashed halves of the keys kept in
+// (dynamic) shared memory; else any number, hashed again where they are read.  One CTA counts the
+// valid pixels before it hashes: where all of them are taken it lists them at once.
+template <bool KEEP, int CTAS>
+__global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(kSampleThreads)
 sample_anchors_kernel(const uint8_t* valid, const float* points, int n, int k, unsigned long long seed,
                       int* out_idx, float* out_pts, int* out_count) {
+    static_assert(KEEP || CTAS > 1, "one CTA keeps its keys");
+    constexpr int kStep = CTAS * kSampleThreads;   // pixels taken per step of all threads
     __shared__ __align__(16) unsigned hist[kSampleBins];
     __shared__ unsigned long long list[kSampleList], all[kSampleList];
     __shared__ unsigned s_warp[kSampleWarps];
     __shared__ unsigned s_n, s_bin, s_before, s_count, s_total;
     __shared__ unsigned long long s_kth;
     cg::cluster_group cluster = cg::this_cluster();
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rank = (int)cluster.block_rank();
+    auto all_ctas = [&]() {
+        if constexpr (CTAS > 1) cluster.sync();
+        else __syncthreads();
+    };
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rank = CTAS > 1 ? (int)cluster.block_rank() : 0;
     // warp gw owns pixels [gw run, (gw + 1) run), lane l of step i pixel 32 i + l of them
-    const unsigned steps = (unsigned)(((long long)n + kSampleStep - 1) / kSampleStep);
+    const unsigned steps = (unsigned)(((long long)n + kStep - 1) / kStep);
     const unsigned first = (unsigned)(rank * kSampleWarps + warp) * steps * 32u + (unsigned)lane;
     extern __shared__ unsigned keys[];             // [step][thread] (KEEP)
     unsigned long long ok = 0;                     // bit i: pixel of step i is valid (KEEP)
+    auto hash = [&](unsigned i) {
+        keys[i * kSampleThreads + tid] = (unsigned)(splitmix64_output(seed, first + 32u * i) >> 32);
+    };
+    unsigned take = 0, want = 0;                   // want: 1-based rank within the prefix
+    bool every = false;                            // every valid pixel is taken
     if constexpr (KEEP) {
         for (unsigned i0 = 0; i0 < steps; i0 += 8) {
             uint8_t v[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) v[u] = first + 32u * (i0 + u) < (unsigned)n && i0 + u < steps ? valid[first + 32u * (i0 + u)] : 0;
+            if constexpr (CTAS > 1) {
 #pragma unroll 2
-            for (int u = 0; u < 8; ++u) {
-                if (i0 + u >= steps) break;
-                keys[(i0 + u) * kSampleThreads + tid] = (unsigned)(splitmix64_output(seed, first + 32u * (i0 + u)) >> 32);
+                for (int u = 0; u < 8; ++u) {
+                    if (i0 + u >= steps) break;
+                    hash(i0 + u);
+                }
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) ok |= (unsigned long long)(v[u] != 0) << (i0 + u);
+        }
+        if constexpr (CTAS == 1) {
+            unsigned total;
+            cta_scan((unsigned)__popcll(ok), s_warp, &total);
+            take = (unsigned)k < total ? (unsigned)k : total;
+            every = take == total;
+            if (!every)
+                for (unsigned i = 0; i < steps; ++i) hash(i);
         }
     }
     // key of this thread's pixel of step i; false when it is not valid
@@ -126,9 +150,8 @@ sample_anchors_kernel(const uint8_t* valid, const float* points, int n, int k, u
 
     // the take-th smallest key (all valid pixels when take is their number)
     unsigned long long kth = ~0ull, prefix = 0, mask = 0;
-    unsigned take = 0, want = 0;                   // want: 1-based rank within the prefix
     if (tid == 0) s_n = 0;
-    for (int shift = 53; shift >= 0; shift = shift > 11 ? shift - 11 : (shift > 0 ? 0 : -1)) {
+    for (int shift = 53; shift >= 0 && !every; shift = shift > 11 ? shift - 11 : (shift > 0 ? 0 : -1)) {
         // digits of the key's bits 63-53, 52-42, 41-31, 30-20, 19-9 (11 bits each) and 8-0
         const unsigned digit_mask = shift == 0 ? 0x1ffu : 0x7ffu;
         reinterpret_cast<uint2*>(hist)[tid] = make_uint2(0u, 0u);
@@ -136,12 +159,16 @@ sample_anchors_kernel(const uint8_t* valid, const float* points, int n, int k, u
         each_valid([&](unsigned long long key) {
             if ((key & mask) == prefix) atomicAdd(&hist[(unsigned)(key >> shift) & digit_mask], 1u);
         });
-        cluster.sync();
+        all_ctas();
         uint2 c = make_uint2(0u, 0u);              // bins 2 tid and 2 tid + 1 over the cluster
+        if constexpr (CTAS > 1) {
 #pragma unroll
-        for (int r = 0; r < kSampleCtas; ++r) {
-            const uint2 o = reinterpret_cast<const uint2*>(cluster.map_shared_rank(hist, r))[tid];
-            c.x += o.x, c.y += o.y;
+            for (int r = 0; r < CTAS; ++r) {
+                const uint2 o = reinterpret_cast<const uint2*>(cluster.map_shared_rank(hist, r))[tid];
+                c.x += o.x, c.y += o.y;
+            }
+        } else {
+            c = reinterpret_cast<const uint2*>(hist)[tid];
         }
         const unsigned sum = c.x + c.y;
         unsigned total;
@@ -149,7 +176,8 @@ sample_anchors_kernel(const uint8_t* valid, const float* points, int n, int k, u
         if (shift == 53) {
             take = (unsigned)k < total ? (unsigned)k : total;
             want = take;
-            if (take == 0 || take == total) break;
+            every = take == total;
+            if (take == 0 || every) break;
         }
         const unsigned before = incl - sum;
         if (before < want && want <= incl) {       // exactly one thread
@@ -167,21 +195,26 @@ sample_anchors_kernel(const uint8_t* valid, const float* points, int n, int k, u
             each_valid([&](unsigned long long key) {
                 if ((key & mask) == prefix) list[atomicAdd(&s_n, 1u)] = key;
             });
-            cluster.sync();
-            // warp r copies CTA r's list behind those of the CTAs before it
-            const unsigned held = lane < kSampleCtas ? *cluster.map_shared_rank(&s_n, lane) : 0u;
-            const unsigned at = __reduce_add_sync(0xffffffffu, held);
-            if (warp < kSampleCtas) {
-                const unsigned m = __shfl_sync(0xffffffffu, held, warp);
-                const unsigned to = __reduce_add_sync(0xffffffffu, lane < warp ? held : 0u);
-                const unsigned long long* src = cluster.map_shared_rank(list, warp);
-                for (unsigned i = lane; i < m; i += 32) all[to + i] = src[i];
+            all_ctas();
+            unsigned at = s_n;
+            const unsigned long long* found = list;
+            if constexpr (CTAS > 1) {
+                // warp r copies CTA r's list behind those of the CTAs before it
+                const unsigned held = lane < CTAS ? *cluster.map_shared_rank(&s_n, lane) : 0u;
+                at = __reduce_add_sync(0xffffffffu, held);
+                if (warp < CTAS) {
+                    const unsigned m = __shfl_sync(0xffffffffu, held, warp);
+                    const unsigned to = __reduce_add_sync(0xffffffffu, lane < warp ? held : 0u);
+                    const unsigned long long* src = cluster.map_shared_rank(list, warp);
+                    for (unsigned i = lane; i < m; i += 32) all[to + i] = src[i];
+                }
+                found = all;
+                __syncthreads();
             }
-            __syncthreads();
             for (unsigned i = tid; i < at; i += kSampleThreads) {
-                const unsigned long long key = all[i];
+                const unsigned long long key = found[i];
                 unsigned less = 0;
-                for (unsigned q = 0; q < at; ++q) less += all[q] < key;
+                for (unsigned q = 0; q < at; ++q) less += found[q] < key;
                 if (less + 1u == want) s_kth = key;
             }
             __syncthreads();
@@ -189,14 +222,14 @@ sample_anchors_kernel(const uint8_t* valid, const float* points, int n, int k, u
             break;
         }
         if (shift == 0) kth = prefix;              // cannot happen: keys are distinct
-        cluster.sync();                            // every CTA has read the histograms
+        all_ctas();                                // every CTA has read the histograms
     }
 
     // selected pixels in increasing order: counts per warp, then a scan over warps and CTAs
     const unsigned lanes_below = (1u << lane) - 1u;
     auto selected = [&](unsigned i) {
         unsigned long long key;
-        return key_of(i, key) && take > 0 && key <= kth;
+        return key_of(i, key) && take > 0 && (every || key <= kth);
     };
     unsigned mine = 0;
     unsigned long long sel = 0;                    // bit i: pixel of step i is selected (KEEP)
@@ -210,10 +243,12 @@ sample_anchors_kernel(const uint8_t* valid, const float* points, int n, int k, u
     unsigned total;
     const unsigned upto = cta_scan(lane == 0 ? in_warp : 0u, s_warp, &total);
     unsigned pos = __shfl_sync(0xffffffffu, upto, 0) - in_warp;    // of this warp within the CTA
-    if (tid == 0) s_total = total;
-    cluster.sync();
-    pos += __reduce_add_sync(0xffffffffu, lane < rank ? *cluster.map_shared_rank(&s_total, lane) : 0u);
-    cluster.sync();                                // the shared totals have been read
+    if constexpr (CTAS > 1) {
+        if (tid == 0) s_total = total;
+        cluster.sync();
+        pos += __reduce_add_sync(0xffffffffu, lane < rank ? *cluster.map_shared_rank(&s_total, lane) : 0u);
+        cluster.sync();                            // the shared totals have been read
+    }
     auto put = [&](bool s, unsigned i) {
         const unsigned bal = __ballot_sync(0xffffffffu, s);
         if (s) {
@@ -249,19 +284,20 @@ extern "C" pilot_status pilot_sample_anchors(const unsigned char* valid, const f
         return PILOT_EINVAL;
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int steps = (int)(((long long)n_pixels + kSampleStep - 1) / kSampleStep);
     cudaError_t e = cudaSuccess;
-    if (steps <= kSampleKeep) {
-        const size_t bytes = sizeof(unsigned) * kSampleThreads * (size_t)steps;
-        e = cudaFuncSetAttribute(sample_anchors_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(unsigned) * kSampleThreads * kSampleKeep);
+    auto launch = [&](auto kernel, int ctas, bool keep) {
+        const int steps = (int)(((long long)n_pixels + ctas * kSampleThreads - 1) / (ctas * kSampleThreads));
+        const size_t bytes = keep ? sizeof(unsigned) * kSampleThreads * (size_t)steps : 0;
+        if (keep && ctas > 1)
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sizeof(unsigned) * kSampleThreads * kSampleKeep);
         if (e == cudaSuccess)
-            sample_anchors_kernel<true><<<kSampleCtas, kSampleThreads, bytes, s>>>(valid, points, n_pixels, n_select,
-                                                                                   seed, out_idx, out_points, out_count);
-    } else {
-        sample_anchors_kernel<false><<<kSampleCtas, kSampleThreads, 0, s>>>(valid, points, n_pixels, n_select, seed,
-                                                                            out_idx, out_points, out_count);
-    }
+            kernel<<<ctas, kSampleThreads, bytes, s>>>(valid, points, n_pixels, n_select, seed, out_idx, out_points, out_count);
+    };
+    if (n_pixels <= kSampleOne) launch(sample_anchors_kernel<true, 1>, 1, true);
+    else if (n_pixels <= kSampleKeep * kSampleCtas * kSampleThreads)
+        launch(sample_anchors_kernel<true, kSampleCtas>, kSampleCtas, true);
+    else launch(sample_anchors_kernel<false, kSampleCtas>, kSampleCtas, false);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
         record_error(cudaGetErrorString(e));
