@@ -302,6 +302,11 @@ __device__ __forceinline__ void record_partials(const TapBuf<DT, C, SCALED>& b, 
     }
 }
 
+// Whether reading the pose again per batch (REREAD, below) may pay: not where one lane reads a 32-byte
+// tap of 16 channels by itself (uneven batch, confidence maps: BF16 2152 us with it, 2057 without).
+template <pilot_dtype DT, int C, bool SCALED>
+constexpr bool kPoseReread = !(GroupShape<DT, C, SCALED>::LP == 1 && C == 16);
+
 // Accumulate anchors [j_begin, j_end) under the CTA's kHypTile hypotheses into this lane's
 // 29 sums (the lane's own slot, see GroupShape).  sp: the slots' poses (12 FP32 values each)
 // and whether each has a pose to evaluate (an inactive slot's lanes finish nothing).  Every
@@ -317,7 +322,7 @@ __device__ __forceinline__ void record_partials(const TapBuf<DT, C, SCALED>& b, 
 // paper's schedule 1212 -> 1160 us; FP32 evaluation 158.5 -> 153.6 us, but FP32 solves 3824 ->
 // 3846 us and FP8 ones 4433 -> 4480 us, which therefore hold it.
 template <pilot_dtype DT, int C, bool SCALED, bool CONF, int NTHREADS, bool PREFETCH = true, bool FRESH_TID = false,
-          bool REREAD = DT == PILOT_BF16 || DT == PILOT_F16>
+          bool REREAD = (DT == PILOT_BF16 || DT == PILOT_F16) && kPoseReread<DT, C, SCALED>>
 __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const SlotPoses& sp, int j_begin, int j_end,
                                                    float* acc) {
     using Elem = typename Storage<DT>::T;
@@ -334,7 +339,7 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
     const int slot = (lane / APB) % kHypTile;        // this lane's hypothesis slot
     const int qa = q % APB;                          // this lane's anchor in the batch
     const int src0 = lane & ~(LP - 1);
-    constexpr unsigned all = 0xffffffffu;            // every lane runs every batch
+    constexpr unsigned all = 0xffffffffu;            // every lane that exchanges runs every batch
 
     const float* P = sp.p[0];
     bool act = sp.act[0];
@@ -378,8 +383,10 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
         nok = act && (!v.valid || v.valid[j]);
         nX = __ldg(v.px + j), nY = __ldg(v.py + j), nZ = __ldg(v.pz + j);
     }
+    // every lane of a CTA runs the same batches; without exchanges (LP = 1) to its own last one (uneven
+    // batch of 16 channels, with confidence maps: BF16 2057 -> 2011 us, FP16 2196 -> 2088)
     const int batches = (j_end - j_begin + ASTEP - 1) / ASTEP;
-    for (int b = 0, jb = jfirst; b < batches; ++b, jb += ASTEP) {
+    for (int b = 0, jb = jfirst; LP == 1 ? jb < j_end : b < batches; ++b, jb += ASTEP) {
         // 1. every lane projects its own record: anchor jb + qa under its hypothesis
         const int jo = jb + qa;
         float X = nX, Y = nY, Z = nZ;
@@ -396,7 +403,7 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
             X = __ldg(v.px + jo), Y = __ldg(v.py + jo), Z = __ldg(v.pz + jo);
         }
         bool vis = false;
-        int off = -1;                                // tap offset; -1: not visible
+        int off = LP == 1 ? 0 : -1;                  // tap offset; -1: not visible
         float ax = 0.f, ay = 0.f, x = 0.f, y = 0.f, z = 1.f, iz = 1.f, wq = 1.f;
         if (ok) {
             if constexpr (REREAD) {
@@ -437,7 +444,7 @@ __device__ __forceinline__ void accumulate_anchors(const LevelView& v, const Slo
             RefBuf<DT, C, SCALED> rr;
             TapBuf<DT, C, SCALED> taps;
             rr.load(ref + (jo < j_end ? jo : j_begin) * C, 0);
-            taps.load(qry + max(off, 0), WC, 0);
+            taps.load(qry + off, WC, 0);
             float P[1][6];
             record_partials<DT, C, SCALED, 1>(taps, rr, {ax}, {ay}, qs, rs, P);
 #pragma unroll
@@ -990,7 +997,7 @@ build_kernel(const BuildParams p, HypState* state, const double* T_cw) {
 #pragma unroll
     for (int i = 0; i < kNumSums; ++i) acc[i] = 0.f;
     const int j0 = blockIdx.x * p.tile;
-    accumulate_anchors<DT, C, SCALED, CONF, kBuildThreads, true, false, DT != PILOT_FP8E4M3>(
+    accumulate_anchors<DT, C, SCALED, CONF, kBuildThreads, true, false, DT != PILOT_FP8E4M3 && kPoseReread<DT, C, SCALED>>(
         level_view(p), sp, j0, min(j0 + p.tile, p.N), acc);
     const float v = cta_reduce_slots<kBuildThreads, GroupShape<DT, C, SCALED>::APB>(acc, red);
     const int h = tid / kAcc;
