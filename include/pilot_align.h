@@ -373,7 +373,8 @@ pilot_status pilot_align_selftest_barrier_timeout(pilot_align_handle* h, double 
  * Returns PILOT_OK when the solve reported the timeout (PILOT_ETIMEOUT) and ended (*elapsed_ms,
  * may be NULL, receives its host wall time); PILOT_EINVAL when no level of the batch takes
  * that schedule (fewer than 2^23 anchor x hypothesis units per iteration and fewer than 4096
- * anchors per job).  The results are discarded; the handle stays usable.  Synchronous. */
+ * anchors per job; frames of one anchor tile, which a solve may run without flags, are taken like
+ * any other).  The results are discarded; the handle stays usable.  Synchronous. */
 pilot_status pilot_align_selftest_flag_timeout(pilot_align_handle* h, const pilot_frame* frames, int n,
                                                double timeout_ms, double* elapsed_ms, void* stream);
 
